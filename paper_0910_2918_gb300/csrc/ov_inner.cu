@@ -789,9 +789,8 @@ __global__ void __launch_bounds__(1024) k_rh_df(int count, int dense_m, const do
 }
 
 // ------------------------------------------------- inner Krylov in double-float
-// k_inner with every operation on the float pipes: the tridiagonal factorisation and the
-// two serial solves per step (the critical path of the inner level) and the vector
-// updates in float pairs, the block reductions in float pairs. Square roots take one
+// k_inner with every operation on the float pipes: the tridiagonal factorisation (serial), the
+// solves and the vector updates in float pairs, the block reductions in float pairs. Square roots take one
 // Newton step y + (x - y^2) / (2 y) from the float root, quotients multiply by the
 // refined reciprocal (Karp and Markstein, ACM TOMS 23 (1997)). Outputs (T, Q) are double.
 __device__ __forceinline__ cdf c_add(cdf a, cdf b) { return {a.re + b.re, a.im + b.im}; }
@@ -839,24 +838,25 @@ __device__ bool tri_factor_df(const InnerSmemDf& S, int k) {
   for (int m = 0; m < k - 1; ++m) {
     const cdf an = e_load(&S.a[m + 1]), dn = e_load(&S.d[m + 1]);
     const cdf cn = (m + 1 <= k - 2) ? e_load(&S.c[m + 1]) : zero;
-    cdf r0, r1, r2, lm;
+    cdf ri, r1, r2, lm;
     if (e_abs2hi(dd) >= e_abs2hi(an)) {
       if (e_abs2hi(dd) == 0.f) return false;
-      lm = e_mul(an, e_inv(dd));
-      r0 = dd; r1 = ee; r2 = zero;
+      ri = e_inv(dd);
+      lm = e_mul(an, ri);
+      r1 = ee; r2 = zero;
       dd = e_submul(dn, lm, ee);
       ee = cn;
       S.sw[m] = 0;
     } else {
-      lm = e_mul(dd, e_inv(an));
-      r0 = an; r1 = dn; r2 = cn;
+      ri = e_inv(an);
+      lm = e_mul(dd, ri);
+      r1 = dn; r2 = cn;
       dd = e_submul(ee, lm, dn);
       ee = e_submul(zero, lm, cn);
       S.sw[m] = 1;
     }
-    // U = D (1 + N) with D = diag(r0): the solves need 1 / r0 and the rows of N, r1 / r0
-    // and r2 / r0, so that each step of their serial recurrences is one multiply-add
-    const cdf ri = e_inv(r0);
+    // U = D (1 + N) with D the pivots (1 / D in ri): the solves need 1 / D and the rows of N,
+    // so that each step of their recurrences is one multiply-add
     e_store(&S.uinv[m], ri);
     e_store(&S.u1[m], e_mul(r1, ri));
     e_store(&S.u2[m], e_mul(r2, ri));
@@ -864,66 +864,219 @@ __device__ bool tri_factor_df(const InnerSmemDf& S, int k) {
   }
   if (e_abs2hi(dd) == 0.f) return false;
   e_store(&S.uinv[k - 1], e_inv(dd));
+  e_store(&S.u1[k - 1], zero);
+  e_store(&S.u2[k - 1], zero);
   return true;
 }
 
-// x = H^{-1} b in three parts: the row interchanges and L (serial, one thread), the scaling
-// by 1 / diag(U) (all threads), then (1 + N) x = g backwards (serial). Each serial step is
-// one complex multiply-add on the recurrence's critical path.
-__device__ void tri_solve_fwd_df(const InnerSmemDf& S, int k, const float4* b, float4* x) {
-  cdf cur = e_load(&b[0]);
-#pragma unroll 2
-  for (int m = 0; m < k - 1; ++m) {
-    const cdf nb = e_load(&b[m + 1]);
-    const bool sw = S.sw[m];
-    const cdf bsel = sw ? nb : cur, asel = sw ? cur : nb;
-    e_store(&x[m], bsel);
-    cur = e_submul(asel, e_load(&S.l[m]), bsel);
-  }
-  e_store(&x[k - 1], cur);
+// ---- the tridiagonal solves of one inner step, in parallel ----------------------------
+// With the pivoted factors, H^{-1} b is two linear recurrences over the rows (the row
+// interchanges with L, of first order, downwards the rows; 1 + N, of second order, back up)
+// and H^{-dag} b two more. A serial sweep costs k times the latency of one complex
+// multiply-add (~70 cycles), and two threads of a 256-thread CTA ran them: 73 us an inner
+// step at k = 333, nearly all of the inner level. Here each side of the inner step has 128
+// lanes; lane t owns the B = ceil(k / 128) rows [tB, (t + 1) B), runs its rows from a zero
+// state, the states that enter the chunks are found by a scan over the lanes, and the rows
+// run again from them. The scan composes x -> P x + C (P: a complex number, or a 2 x 2
+// matrix for the second-order recurrences); every product of P it needs depends on H only
+// and is formed once per check (scan_setup), so a scan level is one shuffle and one multiply-
+// add. P of the first-order recurrences is a product of multipliers |l| <= 1; P of the
+// second-order ones is a block of U_{II}^{-1} U_{IJ} of consecutive rows I, and the inverse of
+// a diagonal block of a triangular matrix is that block of its inverse, so no entry exceeds
+// ||U^{-1}|| ||U||: the growth that the factors allow anyway (measured against the oracle at
+// k = 31 .. 1000: the errors of the serial sweeps). 3 + 5 + 3 dependent multiply-adds replace
+// 333 at k = 333; 12 problems, l = 120: 8.72 -> 1.44 ms. With the chains gone the step is bound
+// by the float pipe of its SM (48% issue, ~6000 instructions a warp and step). 32 or 64 lanes
+// a side do less work in the scans but run longer chunks: 14.0 and 13.2 against 13.1 ms for
+// the whole inner level there, 12.6 and 9.9 against 9.7 ms at k = 700.
+constexpr int kSideLanes = 128;  // lanes of one side (v: threads 0.., w: the rest)
+constexpr int kSideWarps = kSideLanes / 32;
+
+struct cdf2 {  // a second-order state: the two newest values
+  cdf x, y;
+};
+struct cmat2 {
+  cdf a, b, c, d;
+};
+__device__ __forceinline__ cdf c_zero() { return {df_zero(), df_zero()}; }
+__device__ __forceinline__ cdf c_one() { return {{1.f, 0.f}, df_zero()}; }
+__device__ __forceinline__ cdf2 lin(cmat2 m, cdf2 s, cdf2 add) {
+  return {c_addmul(c_addmul(add.x, m.a, s.x), m.b, s.y), c_addmul(c_addmul(add.y, m.c, s.x), m.d, s.y)};
 }
-__device__ void tri_solve_bwd_df(const InnerSmemDf& S, int k, float4* x) {
-  if (k < 2) return;
-  cdf x1 = e_load(&x[k - 1]);
-  cdf x0 = e_submul(e_load(&x[k - 2]), e_load(&S.u1[k - 2]), x1);
-  e_store(&x[k - 2], x0);
-#pragma unroll 2
-  for (int m = k - 3; m >= 0; --m) {
-    const cdf xm = e_submul(e_submul(e_load(&x[m]), e_load(&S.u2[m]), x1), e_load(&S.u1[m]), x0);
-    e_store(&x[m], xm);
-    x1 = x0;
-    x0 = xm;
-  }
+__device__ __forceinline__ cdf lin(cdf m, cdf s, cdf add) { return c_addmul(add, m, s); }
+__device__ __forceinline__ cdf compose(cdf f, cdf g) { return e_mul(f, g); }  // f after g
+__device__ __forceinline__ cmat2 compose(cmat2 f, cmat2 g) {
+  const cdf z = c_zero();
+  return {c_addmul(c_addmul(z, f.a, g.a), f.b, g.c), c_addmul(c_addmul(z, f.a, g.b), f.b, g.d),
+          c_addmul(c_addmul(z, f.c, g.a), f.d, g.c), c_addmul(c_addmul(z, f.c, g.b), f.d, g.d)};
+}
+__device__ __forceinline__ void state_zero(cdf& s) { s = c_zero(); }
+__device__ __forceinline__ void state_zero(cdf2& s) { s = {c_zero(), c_zero()}; }
+__device__ __forceinline__ void map_one(cdf& m) { m = c_one(); }
+__device__ __forceinline__ void map_one(cmat2& m) { m = {c_one(), c_zero(), c_zero(), c_one()}; }
+
+// the value of lane `src` (the loops below are kept rolled and shared by the two sides: the
+// step's straight-line code would not stay in the instruction cache)
+__device__ __forceinline__ float shfl_lane(float v, int src) { return __shfl_sync(0xffffffffu, v, src); }
+__device__ __forceinline__ cdf shfl_lane(cdf v, int src) {
+  return {{shfl_lane(v.re.hi, src), shfl_lane(v.re.lo, src)}, {shfl_lane(v.im.hi, src), shfl_lane(v.im.lo, src)}};
+}
+__device__ __forceinline__ cdf2 shfl_lane(cdf2 v, int src) { return {shfl_lane(v.x, src), shfl_lane(v.y, src)}; }
+__device__ __forceinline__ cmat2 shfl_lane(cmat2 v, int src) {
+  return {shfl_lane(v.a, src), shfl_lane(v.b, src), shfl_lane(v.c, src), shfl_lane(v.d, src)};
+}
+// barrier over one side's warps
+__device__ __forceinline__ void side_sync(int side) {
+  asm volatile("bar.sync %0, %1;" ::"r"(1 + side), "n"(kSideLanes) : "memory");
 }
 
-// z = H^{-dag} b: U^dag = (1 + N)^dag D^dag, so (1 + N^dag) y = b forwards (serial), z =
-// conj(1 / diag(U)) y (all threads), then the interchanges' adjoints backwards (serial)
-__device__ void tri_solve_dag_fwd_df(const InnerSmemDf& S, int k, const float4* b, float4* z) {
-  const cdf zero = {df_zero(), df_zero()};
-  cdf z1 = zero, z2 = zero;  // y[m-1], y[m-2]
-#pragma unroll 2
-  for (int m = 0; m < k; ++m) {
-    cdf t = e_load(&b[m]);
-    if (m >= 2) t = c_submulc(t, e_load(&S.u2[m - 2]), z2);
-    if (m >= 1) t = c_submulc(t, e_load(&S.u1[m - 1]), z1);
-    e_store(&z[m], t);
-    z2 = z1;
-    z1 = t;
-  }
+// the products of chunk maps that one recurrence's scan applies: of the 2^lev lanes ending at
+// this one (lev), of all earlier lanes of the warp (excl), and of each whole warp (total)
+template <class M>
+struct ScanMaps {
+  M lev[5], excl;
+};
+template <class M, class St>
+struct ScanShared {
+  M total[kSideWarps];
+  St carry[kSideWarps];
+};
+// place of this lane and warp along the recurrence; up: the rows ascend with the lanes
+struct ScanPos {
+  int lane, li, wi, dir;
+};
+__device__ __forceinline__ ScanPos scan_pos(bool up) {
+  const int lane = threadIdx.x & 31, w = (threadIdx.x % kSideLanes) >> 5;
+  return {lane, up ? lane : 31 - lane, up ? w : kSideWarps - 1 - w, up ? -1 : 1};
 }
-__device__ void tri_solve_dag_bwd_df(const InnerSmemDf& S, int k, float4* z) {
-  cdf gn = e_load(&z[k - 1]);  // current z[m + 1]
-#pragma unroll 2
-  for (int m = k - 2; m >= 0; --m) {
-    const cdf v = c_submulc(e_load(&z[m]), e_load(&S.l[m]), gn);
+template <class M, class St>
+__device__ __forceinline__ void scan_setup(ScanMaps<M>& f, ScanShared<M, St>& sh, M chunk, ScanPos ps) {
+  M p = chunk;
+#pragma unroll 1
+  for (int lev = 0; lev < 5; ++lev) {
+    f.lev[lev] = p;
+    const M q = shfl_lane(p, (ps.lane + (ps.dir << lev)) & 31);
+    if (ps.li >= (1 << lev)) p = compose(p, q);
+  }
+  f.excl = shfl_lane(p, (ps.lane + ps.dir) & 31);
+  if (ps.li == 0) map_one(f.excl);
+  if (ps.li == 31) sh.total[ps.wi] = p;
+}
+// the state that enters this lane's chunk, from the states c that the chunks leave when they
+// are run from zero (one barrier of the side's warps)
+template <class M, class St>
+__device__ __forceinline__ St scan_in(const ScanMaps<M>& f, ScanShared<M, St>& sh, St c, ScanPos ps, int side) {
+#pragma unroll 1
+  for (int lev = 0; lev < 5; ++lev) {
+    const M m = f.lev[lev];
+    const St q = shfl_lane(c, (ps.lane + (ps.dir << lev)) & 31);
+    if (ps.li >= (1 << lev)) c = lin(m, q, c);
+  }
+  if (ps.li == 31) sh.carry[ps.wi] = c;
+  St in = shfl_lane(c, (ps.lane + ps.dir) & 31);
+  if (ps.li == 0) state_zero(in);
+  side_sync(side);
+  if (ps.wi == 0) return in;
+  St s = sh.carry[0];
+#pragma unroll 1
+  for (int w = 1; w <= ps.wi; ++w) {
+    const bool last = w == ps.wi;
+    s = lin(last ? f.excl : sh.total[w], s, last ? in : sh.carry[w]);
+  }
+  return s;
+}
+
+// One lane's rows [s, e) of the four recurrences; each returns the state it leaves and, with
+// `store`, writes its values.
+// row interchanges and L, down the rows, state: the pending row; x[m] / diag(U) is stored
+__device__ __forceinline__ cdf chunk_l(const InnerSmemDf& S, int k, int s, int e, const float4* b, float4* x, cdf cur,
+                                       bool store) {
+#pragma unroll 1
+  for (int m = s; m < e; ++m) {
+    cdf bsel = cur;
+    if (m < k - 1) {
+      const cdf nb = e_load(&b[m + 1]);
+      const bool sw = S.sw[m];
+      const cdf asel = sw ? cur : nb;
+      bsel = sw ? nb : cur;
+      cur = e_submul(asel, e_load(&S.l[m]), bsel);
+    }
+    if (store) e_store(&x[m], e_mul(bsel, e_load(&S.uinv[m])));
+  }
+  return cur;
+}
+// 1 + N, up the rows, in place, state: x[m + 1], x[m + 2]; rhs = false: without a right-hand side
+__device__ __forceinline__ cdf2 chunk_u(const InnerSmemDf& S, int s, int e, float4* x, cdf2 st, bool store,
+                                        bool rhs = true) {
+#pragma unroll 1
+  for (int m = e - 1; m >= s; --m) {
+    const cdf g = rhs ? e_load(&x[m]) : c_zero();
+    const cdf v = e_submul(e_submul(g, e_load(&S.u2[m]), st.y), e_load(&S.u1[m]), st.x);
+    if (store) e_store(&x[m], v);
+    st = {v, st.x};
+  }
+  return st;
+}
+// (1 + N)^dag, down the rows, state: y[m - 1], y[m - 2]; y[m] / conj(diag(U)) is stored
+__device__ __forceinline__ cdf2 chunk_ud(const InnerSmemDf& S, int s, int e, const float4* b, float4* z, cdf2 st,
+                                         bool store, bool rhs = true) {
+#pragma unroll 1
+  for (int m = s; m < e; ++m) {
+    cdf v = rhs ? e_load(&b[m]) : c_zero();
+    if (m >= 2) v = c_submulc(v, e_load(&S.u2[m - 2]), st.y);
+    if (m >= 1) v = c_submulc(v, e_load(&S.u1[m - 1]), st.x);
+    if (store) e_store(&z[m], e_mul(v, c_conj(e_load(&S.uinv[m]))));
+    st = {v, st.x};
+  }
+  return st;
+}
+// the adjoint interchanges and L^dag, up the rows: step m reads z[m] and fixes z[m + 1], so
+// the lane's steps are m = e - 2 .. s - 1 (it fixes its own rows; zs = z[s - 1] is another
+// lane's, read before the side's barrier); state: the pending z[m + 1]
+__device__ __forceinline__ cdf chunk_ld(const InnerSmemDf& S, int k, int s, int e, float4* z, cdf zs, cdf gn,
+                                        bool store) {
+  if (s >= e) return gn;
+  if (e == k) gn = e_load(&z[k - 1]);
+#pragma unroll 1
+  for (int m = e - 2; m >= s - 1 && m >= 0; --m) {
+    const cdf zm = m >= s ? e_load(&z[m]) : zs;
+    const cdf v = c_submulc(zm, e_load(&S.l[m]), gn);
     const bool sw = S.sw[m];
-    e_store(&z[m + 1], sw ? v : gn);
+    if (store) e_store(&z[m + 1], sw ? v : gn);
     gn = sw ? gn : v;
   }
-  e_store(&z[0], gn);
+  if (store && s == 0) e_store(&z[0], gn);
+  return gn;
+}
+// a chunk's map of the first-order recurrences (the product of its multipliers) and of the
+// second-order ones (the recurrence on the two unit states)
+__device__ __forceinline__ cdf map_l(const InnerSmemDf& S, int first, int last, bool conj) {
+  cdf p = c_one();
+  for (int m = first; m <= last; ++m)
+    if (!S.sw[m]) {
+      const cdf lm = e_load(&S.l[m]);
+      p = e_submul(c_zero(), conj ? c_conj(lm) : lm, p);
+    }
+  return p;
 }
 
-__global__ void __launch_bounds__(kInnerThreads) k_inner_df(const int* __restrict__ k_dev,
+// sums of NQ values over the warps [w0, w0 + n) of the block, each thread gets them
+template <int NQ>
+__device__ __forceinline__ void warps_to_red(df64 (&v)[NQ], df64* red) {
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) v[q] = warp_sum(v[q]);
+  if ((threadIdx.x & 31) == 0)
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) red[(threadIdx.x >> 5) * NQ + q] = v[q];
+}
+__device__ __forceinline__ df64 red_sum(const df64* red, int w0, int nq, int q) {
+  df64 s = red[w0 * nq + q];
+#pragma unroll
+  for (int w = 1; w < kSideWarps; ++w) s = s + red[(w0 + w) * nq + q];
+  return s;
+}
+
+__global__ void __launch_bounds__(2 * kSideLanes) k_inner_df(const int* __restrict__ k_dev,
                                                             const int* __restrict__ l_dev, int hermitian,
                                                             const double2* __restrict__ alp,
                                                             const double2* __restrict__ bet,
@@ -969,81 +1122,146 @@ __global__ void __launch_bounds__(kInnerThreads) k_inner_df(const int* __restric
     if (tid == 0) { w.fail[prob] = 1; w.leff[prob] = 0; }
     return;
   }
-  double2* Q = w.Q + (size_t)prob * w.ld * kMaxL;
+  // side 0 (threads 0..127) carries q, side 1 the two-sided process's w; lane t's rows
+  const int side = tid / kSideLanes, t = tid % kSideLanes;
+  const int rows = (k + kSideLanes - 1) / kSideLanes;
+  const int r0 = min(t * rows, k), r1 = min(r0 + rows, k);
+  const bool work = side == 0 || !hermitian;
+  __shared__ ScanShared<cdf, cdf> sh1[2];
+  __shared__ ScanShared<cmat2, cdf2> sh2[2];
+  ScanMaps<cdf> f1;
+  ScanMaps<cmat2> f2;
+  const ScanPos pos1 = scan_pos(side == 0), pos2 = scan_pos(side == 1);
+  {
+    const cdf2 e1 = {c_one(), zero}, e2 = {zero, c_one()};
+    cdf2 m1, m2;
+    if (side == 0) {
+      m1 = chunk_u(S, r0, r1, S.u, e1, false, false);
+      m2 = chunk_u(S, r0, r1, S.u, e2, false, false);
+    } else {
+      m1 = chunk_ud(S, r0, r1, S.w, S.z, e1, false, false);
+      m2 = chunk_ud(S, r0, r1, S.w, S.z, e2, false, false);
+    }
+    scan_setup(f2, sh2[side], cmat2{m1.x, m2.x, m1.y, m2.y}, pos2);
+    const int first = side == 0 ? r0 : max(r0 - 1, 0), last = side == 0 ? min(r1, k - 1) - 1 : r1 - 2;
+    scan_setup(f1, sh1[side], map_l(S, first, r0 < r1 ? last : first - 1, side == 1), pos1);
+  }
+  __syncthreads();
+  // the side's vectors and coefficients: M = H + H^{-1} on q; M^dag on w, whose H^dag has
+  // conj(c[m - 1]) below and conj(a[m + 1]) above the diagonal
+  float4* const X = side == 0 ? S.q : S.w;
+  float4* const XP = side == 0 ? S.qp : S.wp;
+  float4* const U = side == 0 ? S.u : S.z;
+  const float4* const below = side == 0 ? S.a : S.c - 1;
+  const float4* const above = side == 0 ? S.c : S.a + 1;
+  const bool cj = side == 1;
+  // Q keeps the float pairs as they are (k_combine widens them)
+  float4* Q = (float4*)(w.Q + (size_t)prob * w.ld * kMaxL);
   double2* T = w.T + (size_t)prob * kMaxL * 3;
   df64 b_i = df_zero();
   cdf g_i = zero;
   int done = 0;
   const float exhaust_tol = 1e-13f;
   for (int i = 0; i < l; ++i) {
-    for (int m = tid; m < k; m += blockDim.x) Q[(size_t)m * kMaxL + i] = e_to2(e_load(&S.q[m]));
-    if (tid == 0) tri_solve_fwd_df(S, k, S.q, S.u);
-    if (!hermitian && tid == 32) tri_solve_dag_fwd_df(S, k, S.w, S.z);
-    __syncthreads();
-    for (int m = tid; m < k; m += blockDim.x) {
-      const cdf ri = e_load(&S.uinv[m]);
-      e_store(&S.u[m], e_mul(e_load(&S.u[m]), ri));
-      if (!hermitian) e_store(&S.z[m], e_mul(e_load(&S.z[m]), c_conj(ri)));
-    }
-    __syncthreads();
-    if (tid == 0) tri_solve_bwd_df(S, k, S.u);
-    if (!hermitian && tid == 32) tri_solve_dag_bwd_df(S, k, S.z);
-    __syncthreads();
-    float mq2 = 0.f;
-    for (int m = tid; m < k; m += blockDim.x) {
-      cdf t = e_mul(e_load(&S.d[m]), e_load(&S.q[m]));
-      if (m >= 1) t = c_addmul(t, e_load(&S.a[m]), e_load(&S.q[m - 1]));
-      if (m + 1 < k) t = c_addmul(t, e_load(&S.c[m]), e_load(&S.q[m + 1]));
-      t = c_add(t, e_load(&S.u[m]));
-      mq2 += e_abs2hi(t);
-      const cdf qp = e_load(&S.qp[m]);
-      e_store(&S.u[m], hermitian ? e_submul(t, cdf{b_i, df_zero()}, qp) : e_submul(t, g_i, qp));  // p
-      if (!hermitian) {
-        cdf y = e_mul(c_conj(e_load(&S.d[m])), e_load(&S.w[m]));
-        if (m >= 1) y = c_addmulc(y, e_load(&S.c[m - 1]), e_load(&S.w[m - 1]));
-        if (m + 1 < k) y = c_addmulc(y, e_load(&S.a[m + 1]), e_load(&S.w[m + 1]));
-        y = c_add(y, e_load(&S.z[m]));
-        e_store(&S.z[m], e_submul(y, cdf{b_i, df_zero()}, e_load(&S.wp[m])));  // r
+    // u = H^{-1} q, then p = M q - g_i q_{i-1}; z = H^{-dag} w, then r = M^dag w - b_i w_{i-1}
+    // (rows of this lane only, but for the barriers of the scans). Side 0 runs the first-order
+    // recurrence and then the second-order one, side 1 the other way round; each recurrence
+    // from a zero state, then from the state the scan gives.
+    df64 dots[3] = {df_zero(), df_zero(), df_zero()};  // alpha = w^dag p, ||M q||^2
+    if (work) {
+      if (side == 0)
+        for (int m = r0; m < r1; ++m) Q[(size_t)m * kMaxL + i] = S.q[m];
+#pragma unroll 1
+      for (int stage = 0; stage < 2; ++stage) {
+        if (stage == side) {
+          const cdf head = side == 0 && t == 0 ? e_load(&S.q[0]) : zero;  // the first pending row
+          const cdf zs = side == 1 && r0 >= 1 && r0 < r1 ? e_load(&S.z[r0 - 1]) : zero;
+          cdf st = head;
+#pragma unroll 1
+          for (int pass = 0; pass < 2; ++pass) {
+            if (side == 0) st = chunk_l(S, k, r0, r1, S.q, S.u, st, pass == 1);
+            else st = chunk_ld(S, k, r0, r1, S.z, zs, st, pass == 1);
+            if (pass == 0) {
+              st = scan_in(f1, sh1[side], st, pos1, side);
+              if (side == 0 && t == 0) st = head;
+            }
+          }
+        } else {
+          cdf2 st = {zero, zero};
+#pragma unroll 1
+          for (int pass = 0; pass < 2; ++pass) {
+            if (side == 0) st = chunk_u(S, r0, r1, S.u, st, pass == 1);
+            else st = chunk_ud(S, r0, r1, S.w, S.z, st, pass == 1);
+            if (pass == 0) st = scan_in(f2, sh2[side], st, pos2, side);
+          }
+        }
+        side_sync(side);  // the second sweep of side 1 reads the row before this lane's
       }
+      float mq2 = 0.f;
+      const cdf gi = side == 1 || hermitian ? cdf{b_i, df_zero()} : g_i;
+#pragma unroll 1
+      for (int m = r0; m < r1; ++m) {
+        const cdf xm = e_load(&X[m]);
+        cdf dm = e_load(&S.d[m]);
+        if (cj) dm = c_conj(dm);
+        cdf v = c_addmul(e_load(&U[m]), dm, xm);
+        if (m >= 1) {
+          cdf f = e_load(&below[m]);
+          if (cj) f = c_conj(f);
+          v = c_addmul(v, f, e_load(&X[m - 1]));
+        }
+        if (m + 1 < k) {
+          cdf f = e_load(&above[m]);
+          if (cj) f = c_conj(f);
+          v = c_addmul(v, f, e_load(&X[m + 1]));
+        }
+        mq2 += e_abs2hi(v);
+        const cdf pm = e_submul(v, gi, e_load(&XP[m]));
+        e_store(&U[m], pm);
+        if (side == 0) {
+          const cdf wm = hermitian ? xm : e_load(&S.w[m]);
+          dots[0] = df_axpy2(dots[0], wm.re, pm.re, wm.im, pm.im);
+          dots[1] = df_axpy2(dots[1], wm.re, pm.im, -wm.im, pm.re);
+        }
+      }
+      dots[2] = {mq2, 0.f};
+      if (side == 0) warps_to_red(dots, S.red);
     }
     __syncthreads();
-    // alpha = w^dag p (q^dag p in the Hermitian case)
-    df64 are = df_zero(), aim = df_zero();
-    for (int m = tid; m < k; m += blockDim.x) {
-      const cdf wm = e_load(hermitian ? &S.q[m] : &S.w[m]);
-      const cdf pm = e_load(&S.u[m]);
-      are = df_axpy2(are, wm.re, pm.re, wm.im, pm.im);
-      aim = df_axpy2(aim, wm.re, pm.im, -wm.im, pm.re);
-    }
-    are = block_sum_df(are, S.red);
-    aim = hermitian ? df_zero() : block_sum_df(aim, S.red);
-    const df64 mqn = df_sqrt(block_sum_df(df64{mq2, 0.f}, S.red));
+    const df64 are = red_sum(S.red, 0, 3, 0);
+    const df64 aim = hermitian ? df_zero() : red_sum(S.red, 0, 3, 1);
+    const df64 mqn = df_sqrt(red_sum(S.red, 0, 3, 2));
     const cdf a_i = {are, aim};
     if (tid == 0) T[i * 3 + 0] = e_to2(a_i);
     done = i + 1;
     if (i == l - 1) break;
-    // q~ = p - alpha q ; w~ = r - conj(alpha) w ; delta = w~^dag q~
-    df64 dre = df_zero(), dim = df_zero(), n2 = df_zero();
-    for (int m = tid; m < k; m += blockDim.x) {
-      const cdf qt = e_submul(e_load(&S.u[m]), a_i, e_load(&S.q[m]));
-      e_store(&S.u[m], qt);
-      if (hermitian) {
-        n2 = df_axpy2(n2, qt.re, qt.re, qt.im, qt.im);
-      } else {
-        const cdf wt = c_submulc(e_load(&S.z[m]), a_i, e_load(&S.w[m]));
-        e_store(&S.z[m], wt);
-        dre = df_axpy2(dre, wt.re, qt.re, wt.im, qt.im);
-        dim = df_axpy2(dim, wt.re, qt.im, -wt.im, qt.re);
-      }
+    // q~ = p - alpha q ; w~ = r - conj(alpha) w ; delta = w~^dag q~ (side 0 its real part,
+    // side 1 the imaginary part)
+    df64 dl[1] = {df_zero()};
+    const cdf as = cj ? c_conj(a_i) : a_i;
+#pragma unroll 1
+    for (int m = r0; work && m < r1; ++m) {
+      const cdf v = e_submul(e_load(&U[m]), as, e_load(&X[m]));
+      e_store(&U[m], v);
+      if (hermitian) dl[0] = df_axpy2(dl[0], v.re, v.re, v.im, v.im);
     }
+    __syncthreads();  // both sides' q~, w~; S.red is free again
+    if (!hermitian)
+#pragma unroll 1
+      for (int m = r0; m < r1; ++m) {
+        const cdf qt = e_load(&S.u[m]), wt = e_load(&S.z[m]);
+        const df64 y1 = side == 0 ? qt.re : qt.im, y2 = side == 0 ? qt.im : -qt.re;
+        dl[0] = df_axpy2(dl[0], wt.re, y1, wt.im, y2);
+      }
+    warps_to_red(dl, S.red);
+    __syncthreads();
     df64 bn;
     cdf gn;
     if (hermitian) {
-      bn = df_sqrt(block_sum_df(n2, S.red));
+      bn = df_sqrt(red_sum(S.red, 0, 1, 0));
       gn = {bn, df_zero()};
     } else {
-      dre = block_sum_df(dre, S.red);
-      dim = block_sum_df(dim, S.red);
+      const df64 dre = red_sum(S.red, 0, 1, 0), dim = red_sum(S.red, kSideWarps, 1, 0);
       bn = df_sqrt(df_sqrt(df_axpy2(df_zero(), dre, dre, dim, dim)));
       const df64 rb = bn.hi > 0.f ? df_recip(bn) : df_zero();
       gn = {dre * rb, dim * rb};
@@ -1053,15 +1271,12 @@ __global__ void __launch_bounds__(kInnerThreads) k_inner_df(const int* __restric
       T[(i + 1) * 3 + 1] = make_double2(df_to_double(bn), 0.0);
       T[(i + 1) * 3 + 2] = e_to2(gn);
     }
-    const cdf wdiv = e_inv(c_conj(gn));
-    const df64 rbn = df_recip(bn);
-    __syncthreads();
-    for (int m = tid; m < k; m += blockDim.x) {
-      e_store(&S.qp[m], e_load(&S.q[m]));
-      e_store(&S.q[m], c_scale(e_load(&S.u[m]), rbn));
-      if (!hermitian) {
-        e_store(&S.wp[m], e_load(&S.w[m]));
-        e_store(&S.w[m], e_mul(e_load(&S.z[m]), wdiv));
+    if (work) {
+      const cdf sc = e_inv(side == 0 ? cdf{bn, df_zero()} : c_conj(gn));
+#pragma unroll 1
+      for (int m = r0; m < r1; ++m) {
+        XP[m] = X[m];
+        e_store(&X[m], e_mul(e_load(&U[m]), sc));
       }
     }
     b_i = bn;
@@ -1091,7 +1306,9 @@ __global__ void __launch_bounds__(kInnerThreads) k_combine(int count, const int*
   const int le = w.leff[prob];
   const int le2 = le - dl;
   const int tid = threadIdx.x;
+  // the double-float inner level keeps Q as float pairs in the doubles' bytes
   const double2* Q = w.Q + (size_t)prob * w.ld * kMaxL;
+  const bool pairs = w.arith == OV_INNER_DF64;
   const double2* s1 = w.s + (size_t)prob * kMaxL;
   const double2* s2 = w.s + (size_t)(count + prob) * kMaxL;
   const bool bad = fail[prob] != 0 || le <= 0 || !w.rh_ok[prob];
@@ -1111,7 +1328,7 @@ __global__ void __launch_bounds__(kInnerThreads) k_combine(int count, const int*
     double2 v = make_double2(0.0, 0.0), v2 = make_double2(0.0, 0.0);
     if (!bad) {
       for (int i = 0; i < le; ++i) {
-        const double2 qv = Q[(size_t)m * kMaxL + i];
+        const double2 qv = pairs ? e_to2(e_load((const float4*)&Q[(size_t)m * kMaxL + i])) : Q[(size_t)m * kMaxL + i];
         v = zadd(v, zmul(qv, s1[i]));
         if (have_est && i < le2) v2 = zadd(v2, zmul(qv, s2[i]));
       }
@@ -1168,7 +1385,7 @@ cudaError_t run_inner(int count, const int* k_dev, const int* l_dev, int hermiti
     if (w.arith == OV_INNER_DF64) {
       e = cudaFuncSetAttribute(k_inner_df, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
       if (e != cudaSuccess) return e;
-      k_inner_df<<<count, kInnerThreads, sm, st>>>(k_dev, l_dev, hermitian, alp, bet, gam, ldc, w);
+      k_inner_df<<<count, 2 * kSideLanes, sm, st>>>(k_dev, l_dev, hermitian, alp, bet, gam, ldc, w);
     } else {
       e = cudaFuncSetAttribute(k_inner, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
       if (e != cudaSuccess) return e;
