@@ -323,7 +323,7 @@ int ov_mlp_train(float* theta, int n, const float* X, const float* Y, int epochs
  * stopping check at the smallest predicted k* and uses the predicted l (rounded up to a
  * multiple of 8, clamped to [l_min, min(l_max, l)]). The a-posteriori estimates still
  * decide: checks continue past a short prediction, and an inner estimate above tol grows
- * l by 16 and repeats the check (and, for its outer estimate, the one before it). */
+ * l by 16 and repeats the check. */
 int ov_set_sizer(ov_handle* h, const float* theta, int l_min, int l_max);
 /* Coefficients of the last ov_sign_apply / ov_apply for right-hand side `rhs`:
  * alpha_j, beta_j, gamma_j for j = 1..k (complex doubles, host; beta_1 = gamma_1 = 0),

@@ -739,7 +739,7 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
 
   // host-side per-RHS state
   std::vector<int> done(nrhs, 0), kfin(nrhs, 0), lfin(nrhs, 0), itfin(nrhs, 0), stat(nrhs, OV_OK);
-  std::vector<int> kprev(nrhs, 0), kcur(nrhs, 0), kbase(nrhs, 0), lreq(nrhs, std::min(l, kMaxL));
+  std::vector<int> kprev(nrhs, 0), kcur(nrhs, 0), lreq(nrhs, std::min(l, kMaxL));
   std::vector<double> estfin(nrhs, INFINITY), estin(nrhs, NAN);
   std::vector<int> dstatus(nrhs), dkbreak(nrhs), rhst(nrhs), rhit(nrhs), leff(nrhs);
   std::vector<double> eo(nrhs), ei(nrhs);
@@ -994,7 +994,6 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
     for (int r = 0; r < nrhs; ++r) kcur[r] = (dstatus[r] != kStOK && dkbreak[r] > 0) ? std::min(dkbreak[r], j) : j;
     CK(cudaMemcpyAsync(h->ck.p, kcur.data(), sizeof(int) * nrhs, cudaMemcpyHostToDevice, cs));
     CK(cudaMemcpyAsync(h->ckprev.p, kprev.data(), sizeof(int) * nrhs, cudaMemcpyHostToDevice, cs));
-    for (int r = 0; r < nrhs; ++r) kbase[r] = std::max(kprev[r], 1);  // the previous check's k
     const Phase ph_check("stopping check");
     bool regrow = false;
     do {
@@ -1132,19 +1131,7 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
         }
       }
     }
-    if (regrow) {
-      CK(cudaMemcpyAsync(h->cl.p, lreq.data(), sizeof(int) * nrhs, cudaMemcpyHostToDevice, cs));
-      // the check before this one with the grown l as well (unchanged where l did not grow):
-      // against its c with the smaller l the outer estimate would see that c's inner error and
-      // the run would go on for another interval (24^3 x 48 with learned sizing: k = 249 -> 239)
-      CK(cudaMemcpyAsync(h->ck.p, kbase.data(), sizeof(int) * nrhs, cudaMemcpyHostToDevice, cs));
-      CK(run_inner(nrhs, (const int*)h->ck.p, (const int*)h->cl.p, herm ? 1 : 0, c.alp, c.bet, c.gam, c.nv, ld, iw,
-                   o.rh_tol, o.rh_maxit, o.inner_dl, (double2*)h->cc_prev.p, ld, nullptr, h->prec,
-                   (double*)h->c_est_in.p, nullptr, ld, nullptr, nullptr, (int*)h->c_rhst.p, (int*)h->c_rhit.p, 1, cs));
-      h->stats.launches += 3;
-      h->stats.inner_launches += 3;
-      CK(cudaMemcpyAsync(h->ck.p, kcur.data(), sizeof(int) * nrhs, cudaMemcpyHostToDevice, cs));
-    }
+    if (regrow) CK(cudaMemcpyAsync(h->cl.p, lreq.data(), sizeof(int) * nrhs, cudaMemcpyHostToDevice, cs));
     } while (regrow);
     eo_last_max = 0.0;  // an estimate without a previous check (infinite) means unknown
     for (int r = 0; r < nrhs; ++r)
