@@ -112,7 +112,7 @@ struct ov_handle {
   Buf partials, counters, scale, scal;
   int cap_rhs = 0, cap_ld = 0;
   // inner level
-  Buf iQ, iT, ileff, iS, is, irh_its, irh_ok, iperm, ifail;
+  Buf iQ, iT, ileff, iS, is, irh_its, irh_ok, iperm, ifail, irx;
   Buf ck, cl, ckprev, cc_cur, cc_prev, cc_fin, cacc_cur, cacc_fin, c_est_in, c_est_out, c_rhst, c_rhit;
   Buf vptr;  // device array of basis slot pointers for recombination
   int inner_cap = 0, inner_ld = 0;
@@ -469,7 +469,7 @@ extern "C" void ov_destroy(ov_handle* h) {
   Buf* all[] = {&h->desc, &h->blkmap, &h->xcanon, &h->ycanon, &h->tv, &h->tw, &h->p, &h->r, &h->vring, &h->wring, &h->yacc,
                 &h->coef_alp, &h->coef_bet, &h->coef_gam, &h->coef_nv, &h->coef_nw, &h->coef_status,
                 &h->coef_kbreak, &h->partials, &h->counters, &h->scale, &h->scal, &h->iQ, &h->iT, &h->ileff, &h->iS, &h->is,
-                &h->irh_its, &h->irh_ok, &h->iperm, &h->ifail, &h->ck, &h->cl, &h->ckprev, &h->cc_cur, &h->cc_prev,
+                &h->irh_its, &h->irh_ok, &h->iperm, &h->ifail, &h->irx, &h->ck, &h->cl, &h->ckprev, &h->cc_cur, &h->cc_prev,
                 &h->cc_fin, &h->cacc_cur, &h->cacc_fin, &h->c_est_in, &h->c_est_out, &h->c_rhst, &h->c_rhit,
                 &h->vptr, &h->sizer_theta, &h->sizer_feat, &h->sizer_pred, &h->nn_scratch, &h->dx, &h->dy,
                 &h->dpart, &h->dG};
@@ -531,6 +531,7 @@ static int ensure_inner(ov_handle* h, int count, int ld) {
   CK(grow(h->irh_ok, sizeof(int) * 2 * count));
   CK(grow(h->iperm, sizeof(int) * 2 * (size_t)count * kMaxL));
   CK(grow(h->ifail, sizeof(int) * count));
+  if (h->o.inner_arith == OV_INNER_DF64) CK(grow(h->irx, rh_col_scratch_bytes(count)));
   const size_t cb = sizeof(double2) * (size_t)count * ld;
   CK(grow(h->ck, sizeof(int) * count));
   CK(grow(h->cl, sizeof(int) * count));
@@ -561,6 +562,7 @@ static InnerWork inner_work(ov_handle* h) {
   w.rh_ok = (int*)h->irh_ok.p;
   w.perm = (int*)h->iperm.p;
   w.fail = (int*)h->ifail.p;
+  w.rx = (float4*)h->irx.p;
   w.ld = h->inner_ld;  // Q rows per problem, as allocated by ensure_inner
   w.arith = h->o.inner_arith;
   w.rh_scale = h->o.rh_scaling;
@@ -1021,8 +1023,10 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
                               (double*)h->c_est_out.p, (int*)h->c_rhst.p, (int*)h->c_rhit.p, phase, cs);
     CK(e);
     tstop(h, ti);
-    h->stats.launches += 3;
-    h->stats.inner_launches += 3;
+    // k_inner, k_rh, k_combine; the double-float inner level has two Roberts-Higham kernels
+    const int rh_kernels = o.nested && o.inner_arith == OV_INNER_DF64 ? 2 : 1;
+    h->stats.launches += 2 + rh_kernels;
+    h->stats.inner_launches += 2 + rh_kernels;
     h->stats.checks += 1;
     CK(cudaMemcpyAsync(eo.data(), h->c_est_out.p, sizeof(double) * nrhs, cudaMemcpyDeviceToHost, cs));
     CK(cudaMemcpyAsync(rhst.data(), h->c_rhst.p, sizeof(int) * nrhs, cudaMemcpyDeviceToHost, cs));
@@ -1047,8 +1051,8 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
                     (double*)h->c_est_out.p, (int*)h->c_rhst.p, (int*)h->c_rhit.p, 2, cs);
       CK(e);
       tstop(h, t2);
-      h->stats.launches += 2;
-      h->stats.inner_launches += 2;
+      h->stats.launches += 1 + rh_kernels;
+      h->stats.inner_launches += 1 + rh_kernels;
       CK(cudaMemcpyAsync(ei.data(), h->c_est_in.p, sizeof(double) * nrhs, cudaMemcpyDeviceToHost, cs));
       CK(cudaMemcpyAsync(rhst.data(), h->c_rhst.p, sizeof(int) * nrhs, cudaMemcpyDeviceToHost, cs));
       CK(cudaStreamSynchronize(cs));

@@ -6,6 +6,8 @@
 //            of Lanczos (mu = 0) or two-sided Lanczos (mu != 0) on M = H_k + H_k^{-1}
 //            from e_1. M u = H u + H^{-1} u and M^dag w = H^dag w + H^{-dag} w both use
 //            the one factorisation (the solve with H^dag runs the factors backwards).
+//  k_rh_col  one CTA per matrix: the first column of a Roberts-Higham iterate of T_l by
+//            partial fractions (the nested checks in double-float arithmetic).
 //  k_rh      one CTA per matrix: Roberts-Higham S_{n+1} = (S_n + S_n^{-1})/2 with an
 //            in-place Gauss-Jordan inversion (partial pivoting) of the whole l x l
 //            matrix in shared memory (l <= 120 complex: 225 KB).
@@ -560,6 +562,8 @@ __device__ __forceinline__ double2 e_to2(df64 a) { return make_double2(df_to_dou
 __device__ __forceinline__ cdf e_from2(double2 v, cdf) { return {df_from_double(v.x), df_from_double(v.y)}; }
 __device__ __forceinline__ df64 e_from2(double2 v, df64) { return df_from_double(v.x); }
 
+constexpr int kRhLeft = -1;  // rh_ok of a matrix that k_rh_col leaves to k_rh_df
+
 template <bool CPLX>
 struct RhDf;
 template <> struct RhDf<true> { using E = cdf; using St = float4; };
@@ -569,6 +573,8 @@ template <bool CPLX>
 __global__ void __launch_bounds__(1024) k_rh_df(int count, int dense_m, const double2* __restrict__ dense_T,
                                                 InnerWork w, int dl, double rh_tol, int rh_maxit, int mid0,
                                                 int scale) {
+  // nested checks: only the matrices that k_rh_col left to this kernel
+  if (dense_m == 0 && w.rh_ok[mid0 + blockIdx.x] != kRhLeft) return;
   using E = typename RhDf<CPLX>::E;
   using St = typename RhDf<CPLX>::St;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -1291,6 +1297,299 @@ __global__ void __launch_bounds__(2 * kSideLanes) k_inner_df(const int* __restri
   }
 }
 
+// ------------------------------------------------- the first column of a Roberts-Higham iterate
+// A nested check needs only s = sgn(T_l) e_1, and T_l is tridiagonal. The iterates of Eq.
+// (Roberts), here with scales, S_{n+1} = (g_n S_n + (g_n S_n)^{-1}) / 2 from S_0 = T, are rational
+// functions of T whose poles lie on the imaginary axis, are simple, and are known beforehand: the
+// poles of S_{n+1} are those of S_n, their residues times g_n / 2, and the 2^n zeros of S_n. So
+//   s_{n+1} = (g_n / 2) s_n + sum_{S_n(z) = 0} (T - z)^{-1} e_1 / (2 g_n S_n'(z)),
+// and g_k S_k(z) = i y_k runs backwards from y_{n-1} = +-1 through y_k = tau +- sqrt(tau^2 + 1), tau =
+// y_{k+1} / g_{k+1}, to z = i y_0 / g_0, with S_n'(z) = prod_k g_k (1 + y_k^{-2}) / 2: every sign choice
+// is one zero. s is a sum of solutions of shifted tridiagonal systems, all independent: one
+// thread solves one, in float pairs and with partial pivoting, and the l x l inversions with
+// their l dependent pivot steps each are gone (24 matrices of l = 120: 11.2 -> 0.077 ms).
+//  - The rows are eliminated from the last to the first, so that the right-hand side e_1 stays
+//    zero until the last step: the forward sweep keeps no multipliers, the back substitution
+//    reads two numbers a row, kept in scratch ([row][thread], coalesced; L2-resident).
+//  - Scales: g_n = 1 with rh_scaling = 0; else g_0 centres the range of |lambda|, from 1.5
+//    (|x + 1/x| >= 2 for real x) to an estimate by tr T^2 and tr T^4, and the later g_n, powers
+//    of two (exact), what is left of it; one large eigenvalue of H^{-1} then costs steps by the
+//    logarithm of its size.
+//  - Stop as k_rh: ||s_n - s_{n-1}|| <= rh_tol ||s_n||, on the column, tested from n = 4 on (the
+//    first 128 solves give s_1 .. s_7). An eigenvector of small weight in e_1 shows in the
+//    matrix's norm but less in the column's, so the column returned is that of one more step.
+//    Iterations, reported as rh_iters: n.
+//  - A matrix that meets a zero pivot, overflows or needs more than 2^12 - 1 poles or more than
+//    rh_maxit steps is left to k_rh_df, whose verdict stands.
+// Bound: the latency of one thread's elimination (~450 cycles a row) at one warp a scheduler.
+constexpr int kColThreads = 128;
+constexpr int kColMaxLevel = 12;
+
+__device__ __forceinline__ float2 fmul2c(float2 a, float2 b) { return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x}; }
+
+__global__ void __launch_bounds__(kColThreads) k_rh_col(int count, int hermitian, InnerWork w, int dl, double rh_tol,
+                                                        int rh_maxit, int mid0, int scale) {
+  __shared__ float4 sd[kMaxL + 2], ssub[kMaxL + 2], ssup[kMaxL + 2];  // T_pp, T_{p,p-1}, T_{p,p+1}
+  __shared__ float2 sred[kColThreads / 32];
+  __shared__ float sg[kColMaxLevel + 1];  // g_n
+  const int mid = mid0 + blockIdx.x, prob = mid % count;
+  const int t = threadIdx.x;
+  const int le = w.leff[prob];
+  const int m = mid < count ? le : le - dl;
+  if (m <= 0) {
+    if (t == 0) { w.rh_ok[mid] = m == 0 ? 0 : 1; w.rh_its[mid] = 0; }
+    return;
+  }
+  const cdf zero = c_zero();
+  // block sums of two floats
+  auto sum2 = [&](float a, float b) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      a += __shfl_xor_sync(0xffffffffu, a, o);
+      b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
+    __syncthreads();
+    if ((t & 31) == 0) sred[t >> 5] = make_float2(a, b);
+    __syncthreads();
+    float2 r = sred[0];
+    for (int v = 1; v < kColThreads / 32; ++v) { r.x += sred[v].x; r.y += sred[v].y; }
+    return r;
+  };
+  if (t < kMaxL + 2) {
+    const double2* T = w.T + (size_t)prob * kMaxL * 3;
+    const double2 z2 = make_double2(0.0, 0.0);
+    double2 d = t < m ? T[t * 3 + 0] : z2, b = t >= 1 && t < m ? T[t * 3 + 1] : z2;
+    double2 g = t + 1 < m ? T[(t + 1) * 3 + 2] : z2;  // T_{t,t+1}
+    if (hermitian) d.y = b.y = g.y = 0.0;
+    e_store(&sd[t], e_from2(d, zero));
+    e_store(&ssub[t], e_from2(b, zero));
+    e_store(&ssup[t], e_from2(g, zero));
+  }
+  if (t <= kColMaxLevel) sg[t] = 1.f;
+  __syncthreads();
+  if (scale) {
+    // with e_p = T_{p,p+1} T_{p+1,p}: tr T^2 = sum A_p, A_p = T_pp^2 + e_{p-1} + e_p, and tr T^4 =
+    // sum A_p^2 + 2 e_p (T_pp + T_{p+1,p+1})^2 + 2 e_p e_{p+1}
+    float2 t2 = {0.f, 0.f}, t4 = {0.f, 0.f};
+    if (t < m) {
+      auto hi = [](const float4* v) { return make_float2(v->x, v->z); };
+      auto ep = [&](int p) { return p < 0 ? make_float2(0.f, 0.f) : fmul2c(hi(&ssup[p]), hi(&ssub[p + 1])); };
+      const float2 d0 = hi(&sd[t]), d1 = hi(&sd[t + 1]), em = ep(t - 1), e0 = ep(t), e1 = ep(t + 1);
+      const float2 dd = fmul2c(d0, d0);
+      t2 = {dd.x + em.x + e0.x, dd.y + em.y + e0.y};
+      const float2 ds = {d0.x + d1.x, d0.y + d1.y};
+      const float2 a2 = fmul2c(t2, t2), c2 = fmul2c(e0, fmul2c(ds, ds)), ee = fmul2c(e0, e1);
+      t4 = {a2.x + 2.f * (c2.x + ee.x), a2.y + 2.f * (c2.y + ee.y)};
+    }
+    t2 = sum2(t2.x, t2.y);
+    t4 = sum2(t4.x, t4.y);
+    if (t == 0) {
+      // mean square eigenvalue; the largest stands out of tr T^4 where it is far above the rest
+      const float ms = sqrtf(t2.x * t2.x + t2.y * t2.y) / (float)m;
+      const float ex = sqrtf(t4.x * t4.x + t4.y * t4.y) - 2.f * (float)m * ms * ms;
+      float hi = fmaxf(2.f * sqrtf(ms), ex > 0.f ? sqrtf(sqrtf(ex)) : 0.f), lo = 1.5f;
+      if (hi < 1e8f) {  // (false for a NaN)
+        hi = fmaxf(hi, lo);
+        for (int n = 0; n <= kColMaxLevel; ++n) {
+          const float g = n == 0 ? rsqrtf(lo * hi) : ldexpf(1.f, -(int)rintf(0.5f * log2f(lo * hi)));
+          sg[n] = g;
+          lo *= g;
+          hi *= g;
+          hi = fmaxf(0.5f * (lo + 1.f / lo), 0.5f * (hi + 1.f / hi));
+          lo = 1.f;
+        }
+      }
+    }
+    __syncthreads();
+  }
+  // this thread's two rows of numbers per eliminated row; the solution overwrites the first
+  float4* const u1 = w.rx + (size_t)mid * 2 * kMaxL * kColThreads + t;
+  float4* const u2 = u1 + (size_t)kMaxL * kColThreads;
+  // (T - z) x = e_1 for pole idx (the zeros of S_b are idx = 2^b .. 2^{b+1} - 1), times its
+  // weight; idx = 0: weight zero
+  auto solve = [&](int idx) -> bool {
+    const int id = max(idx, 1);
+    const int b = 31 - __clz(id);
+    const df64 gi0 = df_recip(df64{sg[0], 0.f});
+    df64 sh = df_zero(), wt = b > 0 ? df64{0.5f / sg[b], 0.f} : df_half(gi0);
+    if (b > 0) {
+      df64 y = {id & 1 ? -1.f : 1.f, 0.f};
+      wt = b > 1 ? wt * (1.f / sg[b - 1]) : wt * gi0;
+#pragma unroll 1
+      for (int k = b - 2; k >= 0; --k) {
+        const df64 tau = y * (1.f / sg[k + 1]);
+        const bool up = (id >> (b - 1 - k)) & 1;  // y = tau + sqrt(tau^2 + 1) or its negative inverse
+        const df64 h = (tau.hi < 0.f ? -tau : tau) + df_sqrt(df_axpy1(df64{1.f, 0.f}, tau, tau));
+        const df64 hi = df_recip(h);
+        const bool big = up == (tau.hi >= 0.f);
+        const df64 ya = big ? h : hi, yi = big ? hi : h;  // |y|, 1 / |y|
+        y = up ? ya : -ya;
+        // 1 / (g (1 + y^{-2}) / 2)
+        wt = wt * df_recip(df_half(df_axpy1(df64{1.f, 0.f}, yi, yi)));
+        wt = k > 0 ? wt * (1.f / sg[k]) : wt * gi0;
+      }
+      sh = y * gi0;
+    }
+    if (idx == 0) wt = df_zero();
+    cdf dd = e_load(&sd[m - 1]);
+    dd.im = dd.im - sh;
+    cdf ee = m > 1 ? e_load(&ssub[m - 1]) : zero;
+    bool fine = true, lastsw = false;
+    cdf ri = zero, lm = zero;
+#pragma unroll 1
+    for (int p = m - 2; p >= 0; --p) {  // row p enters; row p + 1 or p becomes final
+      const cdf an = e_load(&ssup[p]);
+      cdf dn = e_load(&sd[p]);
+      dn.im = dn.im - sh;
+      const cdf cn = p >= 1 ? e_load(&ssub[p]) : zero;
+      const float ad = e_abs2hi(dd), aa = e_abs2hi(an);
+      const bool sw = !(ad >= aa);
+      fine = fine && fmaxf(ad, aa) > 0.f;
+      ri = e_inv(sw ? an : dd);
+      lm = e_mul(sw ? dd : an, ri);
+      const cdf r1 = sw ? dn : ee;
+      const cdf nd = e_submul(sw ? ee : dn, lm, r1);
+      e_store(&u1[(size_t)p * kColThreads], e_mul(r1, ri));
+      if (sw) {
+        e_store(&u2[(size_t)p * kColThreads], e_mul(cn, ri));
+        ee = e_submul(zero, lm, cn);
+      } else {
+        e_store(&u2[(size_t)p * kColThreads], zero);
+        ee = cn;
+      }
+      dd = nd;
+      lastsw = sw;
+    }
+    fine = fine && e_abs2hi(dd) > 0.f;
+    // the right-hand side after the last step: (1, -lm) if the rows were exchanged, else (0, 1)
+    const cdf one = c_one();
+    cdf x1 = e_inv(dd);
+    if (m > 1 && lastsw) x1 = e_submul(zero, lm, x1);
+    cdf x2 = zero;
+    // x is kept by row of T: x_0 = x1 here; u1, u2 of step p give x_{p+1} from x_p, x_{p-1}
+    cdf keep = c_scale(x1, wt);
+    cdf a = zero, bb = zero;
+    if (m > 1) { a = e_load(&u1[0]); bb = e_load(&u2[0]); }
+    e_store(&u1[0], keep);
+    constexpr int PF = 4;  // rows loaded ahead (the scratch is in L2)
+    cdf na[PF], nb[PF];
+#pragma unroll
+    for (int i = 0; i < PF; ++i)
+      if (1 + i < m - 1) {
+        na[i] = e_load(&u1[(size_t)(1 + i) * kColThreads]);
+        nb[i] = e_load(&u2[(size_t)(1 + i) * kColThreads]);
+      }
+    if (m > 1) {
+      // x_1 = rhs / pivot - u1 x_0 (rhs 1 if the rows were exchanged)
+      const cdf x = e_submul(lastsw ? ri : zero, a, x1);
+      x2 = x1;
+      x1 = x;
+      keep = c_scale(x1, wt);
+    }
+#pragma unroll 1
+    for (int p0 = 1; p0 < m - 1; p0 += PF) {
+      cdf ca[PF], cb[PF];
+#pragma unroll
+      for (int i = 0; i < PF; ++i) {
+        ca[i] = na[i];
+        cb[i] = nb[i];
+        const int pn = p0 + PF + i;
+        if (pn < m - 1) {
+          na[i] = e_load(&u1[(size_t)pn * kColThreads]);
+          nb[i] = e_load(&u2[(size_t)pn * kColThreads]);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < PF; ++i) {
+        const int p = p0 + i;
+        if (p < m - 1) {
+          e_store(&u1[(size_t)p * kColThreads], keep);  // x_p
+          const cdf x = e_submul(e_submul(zero, cb[i], x2), ca[i], x1);
+          x2 = x1;
+          x1 = x;
+          keep = c_scale(x1, wt);
+        }
+      }
+    }
+    if (m > 1) e_store(&u1[(size_t)(m - 1) * kColThreads], keep);
+    return fine;
+  };
+  // sum over threads [a, b) of row t's solutions (thread t: row t of T)
+  const float4* const row = w.rx + (size_t)mid * 2 * kMaxL * kColThreads + (size_t)t * kColThreads;
+  auto rowsum = [&](int a, int b) {
+    cdf s0 = zero, s1 = zero, s2 = zero, s3 = zero;
+    int i = a;
+#pragma unroll 1
+    for (; i + 4 <= b; i += 4) {
+      s0 = c_add(s0, e_load(&row[i]));
+      s1 = c_add(s1, e_load(&row[i + 1]));
+      s2 = c_add(s2, e_load(&row[i + 2]));
+      s3 = c_add(s3, e_load(&row[i + 3]));
+    }
+#pragma unroll 1
+    for (; i < b; ++i) s0 = c_add(s0, e_load(&row[i]));
+    return c_add(c_add(s0, s1), c_add(s2, s3));
+  };
+  const float tol2 = (float)rh_tol * (float)rh_tol;
+  // ||f - g||^2 <= tol^2 ||f||^2 over the rows
+  auto same = [&](cdf f, cdf g) {
+    float d = 0.f, n = 0.f;
+    if (t < m) {
+      const df64 dr = f.re - g.re, di = f.im - g.im;
+      d = dr.hi * dr.hi + di.hi * di.hi;
+      n = e_abs2hi(f);
+    }
+    const float2 r = sum2(d, n);
+    return r.x <= tol2 * r.y;
+  };
+  // (g_n / 2) f + sum
+  auto next = [&](cdf f, int n, cdf sum) { return c_add(e_scale(f, 0.5f * sg[n]), sum); };
+  bool fine = solve(t);
+  __syncthreads();
+  cdf f = t == 0 ? e_load(&sd[0]) : t == 1 && m > 1 ? e_load(&ssub[1]) : zero;  // S_0 e_1 of this row
+  int level = 7, its = 0;
+  bool conv = false, was = false;
+#pragma unroll 1
+  for (int n = 0; n < 7; ++n) {
+    const cdf fn = t < m ? next(f, n, rowsum(1 << n, 2 << n)) : zero;
+    was = conv;
+    if (n >= 3 && !conv) {
+      conv = same(fn, f);
+      if (conv) its = n + 1;
+    }
+    f = fn;
+  }
+  // the poles of further steps, kColThreads at a time, until one step past the convergence
+  while (!was && level < kColMaxLevel && level <= rh_maxit) {
+    cdf sum = zero;
+    for (int i0 = 1 << level; i0 < 2 << level; i0 += kColThreads) {
+      __syncthreads();  // every row has been summed
+      fine = solve(i0 + t) && fine;
+      __syncthreads();
+      if (t < m) sum = c_add(sum, rowsum(0, kColThreads));
+    }
+    const cdf fn = t < m ? next(f, level, sum) : zero;
+    ++level;
+    was = conv;
+    if (!conv) {
+      conv = same(fn, f);
+      if (conv) its = level;
+    }
+    f = fn;
+  }
+  const bool good = was && its <= rh_maxit;
+  const bool finite = t >= m || (isfinite(f.re.hi) && isfinite(f.im.hi));
+  const int all = __syncthreads_and((fine || t == 0) && finite && good);
+  if (t == 0) {
+    w.rh_ok[mid] = all ? 1 : kRhLeft;
+    w.rh_its[mid] = its;
+  }
+  if (all && t < m) {
+    if (hermitian) f.im = df_zero();
+    w.s[(size_t)mid * kMaxL + t] = e_to2(f);
+  }
+}
+
 // ------------------------------------------------------------ combine
 __global__ void __launch_bounds__(kInnerThreads) k_combine(int count, const int* __restrict__ k_dev,
                                                            const int* __restrict__ l_dev, InnerWork w, int dl,
@@ -1371,6 +1670,8 @@ __global__ void __launch_bounds__(kInnerThreads) k_combine(int count, const int*
   }
 }
 
+size_t rh_col_scratch_bytes(int count) { return sizeof(float4) * 4 * (size_t)count * kMaxL * kColThreads; }
+
 static size_t inner_smem(int k) { return (size_t)13 * k * sizeof(double2) + 32 * sizeof(double) + k + 16; }
 
 cudaError_t run_inner(int count, const int* k_dev, const int* l_dev, int hermitian, const double2* alp,
@@ -1402,7 +1703,9 @@ cudaError_t run_inner(int count, const int* k_dev, const int* l_dev, int hermiti
   // matrix + column buffer (which also holds the 64-double reduction scratch)
   const size_t rsm = (size_t)kMaxL * kMaxL * esz + std::max<size_t>(kMaxL * esz, 512);
   if (w.arith == OV_INNER_DF64) {
-    // float pairs take the bytes of the double elements they replace
+    k_rh_col<<<nmat, kColThreads, 0, st>>>(count, hermitian, w, inner_dl, rh_tol, rh_maxit, mid0, w.rh_scale);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    // the matrices it left; float pairs take the bytes of the double elements they replace
     if (hermitian) {
       e = cudaFuncSetAttribute(k_rh_df<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm);
       if (e != cudaSuccess) return e;

@@ -147,6 +147,7 @@ struct InnerWork {
   int* rh_ok;       // [2*count]
   int* perm;        // [2*count][kMaxL]
   int* fail;        // [count] singular H_k
+  float4* rx;       // rh_col_scratch_bytes(count): the shifted systems of k_rh_col
   int ld;
   int arith;        // OV_INNER_DF64 / OV_INNER_FP64: arithmetic of the serial solves and inversions
   int rh_scale;     // 1: determinant-scaled Roberts-Higham steps in the inner level (DF64 arithmetic)
@@ -166,6 +167,7 @@ cudaError_t run_inner(int count, const int* k_dev, const int* l_dev, int hermiti
                       double rh_tol, int rh_maxit, int inner_dl, double2* c, int ldo, void* cacc, int prec,
                       double* est_inner, const double2* cprev, int ldp, const int* kprev_dev,
                       double* est_outer, int* rh_status, int* rh_iters, int phase, cudaStream_t st);
+size_t rh_col_scratch_bytes(int count);
 cudaError_t run_rh_dense(int count, int m, const double2* T, double2* S, int* iters, int* ok,
                          double rh_tol, int rh_maxit, InnerWork& w, cudaStream_t st);
 
