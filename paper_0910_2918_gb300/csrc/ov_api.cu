@@ -112,7 +112,7 @@ struct ov_handle {
   Buf partials, counters, scale, scal;
   int cap_rhs = 0, cap_ld = 0;
   // inner level
-  Buf iQ, iT, ileff, iS, is, irh_its, irh_ok, iperm, ifail, irx;
+  Buf iQ, iT, ileff, iS, is, irh_its, irh_ok, iperm, ifail, irx, icn;
   Buf ck, cl, ckprev, cc_cur, cc_prev, cc_fin, cacc_cur, cacc_fin, c_est_in, c_est_out, c_rhst, c_rhit;
   Buf vptr;  // device array of basis slot pointers for recombination
   int inner_cap = 0, inner_ld = 0;
@@ -469,7 +469,7 @@ extern "C" void ov_destroy(ov_handle* h) {
   Buf* all[] = {&h->desc, &h->blkmap, &h->xcanon, &h->ycanon, &h->tv, &h->tw, &h->p, &h->r, &h->vring, &h->wring, &h->yacc,
                 &h->coef_alp, &h->coef_bet, &h->coef_gam, &h->coef_nv, &h->coef_nw, &h->coef_status,
                 &h->coef_kbreak, &h->partials, &h->counters, &h->scale, &h->scal, &h->iQ, &h->iT, &h->ileff, &h->iS, &h->is,
-                &h->irh_its, &h->irh_ok, &h->iperm, &h->ifail, &h->irx, &h->ck, &h->cl, &h->ckprev, &h->cc_cur, &h->cc_prev,
+                &h->irh_its, &h->irh_ok, &h->iperm, &h->ifail, &h->irx, &h->icn, &h->ck, &h->cl, &h->ckprev, &h->cc_cur, &h->cc_prev,
                 &h->cc_fin, &h->cacc_cur, &h->cacc_fin, &h->c_est_in, &h->c_est_out, &h->c_rhst, &h->c_rhit,
                 &h->vptr, &h->sizer_theta, &h->sizer_feat, &h->sizer_pred, &h->nn_scratch, &h->dx, &h->dy,
                 &h->dpart, &h->dG};
@@ -531,6 +531,7 @@ static int ensure_inner(ov_handle* h, int count, int ld) {
   CK(grow(h->irh_ok, sizeof(int) * 2 * count));
   CK(grow(h->iperm, sizeof(int) * 2 * (size_t)count * kMaxL));
   CK(grow(h->ifail, sizeof(int) * count));
+  CK(grow(h->icn, sizeof(double) * count));
   if (h->o.inner_arith == OV_INNER_DF64) CK(grow(h->irx, rh_col_scratch_bytes(count)));
   const size_t cb = sizeof(double2) * (size_t)count * ld;
   CK(grow(h->ck, sizeof(int) * count));
@@ -551,8 +552,10 @@ static int ensure_inner(ov_handle* h, int count, int ld) {
   return OV_OK;
 }
 
-static InnerWork inner_work(ov_handle* h) {
+static InnerWork inner_work(ov_handle* h, int rows) {
   InnerWork w;
+  w.rows = rows;
+  w.cnorm = (double*)h->icn.p;
   w.Q = (double2*)h->iQ.p;
   w.T = (double2*)h->iT.p;
   w.leff = (int*)h->ileff.p;
@@ -748,7 +751,7 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
   CK(cudaMemcpyAsync(h->cl.p, lreq.data(), sizeof(int) * nrhs, cudaMemcpyHostToDevice, st));
   CK(cudaMemsetAsync(h->cc_fin.p, 0, sizeof(double2) * (size_t)nrhs * ld, st));
   CK(cudaMemsetAsync(h->cacc_fin.p, 0, acc_elem_bytes(h->prec) * (size_t)nrhs * ld, st));
-  InnerWork iw = inner_work(h);
+  InnerWork iw = inner_work(h, nrhs);
   int ndone = 0;
   int j = 0;
   const int first = o.first_check > 0 ? o.first_check : o.check_interval;
@@ -1023,10 +1026,10 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
                               (double*)h->c_est_out.p, (int*)h->c_rhst.p, (int*)h->c_rhit.p, phase, cs);
     CK(e);
     tstop(h, ti);
-    // k_inner, k_rh, k_combine; the double-float inner level has two Roberts-Higham kernels
+    // k_inner, k_rh, k_combine, k_estimate; the double-float inner level has two Roberts-Higham kernels
     const int rh_kernels = o.nested && o.inner_arith == OV_INNER_DF64 ? 2 : 1;
-    h->stats.launches += 2 + rh_kernels;
-    h->stats.inner_launches += 2 + rh_kernels;
+    h->stats.launches += 3 + rh_kernels;
+    h->stats.inner_launches += 3 + rh_kernels;
     h->stats.checks += 1;
     CK(cudaMemcpyAsync(eo.data(), h->c_est_out.p, sizeof(double) * nrhs, cudaMemcpyDeviceToHost, cs));
     CK(cudaMemcpyAsync(rhst.data(), h->c_rhst.p, sizeof(int) * nrhs, cudaMemcpyDeviceToHost, cs));
@@ -1051,8 +1054,8 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
                     (double*)h->c_est_out.p, (int*)h->c_rhst.p, (int*)h->c_rhit.p, 2, cs);
       CK(e);
       tstop(h, t2);
-      h->stats.launches += 1 + rh_kernels;
-      h->stats.inner_launches += 1 + rh_kernels;
+      h->stats.launches += 2 + rh_kernels;
+      h->stats.inner_launches += 2 + rh_kernels;
       CK(cudaMemcpyAsync(ei.data(), h->c_est_in.p, sizeof(double) * nrhs, cudaMemcpyDeviceToHost, cs));
       CK(cudaMemcpyAsync(rhst.data(), h->c_rhst.p, sizeof(int) * nrhs, cudaMemcpyDeviceToHost, cs));
       CK(cudaStreamSynchronize(cs));
@@ -1786,7 +1789,7 @@ extern "C" int ov_inner_sign(ov_handle* h, int count, int ld, const int* k, cons
   cudaMemcpyAsync(dG.p, G.data(), cb, cudaMemcpyHostToDevice, st);
   cudaMemcpyAsync(h->ck.p, k, sizeof(int) * count, cudaMemcpyHostToDevice, st);
   cudaMemcpyAsync(h->cl.p, lv.data(), sizeof(int) * count, cudaMemcpyHostToDevice, st);
-  InnerWork iw = inner_work(h);
+  InnerWork iw = inner_work(h, count);
   cudaError_t e = run_inner(count, (const int*)h->ck.p, (const int*)h->cl.p, hermitian ? 1 : 0, (double2*)dA.p,
                             (double2*)dB.p, (double2*)dG.p, nullptr, ldi, iw, h->o.rh_tol, h->o.rh_maxit, h->o.inner_dl,
                             (double2*)h->cc_cur.p, ldi, nullptr, h->prec, (double*)h->c_est_in.p, nullptr, ldi,
@@ -1866,7 +1869,7 @@ extern "C" int ov_rh_sign(ov_handle* h, int count, int m, const void* T, void* S
     cleanup();
     return OV_ERR_NOMEM;
   }
-  InnerWork iw = inner_work(h);
+  InnerWork iw = inner_work(h, count);
   cudaError_t e = cudaMemcpyAsync(dT.p, T, mb, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess)
     e = run_rh_dense(count, m, (const double2*)dT.p, (double2*)dS.p, (int*)dI.p, (int*)dI.p + count, h->o.rh_tol,

@@ -11,8 +11,9 @@
 //  k_rh      one CTA per matrix: Roberts-Higham S_{n+1} = (S_n + S_n^{-1})/2 with an
 //            in-place Gauss-Jordan inversion (partial pivoting) of the whole l x l
 //            matrix in shared memory (l <= 120 complex: 225 KB).
-//  k_combine one CTA per problem: c = Q_l s, the inner estimate against the leading
-//            (l - dl) block, the outer estimate against the previous check.
+//  k_combine a cluster of CTAs per problem: c = Q_l s and the inner estimate against the
+//            leading (l - dl) block; k_estimate: the outer estimate against the previous check.
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include <algorithm>
@@ -174,9 +175,10 @@ __global__ void __launch_bounds__(kInnerThreads) k_inner(const int* __restrict__
     S.red = (double*)(base + 13 * k);
     S.sw = (unsigned char*)(S.red + 32);
   }
-  const double2* al = alp + (size_t)prob * ldc;
-  const double2* be = bet + (size_t)prob * ldc;
-  const double2* ga = gam + (size_t)prob * ldc;
+  const size_t crow = (size_t)(prob % w.rows) * ldc;
+  const double2* al = alp + crow;
+  const double2* be = bet + crow;
+  const double2* ga = gam + crow;
   for (int m = tid; m < k; m += blockDim.x) {
     double2 dm = al[m + 1];
     double2 am = m >= 1 ? be[m + 1] : make_double2(0.0, 0.0);
@@ -485,6 +487,9 @@ __global__ void __launch_bounds__(1024) k_rh(int count, int dense_m, const doubl
 struct cdf {
   df64 re, im;
 };
+
+__device__ __forceinline__ cdf operator-(cdf a) { return {-a.re, -a.im}; }
+__device__ __forceinline__ cdf operator-(cdf a, cdf b) { return {a.re - b.re, a.im - b.im}; }
 
 __device__ __forceinline__ df64 df_recip(df64 d) {
   const float x = __frcp_rn(d.hi);
@@ -796,141 +801,161 @@ __global__ void __launch_bounds__(1024) k_rh_df(int count, int dense_m, const do
 
 // ------------------------------------------------- inner Krylov in double-float
 // k_inner with every operation on the float pipes: the tridiagonal factorisation (serial), the
-// solves and the vector updates in float pairs, the block reductions in float pairs. Square roots take one
-// Newton step y + (x - y^2) / (2 y) from the float root, quotients multiply by the
-// refined reciprocal (Karp and Markstein, ACM TOMS 23 (1997)). Outputs (T, Q) are double.
+// solves and the vector updates in float pairs, the block reductions in float pairs. Square
+// roots take one Newton step y + (x - y^2) / (2 y) from the float root, quotients multiply by
+// the refined reciprocal (Karp and Markstein, ACM TOMS 23 (1997)). T is written in double, Q in
+// float pairs. At mu = 0 H_k is real symmetric and everything is real (E = df64: a quarter of
+// the arithmetic); E = cdf otherwise.
+__device__ __forceinline__ cdf c_zero() { return {df_zero(), df_zero()}; }
+__device__ __forceinline__ cdf c_one() { return {{1.f, 0.f}, df_zero()}; }
 __device__ __forceinline__ cdf c_add(cdf a, cdf b) { return {a.re + b.re, a.im + b.im}; }
-__device__ __forceinline__ cdf c_conj(cdf a) { return {a.re, -a.im}; }
 __device__ __forceinline__ cdf c_scale(cdf a, df64 s) { return {a.re * s, a.im * s}; }
+__device__ __forceinline__ cdf e_one(cdf) { return c_one(); }
+__device__ __forceinline__ df64 e_one(df64) { return {1.f, 0.f}; }
+__device__ __forceinline__ cdf e_conj(cdf a) { return {a.re, -a.im}; }
+__device__ __forceinline__ df64 e_conj(df64 a) { return a; }
+__device__ __forceinline__ cdf e_real(df64 r, cdf) { return {r, df_zero()}; }
+__device__ __forceinline__ df64 e_real(df64 r, df64) { return r; }
 // a + f r
-__device__ __forceinline__ cdf c_addmul(cdf a, cdf f, cdf r) {
+__device__ __forceinline__ cdf e_addmul(cdf a, cdf f, cdf r) {
   return {df_axpy2(a.re, f.re, r.re, -f.im, r.im), df_axpy2(a.im, f.re, r.im, f.im, r.re)};
 }
-// a + conj(f) r
-__device__ __forceinline__ cdf c_addmulc(cdf a, cdf f, cdf r) {
-  return {df_axpy2(a.re, f.re, r.re, f.im, r.im), df_axpy2(a.im, f.re, r.im, -f.im, r.re)};
-}
+__device__ __forceinline__ df64 e_addmul(df64 a, df64 f, df64 r) { return df_axpy1(a, f, r); }
 // a - conj(f) r
-__device__ __forceinline__ cdf c_submulc(cdf a, cdf f, cdf r) {
+__device__ __forceinline__ cdf e_submulc(cdf a, cdf f, cdf r) {
   return {df_axpy2(a.re, -f.re, r.re, -f.im, r.im), df_axpy2(a.im, -f.re, r.im, f.im, r.re)};
 }
+__device__ __forceinline__ df64 e_submulc(df64 a, df64 f, df64 r) { return df_axpy1(a, -f, r); }
+// d += conj(a) b
+__device__ __forceinline__ void e_dot(df64 (&d)[2], cdf a, cdf b) {
+  d[0] = df_axpy2(d[0], a.re, b.re, a.im, b.im);
+  d[1] = df_axpy2(d[1], a.re, b.im, -a.im, b.re);
+}
+__device__ __forceinline__ void e_dot(df64 (&d)[2], df64 a, df64 b) { d[0] = df_axpy1(d[0], a, b); }
+__device__ __forceinline__ float4 e_pairs(cdf a) { return make_float4(a.re.hi, a.re.lo, a.im.hi, a.im.lo); }
+__device__ __forceinline__ float4 e_pairs(df64 a) { return make_float4(a.hi, a.lo, 0.f, 0.f); }
 __device__ __forceinline__ df64 df_sqrt(df64 x) {
   if (!(x.hi > 0.f)) return df_zero();
   const float y = __fsqrt_rn(x.hi);
   const df64 e = x - df_prod(y, y);
   return df_two_sum(y, __fmul_rn(e.hi, __fdiv_rn(0.5f, y)));
 }
-__device__ __forceinline__ df64 block_sum_df(df64 v, df64* red) {
-  v = warp_sum(v);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  __syncthreads();
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  df64 s = df_zero();
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s = s + red[w];
-  return s;
-}
 
+template <class St>
 struct InnerSmemDf {
-  float4 *d, *a, *c, *uinv, *u1, *u2, *l, *q, *qp, *w, *wp, *u, *z;
+  St *d, *a, *c, *uinv, *u1, *u2, *l, *q, *qp, *w, *wp, *u, *z;
   unsigned char* sw;
   df64* red;
 };
 
-__device__ bool tri_factor_df(const InnerSmemDf& S, int k) {
-  const cdf zero = {df_zero(), df_zero()};
-  cdf dd = e_load(&S.d[0]);
-  cdf ee = k > 1 ? e_load(&S.c[0]) : zero;
+// LU with partial pivoting of the tridiagonal H, U = D (1 + N) (one thread; ia[m] = 1 / H_{m,m-1}
+// beforehand, so that only a row kept in place waits for a reciprocal). False if singular.
+template <class E, class St>
+__device__ bool tri_factor_df(const InnerSmemDf<St>& S, int k, const St* ia) {
+  const E zero = e_zero(E{});
+  E dd = e_load(&S.d[0]);
+  E ee = k > 1 ? e_load(&S.c[0]) : zero;
+  E an = zero, dn = zero, cn = zero, in = zero;
+  if (k > 1) { an = e_load(&S.a[1]); dn = e_load(&S.d[1]); cn = e_load(&S.c[1]); in = e_load(&ia[1]); }
+#pragma unroll 1
   for (int m = 0; m < k - 1; ++m) {
-    const cdf an = e_load(&S.a[m + 1]), dn = e_load(&S.d[m + 1]);
-    const cdf cn = (m + 1 <= k - 2) ? e_load(&S.c[m + 1]) : zero;
-    cdf ri, r1, r2, lm;
-    if (e_abs2hi(dd) >= e_abs2hi(an)) {
-      if (e_abs2hi(dd) == 0.f) return false;
-      ri = e_inv(dd);
-      lm = e_mul(an, ri);
-      r1 = ee; r2 = zero;
-      dd = e_submul(dn, lm, ee);
-      ee = cn;
-      S.sw[m] = 0;
-    } else {
-      ri = e_inv(an);
-      lm = e_mul(dd, ri);
-      r1 = dn; r2 = cn;
-      dd = e_submul(ee, lm, dn);
-      ee = e_submul(zero, lm, cn);
-      S.sw[m] = 1;
+    const E a = an, d = dn, c = cn, ai = in;  // c[k - 1] = 0
+    if (m + 2 < k) {
+      an = e_load(&S.a[m + 2]);
+      dn = e_load(&S.d[m + 2]);
+      cn = e_load(&S.c[m + 2]);
+      in = e_load(&ia[m + 2]);
     }
-    // U = D (1 + N) with D the pivots (1 / D in ri): the solves need 1 / D and the rows of N,
-    // so that each step of their recurrences is one multiply-add
-    e_store(&S.uinv[m], ri);
-    e_store(&S.u1[m], e_mul(r1, ri));
-    e_store(&S.u2[m], e_mul(r2, ri));
-    e_store(&S.l[m], lm);
+    const float pd = e_abs2hi(dd), pa = e_abs2hi(a);
+    if (pd >= pa) {
+      if (pd == 0.f) return false;
+      const E ri = e_inv(dd), lm = e_mul(a, ri);
+      e_store(&S.uinv[m], ri);
+      e_store(&S.u1[m], e_mul(ee, ri));
+      e_store(&S.u2[m], zero);
+      e_store(&S.l[m], lm);
+      S.sw[m] = 0;
+      dd = e_submul(d, lm, ee);
+      ee = c;
+    } else {
+      const E lm = e_mul(dd, ai);
+      e_store(&S.uinv[m], ai);
+      e_store(&S.u1[m], e_mul(d, ai));
+      e_store(&S.u2[m], e_mul(c, ai));
+      e_store(&S.l[m], lm);
+      S.sw[m] = 1;
+      dd = e_submul(ee, lm, d);
+      ee = e_submul(zero, lm, c);
+    }
   }
   if (e_abs2hi(dd) == 0.f) return false;
   e_store(&S.uinv[k - 1], e_inv(dd));
   e_store(&S.u1[k - 1], zero);
   e_store(&S.u2[k - 1], zero);
+  S.sw[k - 1] = 0;
   return true;
 }
 
 // ---- the tridiagonal solves of one inner step, in parallel ----------------------------
 // With the pivoted factors, H^{-1} b is two linear recurrences over the rows (the row
-// interchanges with L, of first order, downwards the rows; 1 + N, of second order, back up)
-// and H^{-dag} b two more. A serial sweep costs k times the latency of one complex
-// multiply-add (~70 cycles), and two threads of a 256-thread CTA ran them: 73 us an inner
-// step at k = 333, nearly all of the inner level. Here each side of the inner step has 128
-// lanes; lane t owns the B = ceil(k / 128) rows [tB, (t + 1) B), runs its rows from a zero
-// state, the states that enter the chunks are found by a scan over the lanes, and the rows
-// run again from them. The scan composes x -> P x + C (P: a complex number, or a 2 x 2
-// matrix for the second-order recurrences); every product of P it needs depends on H only
-// and is formed once per check (scan_setup), so a scan level is one shuffle and one multiply-
-// add. P of the first-order recurrences is a product of multipliers |l| <= 1; P of the
-// second-order ones is a block of U_{II}^{-1} U_{IJ} of consecutive rows I, and the inverse of
-// a diagonal block of a triangular matrix is that block of its inverse, so no entry exceeds
-// ||U^{-1}|| ||U||: the growth that the factors allow anyway (measured against the oracle at
-// k = 31 .. 1000: the errors of the serial sweeps). 3 + 5 + 3 dependent multiply-adds replace
-// 333 at k = 333; 12 problems, l = 120: 8.72 -> 1.44 ms. With the chains gone the step is bound
-// by the float pipe of its SM (48% issue, ~6000 instructions a warp and step). 32 or 64 lanes
-// a side do less work in the scans but run longer chunks: 14.0 and 13.2 against 13.1 ms for
-// the whole inner level there, 12.6 and 9.9 against 9.7 ms at k = 700.
+// interchanges with L downwards, then 1 + N back up) and H^{-dag} b two more. A serial sweep
+// costs k times the latency of one complex multiply-add (~70 cycles), and two threads of a
+// 256-thread CTA ran them: 73 us an inner step at k = 333, nearly all of the inner level. Here
+// each side of the inner step has 128 lanes; a lane owns about B = ceil(k / 128) rows, runs
+// them from a zero state, the states that enter the chunks are found by a scan over the lanes,
+// and the rows run again from them. The scan composes x -> P x + C with numbers P that depend
+// on H only, so every product of P is formed once per check (scan_setup) and a scan level is
+// one shuffle and one multiply-add.
+//  - U has two superdiagonals, the second one only in rows that were exchanged, so two numbers
+//    enter a chunk of 1 + N and P is a 2 x 2 matrix (CPLX). For the real symmetric H_k of mu = 0,
+//    whose eigenvalues lie on both sides of zero, exchanged rows do not follow one another (no
+//    two in a row in the Ritz matrices of this method): there the chunks end at rows that were
+//    not exchanged, at the nominal end or the nearest such row before it, and one number enters.
+//    (In the two-sided process three rows of four are exchanged, runs reach 65 rows and that
+//    form was six times slower.)
+//  - P of the recurrences with L is a product of multipliers |l| <= 1; the elements of P of the
+//    others are elements of U_{II}^{-1} U_{IJ} for consecutive rows I, and the inverse of a
+//    diagonal block of a triangular matrix is that block of its inverse, so |P| <= ||U^{-1}||
+//    ||U||: the growth that the factors allow anyway (measured against the oracle at k = 31 ..
+//    1000: the errors of the serial sweeps).
+// 3 + 5 + 3 dependent multiply-adds replace 333 at k = 333; 12 problems, l = 120: 8.72 -> 1.44 ms
+// (two-sided); at mu = 0, in real arithmetic, the whole inner level 11.0 -> 1.31 ms (1.87 in
+// complex arithmetic). With the chains gone the two-sided step is bound by the
+// float pipe of its SM (48% issue, ~6000 instructions a warp and step). 32 or 64 lanes a side do
+// less work in the scans but run longer chunks: slower from k = 333 on.
 constexpr int kSideLanes = 128;  // lanes of one side (v: threads 0.., w: the rest)
 constexpr int kSideWarps = kSideLanes / 32;
 
-struct cdf2 {  // a second-order state: the two newest values
+// the value of lane `src` (the loops below are kept rolled and shared by the two sides: the
+// step's straight-line code would not stay in the instruction cache)
+__device__ __forceinline__ df64 shfl_lane(df64 v, int src) {
+  return {__shfl_sync(0xffffffffu, v.hi, src), __shfl_sync(0xffffffffu, v.lo, src)};
+}
+__device__ __forceinline__ cdf shfl_lane(cdf v, int src) { return {shfl_lane(v.re, src), shfl_lane(v.im, src)}; }
+struct cdf2 {  // the state of a second-order recurrence: the two newest values
   cdf x, y;
 };
 struct cmat2 {
   cdf a, b, c, d;
 };
-__device__ __forceinline__ cdf c_zero() { return {df_zero(), df_zero()}; }
-__device__ __forceinline__ cdf c_one() { return {{1.f, 0.f}, df_zero()}; }
-__device__ __forceinline__ cdf2 lin(cmat2 m, cdf2 s, cdf2 add) {
-  return {c_addmul(c_addmul(add.x, m.a, s.x), m.b, s.y), c_addmul(c_addmul(add.y, m.c, s.x), m.d, s.y)};
-}
-__device__ __forceinline__ cdf lin(cdf m, cdf s, cdf add) { return c_addmul(add, m, s); }
-__device__ __forceinline__ cdf compose(cdf f, cdf g) { return e_mul(f, g); }  // f after g
-__device__ __forceinline__ cmat2 compose(cmat2 f, cmat2 g) {
-  const cdf z = c_zero();
-  return {c_addmul(c_addmul(z, f.a, g.a), f.b, g.c), c_addmul(c_addmul(z, f.a, g.b), f.b, g.d),
-          c_addmul(c_addmul(z, f.c, g.a), f.d, g.c), c_addmul(c_addmul(z, f.c, g.b), f.d, g.d)};
-}
-__device__ __forceinline__ void state_zero(cdf& s) { s = c_zero(); }
-__device__ __forceinline__ void state_zero(cdf2& s) { s = {c_zero(), c_zero()}; }
-__device__ __forceinline__ void map_one(cdf& m) { m = c_one(); }
-__device__ __forceinline__ void map_one(cmat2& m) { m = {c_one(), c_zero(), c_zero(), c_one()}; }
-
-// the value of lane `src` (the loops below are kept rolled and shared by the two sides: the
-// step's straight-line code would not stay in the instruction cache)
-__device__ __forceinline__ float shfl_lane(float v, int src) { return __shfl_sync(0xffffffffu, v, src); }
-__device__ __forceinline__ cdf shfl_lane(cdf v, int src) {
-  return {{shfl_lane(v.re.hi, src), shfl_lane(v.re.lo, src)}, {shfl_lane(v.im.hi, src), shfl_lane(v.im.lo, src)}};
-}
 __device__ __forceinline__ cdf2 shfl_lane(cdf2 v, int src) { return {shfl_lane(v.x, src), shfl_lane(v.y, src)}; }
 __device__ __forceinline__ cmat2 shfl_lane(cmat2 v, int src) {
   return {shfl_lane(v.a, src), shfl_lane(v.b, src), shfl_lane(v.c, src), shfl_lane(v.d, src)};
 }
+// the map m applied to a state, plus add; the map f after g; the identity
+template <class E>
+__device__ __forceinline__ E lin(E m, E s, E add) { return e_addmul(add, m, s); }
+__device__ __forceinline__ cdf2 lin(cmat2 m, cdf2 s, cdf2 add) {
+  return {e_addmul(e_addmul(add.x, m.a, s.x), m.b, s.y), e_addmul(e_addmul(add.y, m.c, s.x), m.d, s.y)};
+}
+template <class E>
+__device__ __forceinline__ E compose(E f, E g) { return e_mul(f, g); }
+__device__ __forceinline__ cmat2 compose(cmat2 f, cmat2 g) {
+  return {e_addmul(e_mul(f.a, g.a), f.b, g.c), e_addmul(e_mul(f.a, g.b), f.b, g.d),
+          e_addmul(e_mul(f.c, g.a), f.d, g.c), e_addmul(e_mul(f.c, g.b), f.d, g.d)};
+}
+__device__ __forceinline__ cmat2 e_one(cmat2) { return {c_one(), c_zero(), c_zero(), c_one()}; }
+__device__ __forceinline__ cdf2 e_zero(cdf2) { return {c_zero(), c_zero()}; }
 // barrier over one side's warps
 __device__ __forceinline__ void side_sync(int side) {
   asm volatile("bar.sync %0, %1;" ::"r"(1 + side), "n"(kSideLanes) : "memory");
@@ -956,8 +981,7 @@ __device__ __forceinline__ ScanPos scan_pos(bool up) {
   return {lane, up ? lane : 31 - lane, up ? w : kSideWarps - 1 - w, up ? -1 : 1};
 }
 template <class M, class St>
-__device__ __forceinline__ void scan_setup(ScanMaps<M>& f, ScanShared<M, St>& sh, M chunk, ScanPos ps) {
-  M p = chunk;
+__device__ __forceinline__ void scan_setup(ScanMaps<M>& f, ScanShared<M, St>& sh, M p, ScanPos ps) {
 #pragma unroll 1
   for (int lev = 0; lev < 5; ++lev) {
     f.lev[lev] = p;
@@ -965,7 +989,7 @@ __device__ __forceinline__ void scan_setup(ScanMaps<M>& f, ScanShared<M, St>& sh
     if (ps.li >= (1 << lev)) p = compose(p, q);
   }
   f.excl = shfl_lane(p, (ps.lane + ps.dir) & 31);
-  if (ps.li == 0) map_one(f.excl);
+  if (ps.li == 0) f.excl = e_one(M{});
   if (ps.li == 31) sh.total[ps.wi] = p;
 }
 // the state that enters this lane's chunk, from the states c that the chunks leave when they
@@ -980,7 +1004,7 @@ __device__ __forceinline__ St scan_in(const ScanMaps<M>& f, ScanShared<M, St>& s
   }
   if (ps.li == 31) sh.carry[ps.wi] = c;
   St in = shfl_lane(c, (ps.lane + ps.dir) & 31);
-  if (ps.li == 0) state_zero(in);
+  if (ps.li == 0) in = e_zero(St{});
   side_sync(side);
   if (ps.wi == 0) return in;
   St s = sh.carry[0];
@@ -993,17 +1017,17 @@ __device__ __forceinline__ St scan_in(const ScanMaps<M>& f, ScanShared<M, St>& s
 }
 
 // One lane's rows [s, e) of the four recurrences; each returns the state it leaves and, with
-// `store`, writes its values.
+// `store`, writes its values. rhs = false: without a right-hand side (for the chunk's map).
 // row interchanges and L, down the rows, state: the pending row; x[m] / diag(U) is stored
-__device__ __forceinline__ cdf chunk_l(const InnerSmemDf& S, int k, int s, int e, const float4* b, float4* x, cdf cur,
-                                       bool store) {
+template <class E, class St>
+__device__ __forceinline__ E chunk_l(const InnerSmemDf<St>& S, int k, int s, int e, const St* b, St* x, E cur, bool store) {
 #pragma unroll 1
   for (int m = s; m < e; ++m) {
-    cdf bsel = cur;
+    E bsel = cur;
     if (m < k - 1) {
-      const cdf nb = e_load(&b[m + 1]);
+      const E nb = e_load(&b[m + 1]);
       const bool sw = S.sw[m];
-      const cdf asel = sw ? cur : nb;
+      const E asel = sw ? cur : nb;
       bsel = sw ? nb : cur;
       cur = e_submul(asel, e_load(&S.l[m]), bsel);
     }
@@ -1011,9 +1035,9 @@ __device__ __forceinline__ cdf chunk_l(const InnerSmemDf& S, int k, int s, int e
   }
   return cur;
 }
-// 1 + N, up the rows, in place, state: x[m + 1], x[m + 2]; rhs = false: without a right-hand side
-__device__ __forceinline__ cdf2 chunk_u(const InnerSmemDf& S, int s, int e, float4* x, cdf2 st, bool store,
-                                        bool rhs = true) {
+// 1 + N, up the rows, in place, state: x[m + 1], x[m + 2]
+__device__ __forceinline__ cdf2 chunk_u(const InnerSmemDf<float4>& S, int s, int e, float4* x, cdf2 st, bool store,
+                                        bool rhs) {
 #pragma unroll 1
   for (int m = e - 1; m >= s; --m) {
     const cdf g = rhs ? e_load(&x[m]) : c_zero();
@@ -1023,15 +1047,29 @@ __device__ __forceinline__ cdf2 chunk_u(const InnerSmemDf& S, int s, int e, floa
   }
   return st;
 }
+// the same where row e - 1 was not exchanged, state: x[m + 1]
+__device__ __forceinline__ df64 chunk_u(const InnerSmemDf<float2>& S, int s, int e, float2* x, df64 x1, bool store,
+                                        bool rhs) {
+  df64 x2 = df_zero();
+#pragma unroll 1
+  for (int m = e - 1; m >= s; --m) {
+    const df64 g = rhs ? e_load(&x[m]) : df_zero();
+    const df64 v = e_submul(e_submul(g, e_load(&S.u2[m]), x2), e_load(&S.u1[m]), x1);
+    if (store) e_store(&x[m], v);
+    x2 = x1;
+    x1 = v;
+  }
+  return x1;
+}
 // (1 + N)^dag, down the rows, state: y[m - 1], y[m - 2]; y[m] / conj(diag(U)) is stored
-__device__ __forceinline__ cdf2 chunk_ud(const InnerSmemDf& S, int s, int e, const float4* b, float4* z, cdf2 st,
-                                         bool store, bool rhs = true) {
+__device__ __forceinline__ cdf2 chunk_ud(const InnerSmemDf<float4>& S, int s, int e, const float4* b, float4* z, cdf2 st,
+                                         bool store, bool rhs) {
 #pragma unroll 1
   for (int m = s; m < e; ++m) {
     cdf v = rhs ? e_load(&b[m]) : c_zero();
-    if (m >= 2) v = c_submulc(v, e_load(&S.u2[m - 2]), st.y);
-    if (m >= 1) v = c_submulc(v, e_load(&S.u1[m - 1]), st.x);
-    if (store) e_store(&z[m], e_mul(v, c_conj(e_load(&S.uinv[m]))));
+    if (m >= 2) v = e_submulc(v, e_load(&S.u2[m - 2]), st.y);
+    if (m >= 1) v = e_submulc(v, e_load(&S.u1[m - 1]), st.x);
+    if (store) e_store(&z[m], e_mul(v, e_conj(e_load(&S.uinv[m]))));
     st = {v, st.x};
   }
   return st;
@@ -1039,14 +1077,14 @@ __device__ __forceinline__ cdf2 chunk_ud(const InnerSmemDf& S, int s, int e, con
 // the adjoint interchanges and L^dag, up the rows: step m reads z[m] and fixes z[m + 1], so
 // the lane's steps are m = e - 2 .. s - 1 (it fixes its own rows; zs = z[s - 1] is another
 // lane's, read before the side's barrier); state: the pending z[m + 1]
-__device__ __forceinline__ cdf chunk_ld(const InnerSmemDf& S, int k, int s, int e, float4* z, cdf zs, cdf gn,
-                                        bool store) {
+template <class E, class St>
+__device__ __forceinline__ E chunk_ld(const InnerSmemDf<St>& S, int k, int s, int e, St* z, E zs, E gn, bool store) {
   if (s >= e) return gn;
   if (e == k) gn = e_load(&z[k - 1]);
 #pragma unroll 1
   for (int m = e - 2; m >= s - 1 && m >= 0; --m) {
-    const cdf zm = m >= s ? e_load(&z[m]) : zs;
-    const cdf v = c_submulc(zm, e_load(&S.l[m]), gn);
+    const E zm = m >= s ? e_load(&z[m]) : zs;
+    const E v = e_submulc(zm, e_load(&S.l[m]), gn);
     const bool sw = S.sw[m];
     if (store) e_store(&z[m + 1], sw ? v : gn);
     gn = sw ? gn : v;
@@ -1054,19 +1092,19 @@ __device__ __forceinline__ cdf chunk_ld(const InnerSmemDf& S, int k, int s, int 
   if (store && s == 0) e_store(&z[0], gn);
   return gn;
 }
-// a chunk's map of the first-order recurrences (the product of its multipliers) and of the
-// second-order ones (the recurrence on the two unit states)
-__device__ __forceinline__ cdf map_l(const InnerSmemDf& S, int first, int last, bool conj) {
-  cdf p = c_one();
+// the product of the multipliers of steps first .. last (conjugated for the adjoint)
+template <class E, class St>
+__device__ __forceinline__ E map_l(const InnerSmemDf<St>& S, int first, int last, bool conj) {
+  E p = e_one(E{});
   for (int m = first; m <= last; ++m)
     if (!S.sw[m]) {
-      const cdf lm = e_load(&S.l[m]);
-      p = e_submul(c_zero(), conj ? c_conj(lm) : lm, p);
+      const E lm = e_load(&S.l[m]);
+      p = e_submul(e_zero(E{}), conj ? e_conj(lm) : lm, p);
     }
   return p;
 }
 
-// sums of NQ values over the warps [w0, w0 + n) of the block, each thread gets them
+// each warp's sums of NQ values into red[warp][NQ]
 template <int NQ>
 __device__ __forceinline__ void warps_to_red(df64 (&v)[NQ], df64* red) {
 #pragma unroll
@@ -1075,26 +1113,35 @@ __device__ __forceinline__ void warps_to_red(df64 (&v)[NQ], df64* red) {
 #pragma unroll
     for (int q = 0; q < NQ; ++q) red[(threadIdx.x >> 5) * NQ + q] = v[q];
 }
+// sum over the four warps from w0 on
 __device__ __forceinline__ df64 red_sum(const df64* red, int w0, int nq, int q) {
-  df64 s = red[w0 * nq + q];
-#pragma unroll
-  for (int w = 1; w < kSideWarps; ++w) s = s + red[(w0 + w) * nq + q];
-  return s;
+  static_assert(kSideWarps == 4, "four warps a side");
+  const df64 s = red[w0 * nq + q] + red[(w0 + 1) * nq + q];
+  const df64 t = red[(w0 + 2) * nq + q] + red[(w0 + 3) * nq + q];
+  return s + t;
 }
 
-__global__ void __launch_bounds__(2 * kSideLanes) k_inner_df(const int* __restrict__ k_dev,
-                                                            const int* __restrict__ l_dev, int hermitian,
-                                                            const double2* __restrict__ alp,
-                                                            const double2* __restrict__ bet,
-                                                            const double2* __restrict__ gam, int ldc, InnerWork w) {
+template <bool CPLX>
+struct UScan;
+template <> struct UScan<true> { using M = cmat2; using S = cdf2; };
+template <> struct UScan<false> { using M = df64; using S = df64; };
+
+// CPLX: two-sided Lanczos, side 0 (threads 0 .. 127) carries q, side 1 w; else Lanczos on the
+// real symmetric H, one side
+template <bool CPLX>
+__global__ void __launch_bounds__((CPLX ? 2 : 1) * kSideLanes)
+    k_inner_df(const int* __restrict__ k_dev, const int* __restrict__ l_dev, const double2* __restrict__ alp,
+               const double2* __restrict__ bet, const double2* __restrict__ gam, int ldc, InnerWork w) {
+  using E = typename RhDf<CPLX>::E;
+  using St = typename RhDf<CPLX>::St;
   extern __shared__ __align__(16) unsigned char smem[];
   const int prob = blockIdx.x;
   const int k = k_dev[prob];
   const int l = min(l_dev[prob], k);
   const int tid = threadIdx.x;
-  InnerSmemDf S;
+  InnerSmemDf<St> S;
   {
-    float4* base = (float4*)smem;
+    St* base = (St*)smem;
     S.d = base; S.a = base + k; S.c = base + 2 * k;
     S.uinv = base + 3 * k; S.u1 = base + 4 * k; S.u2 = base + 5 * k; S.l = base + 6 * k;
     S.q = base + 7 * k; S.qp = base + 8 * k; S.w = base + 9 * k; S.wp = base + 10 * k;
@@ -1102,19 +1149,20 @@ __global__ void __launch_bounds__(2 * kSideLanes) k_inner_df(const int* __restri
     S.red = (df64*)(base + 13 * k);
     S.sw = (unsigned char*)(S.red + 32);
   }
-  const cdf zero = {df_zero(), df_zero()};
-  const double2* al = alp + (size_t)prob * ldc;
-  const double2* be = bet + (size_t)prob * ldc;
-  const double2* ga = gam + (size_t)prob * ldc;
+  const E zero = e_zero(E{});
+  const size_t crow = (size_t)(prob % w.rows) * ldc;
+  const double2* al = alp + crow;
+  const double2* be = bet + crow;
+  const double2* ga = gam + crow;
+  const double2 z2 = make_double2(0.0, 0.0);
   for (int m = tid; m < k; m += blockDim.x) {
-    double2 dm = al[m + 1];
-    double2 am = m >= 1 ? be[m + 1] : make_double2(0.0, 0.0);
-    double2 cm = m + 1 < k ? ga[m + 2] : make_double2(0.0, 0.0);
-    if (hermitian) { dm.y = 0.0; am.y = 0.0; cm = m + 1 < k ? make_double2(be[m + 2].x, 0.0) : cm; }
-    e_store(&S.d[m], e_from2(dm, zero));
-    e_store(&S.a[m], e_from2(am, zero));
-    e_store(&S.c[m], e_from2(cm, zero));
-    const cdf q0 = m == 0 ? cdf{{1.f, 0.f}, df_zero()} : zero;
+    // at mu = 0 the superdiagonal is beta too, imaginary parts are ignored
+    const E am = e_from2(m >= 1 ? be[m + 1] : z2, zero);
+    e_store(&S.d[m], e_from2(al[m + 1], zero));
+    e_store(&S.a[m], am);
+    e_store(&S.c[m], e_from2(m + 1 < k ? (CPLX ? ga[m + 2] : be[m + 2]) : z2, zero));
+    e_store(&S.u[m], e_inv(am));  // for the factorisation
+    const E q0 = m == 0 ? e_one(E{}) : zero;
     e_store(&S.q[m], q0);
     e_store(&S.w[m], q0);
     e_store(&S.qp[m], zero);
@@ -1122,170 +1170,172 @@ __global__ void __launch_bounds__(2 * kSideLanes) k_inner_df(const int* __restri
   }
   __syncthreads();
   __shared__ int s_ok;
-  if (tid == 0) s_ok = tri_factor_df(S, k) ? 1 : 0;
+  if (tid == 0) s_ok = tri_factor_df<E, St>(S, k, S.u) ? 1 : 0;
   __syncthreads();
   if (!s_ok) {
     if (tid == 0) { w.fail[prob] = 1; w.leff[prob] = 0; }
     return;
   }
-  // side 0 (threads 0..127) carries q, side 1 the two-sided process's w; lane t's rows
-  const int side = tid / kSideLanes, t = tid % kSideLanes;
+  const int side = CPLX ? tid / kSideLanes : 0, t = tid % kSideLanes;
+  // this lane's rows [r0, r1); at mu = 0 the chunks end at rows that were not exchanged
   const int rows = (k + kSideLanes - 1) / kSideLanes;
-  const int r0 = min(t * rows, k), r1 = min(r0 + rows, k);
-  const bool work = side == 0 || !hermitian;
-  __shared__ ScanShared<cdf, cdf> sh1[2];
-  __shared__ ScanShared<cmat2, cdf2> sh2[2];
-  ScanMaps<cdf> f1;
-  ScanMaps<cmat2> f2;
-  const ScanPos pos1 = scan_pos(side == 0), pos2 = scan_pos(side == 1);
+  int r0 = min(t * rows, k), r1 = min((t + 1) * rows, k);
+  if constexpr (!CPLX) {
+    while (r0 < k && r0 > 0 && S.sw[r0 - 1]) --r0;
+    while (r1 < k && r1 > 0 && S.sw[r1 - 1]) --r1;
+  }
+  // fl: the recurrence with L (side 0: down the rows), fu: the one with U (side 1: down the
+  // rows), Mu and Su its maps and states
+  using Mu = typename UScan<CPLX>::M;
+  using Su = typename UScan<CPLX>::S;
+  __shared__ ScanShared<E, E> shl[CPLX ? 2 : 1];
+  __shared__ ScanShared<Mu, Su> shu[CPLX ? 2 : 1];
+  ScanMaps<E> fl;
+  ScanMaps<Mu> fu;
+  const ScanPos posl = scan_pos(side == 0), posu = scan_pos(side == 1);
   {
-    const cdf2 e1 = {c_one(), zero}, e2 = {zero, c_one()};
-    cdf2 m1, m2;
-    if (side == 0) {
-      m1 = chunk_u(S, r0, r1, S.u, e1, false, false);
-      m2 = chunk_u(S, r0, r1, S.u, e2, false, false);
+    if constexpr (CPLX) {
+      const cdf2 e1 = {c_one(), zero}, e2 = {zero, c_one()};
+      const cdf2 m1 = side == 0 ? chunk_u(S, r0, r1, S.u, e1, false, false) : chunk_ud(S, r0, r1, S.w, S.z, e1, false, false);
+      const cdf2 m2 = side == 0 ? chunk_u(S, r0, r1, S.u, e2, false, false) : chunk_ud(S, r0, r1, S.w, S.z, e2, false, false);
+      scan_setup(fu, shu[side], cmat2{m1.x, m2.x, m1.y, m2.y}, posu);
     } else {
-      m1 = chunk_ud(S, r0, r1, S.w, S.z, e1, false, false);
-      m2 = chunk_ud(S, r0, r1, S.w, S.z, e2, false, false);
+      scan_setup(fu, shu[side], chunk_u(S, r0, r1, S.u, e_one(E{}), false, false), posu);
     }
-    scan_setup(f2, sh2[side], cmat2{m1.x, m2.x, m1.y, m2.y}, pos2);
     const int first = side == 0 ? r0 : max(r0 - 1, 0), last = side == 0 ? min(r1, k - 1) - 1 : r1 - 2;
-    scan_setup(f1, sh1[side], map_l(S, first, r0 < r1 ? last : first - 1, side == 1), pos1);
+    scan_setup(fl, shl[side], map_l<E, St>(S, first, r0 < r1 ? last : first - 1, side == 1), posl);
   }
   __syncthreads();
   // the side's vectors and coefficients: M = H + H^{-1} on q; M^dag on w, whose H^dag has
   // conj(c[m - 1]) below and conj(a[m + 1]) above the diagonal
-  float4* const X = side == 0 ? S.q : S.w;
-  float4* const XP = side == 0 ? S.qp : S.wp;
-  float4* const U = side == 0 ? S.u : S.z;
-  const float4* const below = side == 0 ? S.a : S.c - 1;
-  const float4* const above = side == 0 ? S.c : S.a + 1;
+  St* const X = side == 0 ? S.q : S.w;
+  St* const XP = side == 0 ? S.qp : S.wp;
+  St* const U = side == 0 ? S.u : S.z;
+  const St* const below = side == 0 ? S.a : S.c - 1;
+  const St* const above = side == 0 ? S.c : S.a + 1;
   const bool cj = side == 1;
   // Q keeps the float pairs as they are (k_combine widens them)
   float4* Q = (float4*)(w.Q + (size_t)prob * w.ld * kMaxL);
   double2* T = w.T + (size_t)prob * kMaxL * 3;
-  df64 b_i = df_zero();
-  cdf g_i = zero;
+  E b_i = zero, g_i = zero;
   int done = 0;
   const float exhaust_tol = 1e-13f;
   for (int i = 0; i < l; ++i) {
     // u = H^{-1} q, then p = M q - g_i q_{i-1}; z = H^{-dag} w, then r = M^dag w - b_i w_{i-1}
-    // (rows of this lane only, but for the barriers of the scans). Side 0 runs the first-order
-    // recurrence and then the second-order one, side 1 the other way round; each recurrence
-    // from a zero state, then from the state the scan gives.
+    // (rows of this lane only, but for the barriers of the scans). Side 0 runs the recurrence
+    // with L and then the one with U, side 1 the other way round; each from a zero state, then
+    // from the state the scan gives.
     df64 dots[3] = {df_zero(), df_zero(), df_zero()};  // alpha = w^dag p, ||M q||^2
-    if (work) {
-      if (side == 0)
-        for (int m = r0; m < r1; ++m) Q[(size_t)m * kMaxL + i] = S.q[m];
+    if (side == 0)
+      for (int m = r0; m < r1; ++m) Q[(size_t)m * kMaxL + i] = e_pairs(e_load(&S.q[m]));
 #pragma unroll 1
-      for (int stage = 0; stage < 2; ++stage) {
-        if (stage == side) {
-          const cdf head = side == 0 && t == 0 ? e_load(&S.q[0]) : zero;  // the first pending row
-          const cdf zs = side == 1 && r0 >= 1 && r0 < r1 ? e_load(&S.z[r0 - 1]) : zero;
-          cdf st = head;
+    for (int stage = 0; stage < 2; ++stage) {
+      if (stage == side) {
+        const E head = side == 0 && t == 0 ? e_load(&S.q[0]) : zero;  // the first pending row
+        const E zs = side == 1 && r0 >= 1 && r0 < r1 ? e_load(&S.z[r0 - 1]) : zero;
+        E st = head;
 #pragma unroll 1
-          for (int pass = 0; pass < 2; ++pass) {
-            if (side == 0) st = chunk_l(S, k, r0, r1, S.q, S.u, st, pass == 1);
-            else st = chunk_ld(S, k, r0, r1, S.z, zs, st, pass == 1);
-            if (pass == 0) {
-              st = scan_in(f1, sh1[side], st, pos1, side);
-              if (side == 0 && t == 0) st = head;
-            }
-          }
-        } else {
-          cdf2 st = {zero, zero};
-#pragma unroll 1
-          for (int pass = 0; pass < 2; ++pass) {
-            if (side == 0) st = chunk_u(S, r0, r1, S.u, st, pass == 1);
-            else st = chunk_ud(S, r0, r1, S.w, S.z, st, pass == 1);
-            if (pass == 0) st = scan_in(f2, sh2[side], st, pos2, side);
+        for (int pass = 0; pass < 2; ++pass) {
+          if (side == 0) st = chunk_l(S, k, r0, r1, S.q, S.u, st, pass == 1);
+          else if constexpr (CPLX) st = chunk_ld(S, k, r0, r1, S.z, zs, st, pass == 1);
+          if (pass == 0) {
+            st = scan_in(fl, shl[side], st, posl, side);
+            if (side == 0 && t == 0) st = head;
           }
         }
-        side_sync(side);  // the second sweep of side 1 reads the row before this lane's
-      }
-      float mq2 = 0.f;
-      const cdf gi = side == 1 || hermitian ? cdf{b_i, df_zero()} : g_i;
+      } else {
+        Su st = e_zero(Su{});
 #pragma unroll 1
-      for (int m = r0; m < r1; ++m) {
-        const cdf xm = e_load(&X[m]);
-        cdf dm = e_load(&S.d[m]);
-        if (cj) dm = c_conj(dm);
-        cdf v = c_addmul(e_load(&U[m]), dm, xm);
-        if (m >= 1) {
-          cdf f = e_load(&below[m]);
-          if (cj) f = c_conj(f);
-          v = c_addmul(v, f, e_load(&X[m - 1]));
-        }
-        if (m + 1 < k) {
-          cdf f = e_load(&above[m]);
-          if (cj) f = c_conj(f);
-          v = c_addmul(v, f, e_load(&X[m + 1]));
-        }
-        mq2 += e_abs2hi(v);
-        const cdf pm = e_submul(v, gi, e_load(&XP[m]));
-        e_store(&U[m], pm);
-        if (side == 0) {
-          const cdf wm = hermitian ? xm : e_load(&S.w[m]);
-          dots[0] = df_axpy2(dots[0], wm.re, pm.re, wm.im, pm.im);
-          dots[1] = df_axpy2(dots[1], wm.re, pm.im, -wm.im, pm.re);
+        for (int pass = 0; pass < 2; ++pass) {
+          if (side == 0) st = chunk_u(S, r0, r1, S.u, st, pass == 1, true);
+          else if constexpr (CPLX) st = chunk_ud(S, r0, r1, S.w, S.z, st, pass == 1, true);
+          if (pass == 0) st = scan_in(fu, shu[side], st, posu, side);
         }
       }
-      dots[2] = {mq2, 0.f};
-      if (side == 0) warps_to_red(dots, S.red);
+      if (side == 1) side_sync(1);  // its second sweep reads the row before this lane's
     }
+    float mq2 = 0.f;
+    const E gi = side == 1 ? b_i : g_i;
+#pragma unroll 1
+    for (int m = r0; m < r1; ++m) {
+      const E xm = e_load(&X[m]);
+      E dm = e_load(&S.d[m]);
+      if (cj) dm = e_conj(dm);
+      E v = e_addmul(e_load(&U[m]), dm, xm);
+      if (m >= 1) {
+        E f = e_load(&below[m]);
+        if (cj) f = e_conj(f);
+        v = e_addmul(v, f, e_load(&X[m - 1]));
+      }
+      if (m + 1 < k) {
+        E f = e_load(&above[m]);
+        if (cj) f = e_conj(f);
+        v = e_addmul(v, f, e_load(&X[m + 1]));
+      }
+      mq2 += e_abs2hi(v);
+      const E pm = e_submul(v, gi, e_load(&XP[m]));
+      e_store(&U[m], pm);
+      if (side == 0) {
+        df64 d[2] = {dots[0], dots[1]};
+        e_dot(d, CPLX ? e_load(&S.w[m]) : xm, pm);
+        dots[0] = d[0];
+        dots[1] = d[1];
+      }
+    }
+    dots[2] = {mq2, 0.f};
+    if (side == 0) warps_to_red(dots, S.red);
     __syncthreads();
-    const df64 are = red_sum(S.red, 0, 3, 0);
-    const df64 aim = hermitian ? df_zero() : red_sum(S.red, 0, 3, 1);
     const df64 mqn = df_sqrt(red_sum(S.red, 0, 3, 2));
-    const cdf a_i = {are, aim};
+    E a_i;
+    if constexpr (CPLX) a_i = {red_sum(S.red, 0, 3, 0), red_sum(S.red, 0, 3, 1)};
+    else a_i = red_sum(S.red, 0, 3, 0);
     if (tid == 0) T[i * 3 + 0] = e_to2(a_i);
     done = i + 1;
     if (i == l - 1) break;
     // q~ = p - alpha q ; w~ = r - conj(alpha) w ; delta = w~^dag q~ (side 0 its real part,
-    // side 1 the imaginary part)
+    // side 1 the imaginary part) or ||q~||^2
     df64 dl[1] = {df_zero()};
-    const cdf as = cj ? c_conj(a_i) : a_i;
+    const E as = cj ? e_conj(a_i) : a_i;
 #pragma unroll 1
-    for (int m = r0; work && m < r1; ++m) {
-      const cdf v = e_submul(e_load(&U[m]), as, e_load(&X[m]));
+    for (int m = r0; m < r1; ++m) {
+      const E v = e_submul(e_load(&U[m]), as, e_load(&X[m]));
       e_store(&U[m], v);
-      if (hermitian) dl[0] = df_axpy2(dl[0], v.re, v.re, v.im, v.im);
+      if constexpr (!CPLX) dl[0] = df_axpy1(dl[0], v, v);
     }
     __syncthreads();  // both sides' q~, w~; S.red is free again
-    if (!hermitian)
+    if constexpr (CPLX) {
 #pragma unroll 1
       for (int m = r0; m < r1; ++m) {
-        const cdf qt = e_load(&S.u[m]), wt = e_load(&S.z[m]);
+        const E qt = e_load(&S.u[m]), wt = e_load(&S.z[m]);
         const df64 y1 = side == 0 ? qt.re : qt.im, y2 = side == 0 ? qt.im : -qt.re;
         dl[0] = df_axpy2(dl[0], wt.re, y1, wt.im, y2);
       }
+    }
     warps_to_red(dl, S.red);
     __syncthreads();
     df64 bn;
-    cdf gn;
-    if (hermitian) {
-      bn = df_sqrt(red_sum(S.red, 0, 1, 0));
-      gn = {bn, df_zero()};
-    } else {
+    E gn;
+    if constexpr (CPLX) {
       const df64 dre = red_sum(S.red, 0, 1, 0), dim = red_sum(S.red, kSideWarps, 1, 0);
       bn = df_sqrt(df_sqrt(df_axpy2(df_zero(), dre, dre, dim, dim)));
       const df64 rb = bn.hi > 0.f ? df_recip(bn) : df_zero();
       gn = {dre * rb, dim * rb};
+    } else {
+      bn = df_sqrt(red_sum(S.red, 0, 1, 0));
+      gn = bn;
     }
     if (!(bn.hi > exhaust_tol * mqn.hi)) break;  // inner space exhausted: T_i is exact
     if (tid == 0) {
       T[(i + 1) * 3 + 1] = make_double2(df_to_double(bn), 0.0);
       T[(i + 1) * 3 + 2] = e_to2(gn);
     }
-    if (work) {
-      const cdf sc = e_inv(side == 0 ? cdf{bn, df_zero()} : c_conj(gn));
+    const E sc = e_inv(side == 0 ? e_real(bn, zero) : e_conj(gn));
 #pragma unroll 1
-      for (int m = r0; m < r1; ++m) {
-        XP[m] = X[m];
-        e_store(&X[m], e_mul(e_load(&U[m]), sc));
-      }
+    for (int m = r0; m < r1; ++m) {
+      XP[m] = X[m];
+      e_store(&X[m], e_mul(e_load(&U[m]), sc));
     }
-    b_i = bn;
+    b_i = e_real(bn, zero);
     g_i = gn;
     __syncthreads();
   }
@@ -1591,88 +1641,142 @@ __global__ void __launch_bounds__(kColThreads) k_rh_col(int count, int hermitian
 }
 
 // ------------------------------------------------------------ combine
-__global__ void __launch_bounds__(kInnerThreads) k_combine(int count, const int* __restrict__ k_dev,
-                                                           const int* __restrict__ l_dev, InnerWork w, int dl,
-                                                           double2* c, int ldo, void* cacc, const double* nv,
-                                                           int ldn, int prec,
-                                                           double* est_inner, const double2* cprev, int ldp,
-                                                           const int* kprev_dev, double* est_outer, int* rh_status,
-                                                           int* rh_iters, int have_est) {
-  const int* fail = w.fail;
-  __shared__ double red[32];
-  const int prob = blockIdx.x;
+// c = Q_l s and the inner estimate, a cluster of kCombineCtas CTAs a problem (the sums over l
+// are in double, whose pipe gives two multiply-adds a cycle and SM: one CTA a problem took
+// 0.26 ms at k = 333, l = 120, the cluster 0.067). Eight lanes share a row of Q. The difference
+// to the c of the leading l - dl block, c - c' = Q (s - [s'; 0]), only feeds the estimate: in
+// float pairs.
+constexpr int kCombineCtas = 8, kCombineThreads = 128;
+
+__global__ void __cluster_dims__(kCombineCtas, 1, 1) __launch_bounds__(kCombineThreads)
+    k_combine(int count, const int* __restrict__ k_dev, const int* __restrict__ l_dev, InnerWork w, int dl, double2* c,
+              int ldo, void* cacc, const double* nv, int ldn, int prec, double* cnorm, double* est_inner, int* rh_status,
+              int* rh_iters, int have_est) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  __shared__ double2 s_s[kMaxL];
+  __shared__ float4 s_ds[kMaxL];
+  __shared__ double s_red[kCombineThreads / 32][2];
+  __shared__ double s_tot[kCombineCtas][2];
+  const int rank = (int)cluster.block_rank(), prob = blockIdx.x / kCombineCtas, row0 = prob % w.rows;
   const int k = k_dev[prob];
   const int le = w.leff[prob];
   const int le2 = le - dl;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, sub = tid & 7, rl = tid >> 3;
+  const double2* s1 = w.s + (size_t)prob * kMaxL;
+  const double2* s2 = w.s + (size_t)(count + prob) * kMaxL;
+  const bool bad = w.fail[prob] != 0 || le <= 0 || !w.rh_ok[prob];
+  // the inner space is exact when it was exhausted early or spans all of C^k
+  const bool exact = le >= k || le < min(l_dev[prob], k);
+  for (int i = tid; i < le && !bad; i += kCombineThreads) {
+    const double2 v = s1[i];
+    const double2 v2 = have_est && i < le2 ? s2[i] : make_double2(0.0, 0.0);
+    s_s[i] = v;
+    e_store(&s_ds[i], e_from2(make_double2(v.x - v2.x, v.y - v2.y), cdf{}));
+  }
+  __syncthreads();
   // the double-float inner level keeps Q as float pairs in the doubles' bytes
   const double2* Q = w.Q + (size_t)prob * w.ld * kMaxL;
   const bool pairs = w.arith == OV_INNER_DF64;
-  const double2* s1 = w.s + (size_t)prob * kMaxL;
-  const double2* s2 = w.s + (size_t)(count + prob) * kMaxL;
-  const bool bad = fail[prob] != 0 || le <= 0 || !w.rh_ok[prob];
-  // the inner space is exact when it was exhausted early or spans all of C^k
-  const bool exact = le >= k || le < min(l_dev[prob], k);
-  double nc = 0.0, nd = 0.0, no = 0.0;
-  const int kp = kprev_dev ? kprev_dev[prob] : 0;
-  // entries k+1 .. ldo-1 are cleared so that a shorter c never carries stale values
-  for (int m = k + tid; m < ldo - 1; m += blockDim.x) {
-    c[(size_t)prob * ldo + m + 1] = make_double2(0.0, 0.0);
-    if (cacc) {
-      if (prec == OV_PREC_FP64) ((double2*)cacc)[(size_t)prob * ldo + m + 1] = make_double2(0.0, 0.0);
-      else ((float4*)cacc)[(size_t)prob * ldo + m + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-  }
-  for (int m = tid; m < k; m += blockDim.x) {
-    double2 v = make_double2(0.0, 0.0), v2 = make_double2(0.0, 0.0);
-    if (!bad) {
-      for (int i = 0; i < le; ++i) {
-        const double2 qv = pairs ? e_to2(e_load((const float4*)&Q[(size_t)m * kMaxL + i])) : Q[(size_t)m * kMaxL + i];
-        v = zadd(v, zmul(qv, s1[i]));
-        if (have_est && i < le2) v2 = zadd(v2, zmul(qv, s2[i]));
-      }
-    }
+  auto put = [&](int m, double2 v) {
     c[(size_t)prob * ldo + m + 1] = v;
-    if (cacc) {
-      // the recombination sums c_j v_j = (c_j / nv_j) t_j over the unnormalised basis
-      const double sc = nv ? 1.0 / nv[(size_t)prob * ldn + m + 1] : 1.0;
-      const double2 vs = make_double2(v.x * sc, v.y * sc);
-      if (prec == OV_PREC_FP64) {
-        ((double2*)cacc)[(size_t)prob * ldo + m + 1] = vs;
-      } else {
-        const df64 re = df_from_double(vs.x), im = df_from_double(vs.y);
-        ((float4*)cacc)[(size_t)prob * ldo + m + 1] = make_float4(re.hi, re.lo, im.hi, im.lo);
+    if (!cacc) return;
+    // the recombination sums c_j v_j = (c_j / nv_j) t_j over the unnormalised basis
+    const double sc = nv && m < k ? 1.0 / nv[(size_t)row0 * ldn + m + 1] : 1.0;
+    const double2 vs = make_double2(v.x * sc, v.y * sc);
+    if (prec == OV_PREC_FP64) {
+      ((double2*)cacc)[(size_t)prob * ldo + m + 1] = vs;
+    } else {
+      const df64 re = df_from_double(vs.x), im = df_from_double(vs.y);
+      ((float4*)cacc)[(size_t)prob * ldo + m + 1] = make_float4(re.hi, re.lo, im.hi, im.lo);
+    }
+  };
+  double nc = 0.0, nd = 0.0;
+  // entries k+1 .. ldo-1 are cleared so that a shorter c never carries stale values
+  for (int m = k + rank * kCombineThreads + tid; m < ldo - 1; m += kCombineCtas * kCombineThreads)
+    put(m, make_double2(0.0, 0.0));
+  for (int m0 = rank * (kCombineThreads / 8); m0 < k; m0 += kCombineCtas * (kCombineThreads / 8)) {
+    const int m = m0 + rl;
+    double2 v = make_double2(0.0, 0.0);
+    cdf d = {df_zero(), df_zero()};
+    if (!bad && m < k) {
+      for (int i = sub; i < le; i += 8) {
+        const double2* qp = &Q[(size_t)m * kMaxL + i];
+        const cdf qe = pairs ? e_load((const float4*)qp) : e_from2(*qp, cdf{});
+        const double2 qv = pairs ? e_to2(qe) : *qp;
+        v = zadd(v, zmul(qv, s_s[i]));
+        if (have_est) d = e_addmul(d, qe, e_load(&s_ds[i]));
       }
     }
-    nc += zabs2(v);
-    if (le2 >= 1) nd += zabs2(zsub(v, v2));
-    if (kp > 0 && cprev) {
-      const double2 pv = m < kp ? cprev[(size_t)prob * ldp + m + 1] : make_double2(0.0, 0.0);
-      no += zabs2(zsub(v, pv));
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+      v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+      v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+      d.re = d.re + shfl_lane(d.re, (tid & 31) ^ o);
+      d.im = d.im + shfl_lane(d.im, (tid & 31) ^ o);
+    }
+    if (sub == 0 && m < k) {
+      put(m, v);
+      nc += zabs2(v);
+      const double2 dv = e_to2(d);
+      nd += zabs2(dv);
     }
   }
-  nc = block_sum(nc, red);
-  nd = block_sum(nd, red);
-  no = block_sum(no, red);
-  if (tid == 0) {
-    const double cn = sqrt(nc);
+  nc = warp_sum(nc);
+  nd = warp_sum(nd);
+  if ((tid & 31) == 0) { s_red[tid >> 5][0] = nc; s_red[tid >> 5][1] = nd; }
+  __syncthreads();
+  if (tid < 2) {
+    double t = 0.0;
+    for (int q = 0; q < kCombineThreads / 32; ++q) t += s_red[q][tid];
+    *cluster.map_shared_rank(&s_tot[rank][tid], 0) = t;
+  }
+  cluster.sync();
+  if (rank == 0 && tid == 0) {
+    double tc = 0.0, td = 0.0;
+    for (int q = 0; q < kCombineCtas; ++q) { tc += s_tot[q][0]; td += s_tot[q][1]; }
+    const double cn = sqrt(tc);
     // inner estimate: 0 when the inner space is exact (exhausted or l_eff = k)
     double ei;
     if (bad) ei = INFINITY;
     else if (exact) ei = 0.0;
     else if (!have_est) ei = NAN;
     else if (le2 < 1 || w.rh_ok[count + prob] == 0) ei = INFINITY;
-    else ei = sqrt(nd) / cn;
+    else ei = sqrt(td) / cn;
     est_inner[prob] = ei;
-    if (est_outer) est_outer[prob] = (kp > 0 && cprev && !bad) ? sqrt(no) / cn : INFINITY;
-    rh_status[prob] = bad ? (fail[prob] ? 2 : 1) : 0;
+    cnorm[prob] = cn;
+    rh_status[prob] = bad ? (w.fail[prob] ? 2 : 1) : 0;
     rh_iters[prob] = w.rh_its[prob];
   }
+}
+
+// the outer estimate ||c - [c_prev; 0]|| / ||c|| of every problem; c_prev: the same problem's c
+// w.rows places before (the previous check of a group), or row prob of cprev
+__global__ void __launch_bounds__(kCombineThreads) k_estimate(const int* __restrict__ k_dev, InnerWork w, const double2* c,
+                                                              int ldo, const double* cnorm, const int* rh_status,
+                                                              const double2* cprev, int ldp, const int* kprev_dev,
+                                                              double* est_outer) {
+  __shared__ double red[kCombineThreads / 32];
+  const int prob = blockIdx.x;
+  const bool first = prob < w.rows;
+  const int k = k_dev[prob];
+  const int kp = first ? (kprev_dev && cprev ? kprev_dev[prob] : 0) : k_dev[prob - w.rows];
+  const double2* pr = first ? cprev + (size_t)prob * ldp : c + (size_t)(prob - w.rows) * ldo;
+  double no = 0.0;
+  if (kp > 0)
+    for (int m = threadIdx.x; m < k; m += kCombineThreads) {
+      const double2 v = c[(size_t)prob * ldo + m + 1];
+      const double2 pv = m < kp ? pr[m + 1] : make_double2(0.0, 0.0);
+      no += zabs2(zsub(v, pv));
+    }
+  no = block_sum(no, red);
+  if (threadIdx.x == 0) est_outer[prob] = kp > 0 && rh_status[prob] == 0 ? sqrt(no) / cnorm[prob] : INFINITY;
 }
 
 size_t rh_col_scratch_bytes(int count) { return sizeof(float4) * 4 * (size_t)count * kMaxL * kColThreads; }
 
 static size_t inner_smem(int k) { return (size_t)13 * k * sizeof(double2) + 32 * sizeof(double) + k + 16; }
+static size_t inner_smem_real(int k) { return (size_t)13 * k * sizeof(float2) + 32 * sizeof(double) + k + 16; }
 
 cudaError_t run_inner(int count, const int* k_dev, const int* l_dev, int hermitian, const double2* alp,
                       const double2* bet, const double2* gam, const double* nv, int ldc, InnerWork& w,
@@ -1683,10 +1787,15 @@ cudaError_t run_inner(int count, const int* k_dev, const int* l_dev, int hermiti
   cudaError_t e;
   if (phase != 2) {
     const size_t sm = inner_smem(w.ld);  // float pairs take the bytes of the doubles they replace
-    if (w.arith == OV_INNER_DF64) {
-      e = cudaFuncSetAttribute(k_inner_df, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (w.arith == OV_INNER_DF64 && hermitian) {
+      const size_t smr = inner_smem_real(w.ld);
+      e = cudaFuncSetAttribute(k_inner_df<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smr);
       if (e != cudaSuccess) return e;
-      k_inner_df<<<count, 2 * kSideLanes, sm, st>>>(k_dev, l_dev, hermitian, alp, bet, gam, ldc, w);
+      k_inner_df<false><<<count, kSideLanes, smr, st>>>(k_dev, l_dev, alp, bet, gam, ldc, w);
+    } else if (w.arith == OV_INNER_DF64) {
+      e = cudaFuncSetAttribute(k_inner_df<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      if (e != cudaSuccess) return e;
+      k_inner_df<true><<<count, 2 * kSideLanes, sm, st>>>(k_dev, l_dev, alp, bet, gam, ldc, w);
     } else {
       e = cudaFuncSetAttribute(k_inner, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
       if (e != cudaSuccess) return e;
@@ -1725,8 +1834,10 @@ cudaError_t run_inner(int count, const int* k_dev, const int* l_dev, int hermiti
     k_rh<true><<<nmat, 1024, rsm, st>>>(count, 0, nullptr, w, inner_dl, rh_tol, rh_maxit, mid0);
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  k_combine<<<count, kInnerThreads, 0, st>>>(count, k_dev, l_dev, w, inner_dl, c, ldo, cacc, nv, ldc, prec, est_inner,
-                                             cprev, ldp, kprev_dev, est_outer, rh_status, rh_iters, phase != 1);
+  k_combine<<<count * kCombineCtas, kCombineThreads, 0, st>>>(count, k_dev, l_dev, w, inner_dl, c, ldo, cacc, nv, ldc,
+                                                              prec, w.cnorm, est_inner, rh_status, rh_iters, phase != 1);
+  if ((e = cudaGetLastError()) != cudaSuccess || !est_outer) return e;
+  k_estimate<<<count, kCombineThreads, 0, st>>>(k_dev, w, c, ldo, w.cnorm, rh_status, cprev, ldp, kprev_dev, est_outer);
   return cudaGetLastError();
 }
 

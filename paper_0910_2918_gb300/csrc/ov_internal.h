@@ -147,8 +147,11 @@ struct InnerWork {
   int* rh_ok;       // [2*count]
   int* perm;        // [2*count][kMaxL]
   int* fail;        // [count] singular H_k
+  double* cnorm;    // [count] ||c||
   float4* rx;       // rh_col_scratch_bytes(count): the shifted systems of k_rh_col
   int ld;
+  int rows;         // rows of the coefficient arrays: problem i reads row i % rows (several checks of
+                    // the same right-hand sides in one call: problem i is check i / rows)
   int arith;        // OV_INNER_DF64 / OV_INNER_FP64: arithmetic of the serial solves and inversions
   int rh_scale;     // 1: determinant-scaled Roberts-Higham steps in the inner level (DF64 arithmetic)
 };
@@ -158,7 +161,8 @@ struct InnerWork {
 // H_{j-1,j} = gam[j] for j >= 2). Results, index 1..k: c (double2 [count][ldo]) and, if
 // cacc is not NULL, c_j / nv[j] (nv: the normalisations of the unnormalised basis vectors,
 // leading dimension ldc; NULL: 1) in the accumulator type of `prec`; est_inner[i]; est_outer[i]
-// against cprev (rows of length kprev[i], NULL: infinite); rh_status[i] (0 ok, 1 RH not
+// (may be NULL) against cprev (rows of length kprev[i], 0: infinite), for i >= w.rows against c of
+// problem i - w.rows; rh_status[i] (0 ok, 1 RH not
 // converged, 2 singular H); rh_iters[i]. phase 0: everything; phase 1: no inner estimate
 // (est_inner = NaN); phase 2: the inner estimate for the problems of a preceding phase-1
 // call (re-runs only the smaller Roberts-Higham set and the combination).
