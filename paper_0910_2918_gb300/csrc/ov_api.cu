@@ -112,8 +112,11 @@ struct ov_handle {
   Buf partials, counters, scale, scal;
   int cap_rhs = 0, cap_ld = 0;
   // inner level
-  Buf iQ, iT, ileff, iS, is, irh_its, irh_ok, iperm, ifail, irx, icn;
-  Buf ck, cl, ckprev, cc_cur, cc_prev, cc_fin, cacc_cur, cacc_fin, c_est_in, c_est_out, c_rhst, c_rhit;
+  Buf iQ, iT, iS, is, irh_its, irh_ok, iperm, ifail, irx, icn;
+  Buf ck, cl, ckprev, cc_cur, cacc_cur, cacc_fin;
+  Buf chk;  // what a group of checks reports (CheckBuf), with its copy in pinned host memory
+  void* chk_host = nullptr;
+  size_t chk_host_bytes = 0;
   Buf vptr;  // device array of basis slot pointers for recombination
   int inner_cap = 0, inner_ld = 0;
   ov_stats stats{};
@@ -124,7 +127,9 @@ struct ov_handle {
   // stopping checks overlapped with speculative outer steps: a high-priority stream and
   // the events that order it against the handle's stream
   cudaStream_t chk_st = nullptr;
-  cudaEvent_t ev_step = nullptr, ev_chk = nullptr;
+  cudaEvent_t ev_chk = nullptr;
+  std::vector<cudaEvent_t> ev_grid;                           // recorded after the steps of a check
+  cudaEvent_t ev_time[4] = {nullptr, nullptr, nullptr, nullptr};  // around outer steps, around checks
   // captured graphs of U outer steps, one per step precision (strict and relaxed steps)
   struct Graph {
     cudaGraphExec_t exec = nullptr;
@@ -468,9 +473,9 @@ extern "C" void ov_destroy(ov_handle* h) {
   for (Lattice& L : h->lat) release(L.links);
   Buf* all[] = {&h->desc, &h->blkmap, &h->xcanon, &h->ycanon, &h->tv, &h->tw, &h->p, &h->r, &h->vring, &h->wring, &h->yacc,
                 &h->coef_alp, &h->coef_bet, &h->coef_gam, &h->coef_nv, &h->coef_nw, &h->coef_status,
-                &h->coef_kbreak, &h->partials, &h->counters, &h->scale, &h->scal, &h->iQ, &h->iT, &h->ileff, &h->iS, &h->is,
-                &h->irh_its, &h->irh_ok, &h->iperm, &h->ifail, &h->irx, &h->icn, &h->ck, &h->cl, &h->ckprev, &h->cc_cur, &h->cc_prev,
-                &h->cc_fin, &h->cacc_cur, &h->cacc_fin, &h->c_est_in, &h->c_est_out, &h->c_rhst, &h->c_rhit,
+                &h->coef_kbreak, &h->partials, &h->counters, &h->scale, &h->scal, &h->iQ, &h->iT, &h->iS, &h->is,
+                &h->irh_its, &h->irh_ok, &h->iperm, &h->ifail, &h->irx, &h->icn, &h->ck, &h->cl, &h->ckprev, &h->cc_cur,
+                &h->cacc_cur, &h->cacc_fin, &h->chk,
                 &h->vptr, &h->sizer_theta, &h->sizer_feat, &h->sizer_pred, &h->nn_scratch, &h->dx, &h->dy,
                 &h->dpart, &h->dG};
   for (Buf* b : all) release(*b);
@@ -484,8 +489,11 @@ extern "C" void ov_destroy(ov_handle* h) {
     if (gr.exec) cudaGraphExecDestroy(gr.exec);
   if (h->cap_st) cudaStreamDestroy(h->cap_st);
   if (h->chk_st) cudaStreamDestroy(h->chk_st);
-  if (h->ev_step) cudaEventDestroy(h->ev_step);
   if (h->ev_chk) cudaEventDestroy(h->ev_chk);
+  for (cudaEvent_t e : h->ev_grid) cudaEventDestroy(e);
+  for (cudaEvent_t e : h->ev_time)
+    if (e) cudaEventDestroy(e);
+  if (h->chk_host) cudaFreeHost(h->chk_host);
   release(h->jstate);
   release(h->slot_tab);
   delete h;
@@ -520,11 +528,51 @@ static int ensure_outer(ov_handle* h, int nrhs, int ld, size_t pool, int nblocks
   return OV_OK;
 }
 
+// what a group of checks reports, by problem (k, l: what they ran with; status, kbreak: the
+// breakdown state by right-hand side); one block, so that one copy brings it to the host
+struct CheckBuf {
+  double *eo, *ei;
+  int *rhst, *rhit, *leff, *k, *l, *status, *kbreak;
+};
+static size_t check_bytes(int cap) { return (size_t)cap * (2 * sizeof(double) + 7 * sizeof(int)); }
+static CheckBuf check_buf(void* base, int cap) {
+  CheckBuf b;
+  b.eo = (double*)base;
+  b.ei = b.eo + cap;
+  int* i = (int*)(b.ei + cap);
+  b.rhst = i;
+  b.rhit = i + cap;
+  b.leff = i + 2 * (size_t)cap;
+  b.k = i + 3 * (size_t)cap;
+  b.l = i + 4 * (size_t)cap;
+  b.status = i + 5 * (size_t)cap;
+  b.kbreak = i + 6 * (size_t)cap;
+  return b;
+}
+// the breakdown state of right-hand side r as the check at step j sees it: one recorded by a
+// later step is not part of it; one at or before j has both words written before the check
+// began (a pair still being written by a running later step can show the status without its
+// step)
+static int check_status(const CheckBuf& b, int r, int j) {
+  const int s = b.status[r], kb = b.kbreak[r];
+  return (s == kStLucky || s == kStBreakdown) && (kb <= 0 || kb > j) ? kStOK : s;
+}
+// The largest group of checks of a call: one where they cannot be placed beforehand or run
+// otherwise than in the double-float inner level, where the outer steps of an interval take
+// longer than a check anyway (0.3 us a step and 1000 sites on large lattices: 0.75 ms an
+// interval at the line), or where the right-hand sides fill the SMs by themselves.
+static int check_group_cap(const ov_handle* h, int nrhs, size_t pool, const ov_opts& o) {
+  if (!o.nested || o.inner_arith != OV_INNER_DF64 || !o.overlap_checks || o.k_fixed > 0 || h->sizer_on ||
+      o.check_schedule != 0 || o.timing)
+    return 1;
+  if (pool / 12 * (size_t)o.check_interval > 2500000) return 1;
+  return std::max(1, std::min(kMaxGroup, 64 / nrhs));
+}
+
 static int ensure_inner(ov_handle* h, int count, int ld) {
   // ld: leading dimension of the per-problem k-vectors (>= k + 2)
   CK(grow(h->iQ, sizeof(double2) * (size_t)count * ld * kMaxL));
   CK(grow(h->iT, sizeof(double2) * (size_t)count * kMaxL * 3));
-  CK(grow(h->ileff, sizeof(int) * count));
   CK(grow(h->iS, sizeof(double2) * (size_t)2 * count * kMaxL * kMaxL));
   CK(grow(h->is, sizeof(double2) * (size_t)2 * count * kMaxL));
   CK(grow(h->irh_its, sizeof(int) * 2 * count));
@@ -537,16 +585,18 @@ static int ensure_inner(ov_handle* h, int count, int ld) {
   CK(grow(h->ck, sizeof(int) * count));
   CK(grow(h->cl, sizeof(int) * count));
   CK(grow(h->ckprev, sizeof(int) * count));
-  CK(grow(h->cc_cur, cb));
-  CK(grow(h->cc_prev, cb));
-  CK(grow(h->cc_fin, cb));
+  CK(grow(h->cc_cur, 2 * cb));  // the previous check's c before the group's
   const size_t ab = acc_elem_bytes(h->prec) * (size_t)count * ld;
   CK(grow(h->cacc_cur, ab));
   CK(grow(h->cacc_fin, ab));
-  CK(grow(h->c_est_in, sizeof(double) * count));
-  CK(grow(h->c_est_out, sizeof(double) * count));
-  CK(grow(h->c_rhst, sizeof(int) * count));
-  CK(grow(h->c_rhit, sizeof(int) * count));
+  CK(grow(h->chk, check_bytes(count)));
+  if (h->chk_host_bytes < check_bytes(count)) {
+    if (h->chk_host) cudaFreeHost(h->chk_host);
+    h->chk_host = nullptr;
+    h->chk_host_bytes = 0;
+    CK(cudaMallocHost(&h->chk_host, check_bytes(count)));
+    h->chk_host_bytes = check_bytes(count);
+  }
   h->inner_cap = count;
   h->inner_ld = ld;
   return OV_OK;
@@ -558,7 +608,7 @@ static InnerWork inner_work(ov_handle* h, int rows) {
   w.cnorm = (double*)h->icn.p;
   w.Q = (double2*)h->iQ.p;
   w.T = (double2*)h->iT.p;
-  w.leff = (int*)h->ileff.p;
+  w.leff = check_buf(h->chk.p, h->inner_cap).leff;
   w.S = (double2*)h->iS.p;
   w.s = (double2*)h->is.p;
   w.rh_its = (int*)h->irh_its.p;
@@ -686,8 +736,11 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
   if (rc != OV_OK) return rc;
   rc = ensure_outer(h, nrhs, ld, pool, max_blocks(h, lat_of));
   if (rc != OV_OK) return rc;
-  rc = ensure_inner(h, nrhs, ld);
+  const int gcap = check_group_cap(h, nrhs, pool, o);
+  rc = ensure_inner(h, nrhs * gcap, ld);
   if (rc != OV_OK) return rc;
+  for (cudaEvent_t& ev : h->ev_time)
+    if (gcap > 1 && !ev) CK(cudaEventCreate(&ev));
   const size_t canon = sizeof(double2) * pool;
   const double2* xd = (const double2*)x;
   double2* yd = (double2*)y;
@@ -746,10 +799,9 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
   std::vector<int> done(nrhs, 0), kfin(nrhs, 0), lfin(nrhs, 0), itfin(nrhs, 0), stat(nrhs, OV_OK);
   std::vector<int> kprev(nrhs, 0), kcur(nrhs, 0), lreq(nrhs, std::min(l, kMaxL));
   std::vector<double> estfin(nrhs, INFINITY), estin(nrhs, NAN);
-  std::vector<int> dstatus(nrhs), dkbreak(nrhs), rhst(nrhs), rhit(nrhs), leff(nrhs);
+  std::vector<int> dstatus(nrhs), rhst(nrhs), rhit(nrhs), leff(nrhs);
   std::vector<double> eo(nrhs), ei(nrhs);
   CK(cudaMemcpyAsync(h->cl.p, lreq.data(), sizeof(int) * nrhs, cudaMemcpyHostToDevice, st));
-  CK(cudaMemsetAsync(h->cc_fin.p, 0, sizeof(double2) * (size_t)nrhs * ld, st));
   CK(cudaMemsetAsync(h->cacc_fin.p, 0, acc_elem_bytes(h->prec) * (size_t)nrhs * ld, st));
   InnerWork iw = inner_work(h, nrhs);
   int ndone = 0;
@@ -895,23 +947,78 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
     return OV_OK;
   };
   // j: the step the loop has reached (the last check's, or the end of the last span);
-  // jdone >= j: steps run so far, speculative steps run during a check included. The loop
-  // ends when every right-hand side is done or the step at ktarget has been checked, also
-  // where speculative steps already reached ktarget (then no step is run, only the check).
+  // jdone >= j: steps run so far, speculative steps included. The loop ends when every
+  // right-hand side is done or the step at ktarget has been checked, also where speculative
+  // steps already reached ktarget (then no step is run, only the check).
+  //
+  // Checks are evaluated in groups. Where an interval of outer steps takes less time than a
+  // check (small lattices: a step of one 8^4 source takes 27 us, a check ~1.5 ms on one SM), the
+  // steps of several intervals run first and their checks go to the inner level together, on
+  // SMs that a single check leaves idle; their results are judged in the order of the serial
+  // run, which they equal, and what lies behind the one that stops it is dropped. The group
+  // size follows from the measured times of the steps and of the last group, so that steps
+  // and checks, overlapped, take about as long; it only moves time, never the result.
+  const bool fixed = o.k_fixed > 0;
+  const bool overlap = o.overlap_checks && !fixed;
+  int G = 1;              // the group's size
+  double step_ms = -1.0;  // of one outer step, as last measured
+  int span_steps = 0;     // steps between ev_time[0] and ev_time[1], 0: not recorded
+  // steps jdone+1 .. jt; at each check of the grid from next_grid on, an event for its check
+  // to wait for (a check waits for its own steps only, not for the speculative ones behind)
+  std::vector<std::pair<int, cudaEvent_t>> grid_ev;
+  size_t grid_used = 0;
+  auto steps_to = [&](int jt, int grid0) -> int {
+    const bool timed = gcap > 1 && jt - jdone >= 4 && span_steps == 0;
+    if (timed) CK(cudaEventRecord(h->ev_time[0], st));
+    const int from = jdone;
+    while (jdone < jt) {
+      int je = jt;
+      if (grid0 > 0) {
+        const int next = jdone < grid0 ? grid0 : grid0 + ((jdone - grid0) / o.check_interval + 1) * o.check_interval;
+        je = std::min(jt, next);
+      }
+      const int e = run_span(jdone, je);
+      if (e != OV_OK) return e;
+      jdone = je;
+      if (overlap && (jdone == jt || grid0 > 0)) {
+        if (grid_used == h->ev_grid.size()) {
+          cudaEvent_t ev;
+          CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+          h->ev_grid.push_back(ev);
+        }
+        cudaEvent_t ev = h->ev_grid[grid_used++];
+        CK(cudaEventRecord(ev, st));
+        grid_ev.push_back({jdone, ev});
+      }
+    }
+    if (timed) {
+      CK(cudaEventRecord(h->ev_time[1], st));
+      span_steps = jdone - from;
+    }
+    return OV_OK;
+  };
+  // whether steps to jt need no basis memory beyond what is allocated (stored mode; up to
+  // kSpecSteps ahead of the first unjudged check a chunk may be added)
+  auto room = [&](int jt) {
+    return recomb != OV_RECOMB_STORED || jt - j <= kSpecSteps || jt < (int)h->chunks.size() * kChunk;
+  };
   for (;;) {
     if (j >= ktarget || ndone >= nrhs) break;
-    const bool fixed_span = o.k_fixed > 0;
-    int target = fixed_span ? ktarget : std::min(next_check, ktarget);
-    if (h->sizer_on && !fixed_span && j < kSizerSteps && ktarget > kSizerSteps + 1)
+    int target = fixed ? ktarget : std::min(next_check, ktarget);
+    if (h->sizer_on && !fixed && j < kSizerSteps && ktarget > kSizerSteps + 1)
       target = std::min(target, kSizerSteps);
     if (target <= j) target = j + 1;
-    if (target > jdone) {
-      rc = run_span(jdone, target);
+    // the checks of this group (the adaptive schedule and the learned sizing place or repeat
+    // checks by the results of the one before: one at a time)
+    std::vector<int> js(1, target);
+    while ((int)js.size() < std::min(G, gcap) && target == std::min(next_check, ktarget) && js.back() < ktarget &&
+           room(std::min(js.back() + o.check_interval, ktarget)))
+      js.push_back(std::min(js.back() + o.check_interval, ktarget));
+    if (js.back() > jdone) {
+      rc = steps_to(js.back(), gcap > 1 ? target : 0);
       if (rc != OV_OK) return rc;
-      jdone = target;
     }
     j = target;
-    const bool fixed = o.k_fixed > 0;
     if (h->sizer_on && !fixed && j == kSizerSteps && ktarget > kSizerSteps + 1) {
       // learned sizing: f = (Re alpha_1..6, Im alpha_1..6, beta_2..5) -> (log k*, log l*)
       std::vector<double2> fa((size_t)nrhs * 6), fb((size_t)nrhs * 4);
@@ -962,115 +1069,149 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
     }
     const bool check = fixed ? (j == ktarget) : (j >= next_check || j == ktarget);
     if (!check) continue;
-    // the check runs on the check stream while speculative outer steps (at most
-    // kSpecSteps, never past the next check) run on the handle's stream; they only add
-    // coefficients and basis vectors beyond k = j, so the check and the result are those of
-    // the serial order, and the steps count towards the next interval if the run goes on
-    cudaStream_t cs = st;
-    int spec = 0;
-    // (not before the learned sizing has read its 16 steps: it runs where a span ends there;
-    // and not where the run is likely to stop: the previous check's largest outer estimate
-    // within kSpecFactor of tol. The choice only moves time, never the result)
+    const int g = (int)js.size(), n = nrhs * g, jlast = js.back();
+    // the checks run on the check stream while speculative outer steps run on the handle's
+    // stream: at most kSpecSteps and never past the next check, or the steps of the next
+    // group. They only add coefficients and basis vectors beyond k = jlast, so the checks and
+    // the result are those of the serial order, and the steps count towards the next checks if
+    // the run goes on. (Not before the learned sizing has read its 16 steps: it runs where a
+    // span ends there; and not where the run is likely to stop: the previous check's largest
+    // outer estimate within kSpecFactor of tol. The choice only moves time, never the result)
     const bool likely_stop = eo_last_max >= 0.0 && eo_last_max <= kSpecFactor * tol;
-    if (o.overlap_checks && !fixed && j < ktarget && !(h->sizer_on && j < kSizerSteps) && !likely_stop) {
-      spec = std::min(std::min(kSpecSteps, o.check_interval - 1), ktarget - j);
-      if (spec > 0) {
-        if (!h->chk_st) {
-          int lo = 0, hi = 0;
-          CK(cudaDeviceGetStreamPriorityRange(&lo, &hi));
-          CK(cudaStreamCreateWithPriority(&h->chk_st, cudaStreamNonBlocking, hi));
-          CK(cudaEventCreateWithFlags(&h->ev_step, cudaEventDisableTiming));
-          CK(cudaEventCreateWithFlags(&h->ev_chk, cudaEventDisableTiming));
-        }
-        CK(cudaEventRecord(h->ev_step, st));
-        rc = run_span(j, j + spec);
-        if (rc != OV_OK) return rc;
-        CK(cudaStreamWaitEvent(h->chk_st, h->ev_step, 0));
-        cs = h->chk_st;
-      }
+    int spec = 0;
+    if (overlap && jlast < ktarget && !(h->sizer_on && j < kSizerSteps) && !likely_stop) {
+      spec = std::min(std::min(kSpecSteps, o.check_interval - 1), ktarget - jlast);
+      int ahead = 0;
+      while (g > 1 && ahead < g && jlast + (ahead + 1) * o.check_interval <= ktarget &&
+             room(jlast + (ahead + 1) * o.check_interval))
+        ++ahead;
+      if (ahead > 0) spec = ahead * o.check_interval;
     }
-    // read the breakdown state first: a Lanczos breakdown fixes k for that RHS
-    CK(cudaMemcpyAsync(dstatus.data(), c.status, sizeof(int) * nrhs, cudaMemcpyDeviceToHost, cs));
-    CK(cudaMemcpyAsync(dkbreak.data(), c.kbreak, sizeof(int) * nrhs, cudaMemcpyDeviceToHost, cs));
-    CK(cudaStreamSynchronize(cs));
-    // a breakdown recorded by a speculative step (after j) is not part of this check; one at
-    // or before j has both words written before the check began (a pair still being written
-    // by a running speculative step can show the status without its step)
-    for (int r = 0; r < nrhs; ++r)
-      if ((dstatus[r] == kStLucky || dstatus[r] == kStBreakdown) && (dkbreak[r] <= 0 || dkbreak[r] > j))
-        dstatus[r] = kStOK;
-    for (int r = 0; r < nrhs; ++r) kcur[r] = (dstatus[r] != kStOK && dkbreak[r] > 0) ? std::min(dkbreak[r], j) : j;
-    CK(cudaMemcpyAsync(h->ck.p, kcur.data(), sizeof(int) * nrhs, cudaMemcpyHostToDevice, cs));
+    cudaStream_t cs = st;
+    if (spec > 0 || (overlap && jdone > jlast)) {
+      if (!h->chk_st) {
+        int lo = 0, hi = 0;
+        CK(cudaDeviceGetStreamPriorityRange(&lo, &hi));
+        CK(cudaStreamCreateWithPriority(&h->chk_st, cudaStreamNonBlocking, hi));
+        CK(cudaEventCreateWithFlags(&h->ev_chk, cudaEventDisableTiming));
+      }
+      cs = h->chk_st;
+      for (const auto& ge : grid_ev)
+        if (ge.first == jlast) CK(cudaStreamWaitEvent(cs, ge.second, 0));
+    }
     CK(cudaMemcpyAsync(h->ckprev.p, kprev.data(), sizeof(int) * nrhs, cudaMemcpyHostToDevice, cs));
+    // the breakdown state as the checks see it: a Lanczos breakdown fixes k for that RHS
+    CheckSteps cj{};
+    for (int i = 0; i < g; ++i) cj.j[i] = js[i];
+    double2* const cc0 = (double2*)h->cc_cur.p;             // the previous check's c
+    double2* const cc1 = cc0 + (size_t)nrhs * ld;           // the group's, one slot a check
+    const size_t ab = acc_elem_bytes(h->prec);
     const Phase ph_check("stopping check");
-    bool regrow = false;
+    bool regrow = false, spec_run = false;
     do {
     regrow = false;
     const auto tc0 = std::chrono::steady_clock::now();
+    if (gcap > 1) CK(cudaEventRecord(h->ev_time[2], cs));
+    const CheckBuf db = check_buf(h->chk.p, h->inner_cap);
+    const CheckBuf hb = check_buf(h->chk_host, h->inner_cap);
+    CK(launch_check_setup(nrhs, n, cj, c.status, c.kbreak, (const int*)h->cl.p, db.k, db.l, db.status, db.kbreak, cs));
     const int ti = tstart(h, kClsInner, cs);
-    // where a stop is likely, both Roberts-Higham sets (the inner estimate's too) in one
-    // launch instead of a second round trip
-    // (the non-nested check has no inner estimate to defer)
-    const int phase = (!o.nested || (likely_stop && !fixed)) ? 0 : 1;
+    // the double-float inner level takes both Roberts-Higham sets at once (they run side by
+    // side); in FP64 the inner estimate's set runs where it is wanted, or where a stop is
+    // likely (the non-nested check has no inner estimate to defer)
+    const int phase = !o.nested || (!fixed && (likely_stop || o.inner_arith == OV_INNER_DF64)) ? 0 : 1;
     cudaError_t e;
     if (!o.nested) {
+      CK(cudaMemcpyAsync(kcur.data(), db.k, sizeof(int) * nrhs, cudaMemcpyDeviceToHost, cs));
+      CK(cudaStreamSynchronize(cs));
       CK(grow(h->nn_scratch, nonnested_scratch_bytes(nrhs, *std::max_element(kcur.begin(), kcur.end()))));
-      e = run_nonnested(nrhs, kcur.data(), c.alp, c.bet, c.gam, c.nv, ld, o.rh_tol, o.rh_maxit, (double2*)h->cc_cur.p,
-                        ld, h->cacc_cur.p, h->prec, (double*)h->c_est_in.p, (const double2*)h->cc_prev.p, ld,
-                        (const int*)h->ckprev.p, (double*)h->c_est_out.p, (int*)h->c_rhst.p, (int*)h->c_rhit.p,
-                        h->nn_scratch.p, cs);
-    } else
-    e = run_inner(nrhs, (const int*)h->ck.p, (const int*)h->cl.p, herm ? 1 : 0, c.alp, c.bet, c.gam, c.nv, ld, iw,
-                              o.rh_tol, o.rh_maxit, o.inner_dl, (double2*)h->cc_cur.p, ld, h->cacc_cur.p, h->prec,
-                              (double*)h->c_est_in.p, (const double2*)h->cc_prev.p, ld, (const int*)h->ckprev.p,
-                              (double*)h->c_est_out.p, (int*)h->c_rhst.p, (int*)h->c_rhit.p, phase, cs);
+      e = run_nonnested(nrhs, kcur.data(), c.alp, c.bet, c.gam, c.nv, ld, o.rh_tol, o.rh_maxit, cc1, ld, h->cacc_cur.p,
+                        h->prec, db.ei, cc0, ld, (const int*)h->ckprev.p, db.eo, db.rhst, db.rhit, h->nn_scratch.p, cs);
+    } else {
+      e = run_inner(n, db.k, db.l, herm ? 1 : 0, c.alp, c.bet, c.gam, c.nv, ld, iw, o.rh_tol, o.rh_maxit, o.inner_dl, cc1,
+                    ld, h->cacc_cur.p, h->prec, db.ei, cc0, ld, (const int*)h->ckprev.p, db.eo, db.rhst, db.rhit, phase,
+                    cs);
+    }
     CK(e);
     tstop(h, ti);
-    // k_inner, k_rh, k_combine, k_estimate; the double-float inner level has two Roberts-Higham kernels
+    // the check's step kernel, k_inner, k_rh, k_combine, k_estimate; the double-float inner level
+    // has two Roberts-Higham kernels
     const int rh_kernels = o.nested && o.inner_arith == OV_INNER_DF64 ? 2 : 1;
-    h->stats.launches += 3 + rh_kernels;
-    h->stats.inner_launches += 3 + rh_kernels;
-    h->stats.checks += 1;
-    CK(cudaMemcpyAsync(eo.data(), h->c_est_out.p, sizeof(double) * nrhs, cudaMemcpyDeviceToHost, cs));
-    CK(cudaMemcpyAsync(rhst.data(), h->c_rhst.p, sizeof(int) * nrhs, cudaMemcpyDeviceToHost, cs));
-    CK(cudaMemcpyAsync(rhit.data(), h->c_rhit.p, sizeof(int) * nrhs, cudaMemcpyDeviceToHost, cs));
-    CK(cudaMemcpyAsync(leff.data(), h->ileff.p, sizeof(int) * nrhs, cudaMemcpyDeviceToHost, cs));
+    h->stats.launches += 4 + rh_kernels;
+    h->stats.inner_launches += 4 + rh_kernels;
+    h->stats.checks += g;
+    // one copy brings back what the judgement reads
+    CK(cudaMemcpyAsync(h->chk_host, h->chk.p, check_bytes(h->inner_cap), cudaMemcpyDeviceToHost, cs));
+    if (gcap > 1) CK(cudaEventRecord(h->ev_time[3], cs));
+    if (spec > 0 && !spec_run) {
+      spec_run = true;
+      if (jlast + spec > jdone) {
+        rc = steps_to(jlast + spec, g > 1 ? jlast + o.check_interval : 0);
+        if (rc != OV_OK) return rc;
+      }
+    }
     CK(cudaStreamSynchronize(cs));
     // the inner estimate is needed only where the run may stop at this check
-    bool want_inner = false;
-    for (int r = 0; r < nrhs && !fixed; ++r)
-      if (!done[r] && dstatus[r] != kStZero && dstatus[r] != kStBreakdown && rhst[r] == 0 &&
-          (eo[r] <= tol || dstatus[r] == kStLucky || j == ktarget))
-        want_inner = true;
-    std::fill(ei.begin(), ei.end(), NAN);
-    if (want_inner && phase == 0) {
-      CK(cudaMemcpyAsync(ei.data(), h->c_est_in.p, sizeof(double) * nrhs, cudaMemcpyDeviceToHost, cs));
-      CK(cudaStreamSynchronize(cs));
-    } else if (want_inner) {
-      const int t2 = tstart(h, kClsInner, cs);
-      e = run_inner(nrhs, (const int*)h->ck.p, (const int*)h->cl.p, herm ? 1 : 0, c.alp, c.bet, c.gam, c.nv, ld, iw, o.rh_tol,
-                    o.rh_maxit, o.inner_dl, (double2*)h->cc_cur.p, ld, h->cacc_cur.p, h->prec,
-                    (double*)h->c_est_in.p, (const double2*)h->cc_prev.p, ld, (const int*)h->ckprev.p,
-                    (double*)h->c_est_out.p, (int*)h->c_rhst.p, (int*)h->c_rhit.p, 2, cs);
-      CK(e);
-      tstop(h, t2);
-      h->stats.launches += 2 + rh_kernels;
-      h->stats.inner_launches += 2 + rh_kernels;
-      CK(cudaMemcpyAsync(ei.data(), h->c_est_in.p, sizeof(double) * nrhs, cudaMemcpyDeviceToHost, cs));
-      CK(cudaMemcpyAsync(rhst.data(), h->c_rhst.p, sizeof(int) * nrhs, cudaMemcpyDeviceToHost, cs));
-      CK(cudaStreamSynchronize(cs));
+    bool have_ei = phase == 0 && !fixed;
+    if (!have_ei && !fixed) {
+      bool want_inner = false;
+      for (int r = 0; r < nrhs; ++r)
+        if (!done[r] && hb.status[r] != kStZero && check_status(hb, r, j) != kStBreakdown && hb.rhst[r] == 0 &&
+            (hb.eo[r] <= tol || check_status(hb, r, j) == kStLucky || j == ktarget))
+          want_inner = true;
+      if (want_inner) {
+        const int t2 = tstart(h, kClsInner, cs);
+        e = run_inner(n, db.k, db.l, herm ? 1 : 0, c.alp, c.bet, c.gam, c.nv, ld, iw, o.rh_tol, o.rh_maxit, o.inner_dl,
+                      cc1, ld, h->cacc_cur.p, h->prec, db.ei, cc0, ld, (const int*)h->ckprev.p, db.eo, db.rhst, db.rhit,
+                      2, cs);
+        CK(e);
+        tstop(h, t2);
+        h->stats.launches += 2 + rh_kernels;
+        h->stats.inner_launches += 2 + rh_kernels;
+        CK(cudaMemcpyAsync(h->chk_host, h->chk.p, check_bytes(h->inner_cap), cudaMemcpyDeviceToHost, cs));
+        CK(cudaStreamSynchronize(cs));
+        have_ei = true;
+      }
+    }
+    if (gcap > 1) {
+      // times for the next group's size
+      float ms = 0.f;
+      if (span_steps > 0 && cudaEventQuery(h->ev_time[1]) == cudaSuccess) {
+        CK(cudaEventElapsedTime(&ms, h->ev_time[0], h->ev_time[1]));
+        step_ms = ms / span_steps;
+        span_steps = 0;
+      }
+      CK(cudaEventElapsedTime(&ms, h->ev_time[2], h->ev_time[3]));
+      if (step_ms > 0.0)
+        G = std::max(1, std::min(gcap, (int)std::lround(ms / (step_ms * o.check_interval))));
+      cudaGetLastError();  // (a query that was not ready)
     }
     if (h->trace) {
       const double ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - tc0).count();
-      fprintf(stderr, "{\"ov_check\": %d, \"ms\": %.3f, \"speculative_steps\": %d, \"inner_estimate\": %d, \"rh_iters\": [",
-              j, ms, spec, want_inner ? 1 : 0);
-      for (int r = 0; r < nrhs; ++r) fprintf(stderr, "%s%d", r ? "," : "", rhit[r]);
-      fprintf(stderr, "], \"est_outer\": [");
-      for (int r = 0; r < nrhs; ++r) fprintf(stderr, "%s%.3e", r ? "," : "", eo[r]);
-      fprintf(stderr, "], \"l_eff\": [");
-      for (int r = 0; r < nrhs; ++r) fprintf(stderr, "%s%d", r ? "," : "", leff[r]);
-      fprintf(stderr, "]}\n");
+      for (int i = 0; i < g; ++i) {
+        fprintf(stderr, "{\"ov_check\": %d, \"ms\": %.3f, \"group\": %d, \"speculative_steps\": %d, \"inner_estimate\": %d, "
+                        "\"rh_iters\": [", js[i], ms, g, spec, have_ei ? 1 : 0);
+        for (int r = 0; r < nrhs; ++r) fprintf(stderr, "%s%d", r ? "," : "", hb.rhit[i * nrhs + r]);
+        fprintf(stderr, "], \"est_outer\": [");
+        for (int r = 0; r < nrhs; ++r) fprintf(stderr, "%s%.3e", r ? "," : "", hb.eo[i * nrhs + r]);
+        fprintf(stderr, "], \"l_eff\": [");
+        for (int r = 0; r < nrhs; ++r) fprintf(stderr, "%s%d", r ? "," : "", hb.leff[i * nrhs + r]);
+        fprintf(stderr, "]}\n");
+      }
     }
+    // judge the group's checks in order
+    for (int i = 0; i < g && ndone < nrhs; ++i) {
+      j = js[i];
+      for (int r = 0; r < nrhs; ++r) {
+        const int p = i * nrhs + r;
+        kcur[r] = hb.k[p];
+        eo[r] = hb.eo[p];
+        ei[r] = have_ei ? hb.ei[p] : NAN;
+        rhst[r] = hb.rhst[p];
+        rhit[r] = hb.rhit[p];
+        leff[r] = hb.leff[p];
+        dstatus[r] = check_status(hb, r, j);
+      }
     kprev_old = kprev;
     for (int r = 0; r < nrhs; ++r) {
       if (done[r]) continue;
@@ -1120,11 +1261,9 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
         estfin[r] = est;
         estin[r] = ei[r];
         stat[r] = sr;
-        CK(cudaMemcpyAsync((double2*)h->cc_fin.p + (size_t)r * ld, (double2*)h->cc_cur.p + (size_t)r * ld,
-                           sizeof(double2) * ld, cudaMemcpyDeviceToDevice, cs));
-        const size_t ab = acc_elem_bytes(h->prec);
-        CK(cudaMemcpyAsync((char*)h->cacc_fin.p + ab * (size_t)r * ld, (char*)h->cacc_cur.p + ab * (size_t)r * ld,
-                           ab * ld, cudaMemcpyDeviceToDevice, cs));
+        const size_t p = (size_t)i * nrhs + r;
+        CK(cudaMemcpyAsync((char*)h->cacc_fin.p + ab * (size_t)r * ld, (char*)h->cacc_cur.p + ab * p * ld, ab * ld,
+                           cudaMemcpyDeviceToDevice, cs));
       } else {
         kprev[r] = kcur[r];
         // est_outer compares with the previous check, so it measures the error there;
@@ -1141,18 +1280,29 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
         }
       }
     }
+    // (a group of one where l may grow)
+    if (!regrow) {
+      eo_last_max = 0.0;  // an estimate without a previous check (infinite) means unknown
+      for (int r = 0; r < nrhs; ++r)
+        if (!done[r]) eo_last_max = std::max(eo_last_max, std::isnan(eo[r]) ? INFINITY : eo[r]);
+    }
+    }
     if (regrow) CK(cudaMemcpyAsync(h->cl.p, lreq.data(), sizeof(int) * nrhs, cudaMemcpyHostToDevice, cs));
     } while (regrow);
-    eo_last_max = 0.0;  // an estimate without a previous check (infinite) means unknown
-    for (int r = 0; r < nrhs; ++r)
-      if (!done[r]) eo_last_max = std::max(eo_last_max, std::isnan(eo[r]) ? INFINITY : eo[r]);
+    // the group's last c is the next check's previous one
+    if (ndone < nrhs)
+      CK(cudaMemcpyAsync(cc0, cc1 + (size_t)(g - 1) * nrhs * ld, sizeof(double2) * (size_t)nrhs * ld,
+                         cudaMemcpyDeviceToDevice, cs));
     if (cs != st) {
-      // later work on the handle's stream (the final combination) reads the check's results
+      // later work on the handle's stream (a check, the final combination) reads the results
       CK(cudaEventRecord(h->ev_chk, cs));
       CK(cudaStreamWaitEvent(st, h->ev_chk, 0));
-      jdone = j + spec;
     }
-    std::swap(h->cc_cur, h->cc_prev);
+    // events of checks judged are free again
+    if (jdone <= j) {
+      grid_ev.clear();
+      grid_used = 0;
+    }
     // next check: fixed interval, or (adaptive) a jump to where the log-linear decay of
     // the error reaches tol, always followed by a partner check check_interval later
     // (the estimate at a check measures the error at the check before it)
@@ -1787,20 +1937,17 @@ extern "C" int ov_inner_sign(ov_handle* h, int count, int ld, const int* k, cons
   cudaMemcpyAsync(dA.p, A.data(), cb, cudaMemcpyHostToDevice, st);
   cudaMemcpyAsync(dB.p, B.data(), cb, cudaMemcpyHostToDevice, st);
   cudaMemcpyAsync(dG.p, G.data(), cb, cudaMemcpyHostToDevice, st);
-  cudaMemcpyAsync(h->ck.p, k, sizeof(int) * count, cudaMemcpyHostToDevice, st);
-  cudaMemcpyAsync(h->cl.p, lv.data(), sizeof(int) * count, cudaMemcpyHostToDevice, st);
+  const CheckBuf db = check_buf(h->chk.p, h->inner_cap), hb = check_buf(h->chk_host, h->inner_cap);
+  cudaMemcpyAsync(db.k, k, sizeof(int) * count, cudaMemcpyHostToDevice, st);
+  cudaMemcpyAsync(db.l, lv.data(), sizeof(int) * count, cudaMemcpyHostToDevice, st);
   InnerWork iw = inner_work(h, count);
-  cudaError_t e = run_inner(count, (const int*)h->ck.p, (const int*)h->cl.p, hermitian ? 1 : 0, (double2*)dA.p,
-                            (double2*)dB.p, (double2*)dG.p, nullptr, ldi, iw, h->o.rh_tol, h->o.rh_maxit, h->o.inner_dl,
-                            (double2*)h->cc_cur.p, ldi, nullptr, h->prec, (double*)h->c_est_in.p, nullptr, ldi,
-                            nullptr, nullptr, (int*)h->c_rhst.p, (int*)h->c_rhit.p, 0, st);
+  cudaError_t e = run_inner(count, db.k, db.l, hermitian ? 1 : 0, (double2*)dA.p, (double2*)dB.p, (double2*)dG.p, nullptr,
+                            ldi, iw, h->o.rh_tol, h->o.rh_maxit, h->o.inner_dl, (double2*)h->cc_cur.p, ldi, nullptr,
+                            h->prec, db.ei, nullptr, ldi, nullptr, nullptr, db.rhst, db.rhit, 0, st);
   std::vector<double2> C((size_t)count * ldi);
-  std::vector<double> ein(count);
-  std::vector<int> rs(count), ri(count);
   if (e == cudaSuccess) e = cudaMemcpyAsync(C.data(), h->cc_cur.p, cb, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(ein.data(), h->c_est_in.p, sizeof(double) * count, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(rs.data(), h->c_rhst.p, sizeof(int) * count, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(ri.data(), h->c_rhit.p, sizeof(int) * count, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(h->chk_host, h->chk.p, check_bytes(h->inner_cap), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   cleanup();
   if (e != cudaSuccess) {
@@ -1811,9 +1958,9 @@ extern "C" int ov_inner_sign(ov_handle* h, int count, int ld, const int* k, cons
   int worst = OV_OK;
   for (int i = 0; i < count; ++i) {
     for (int jj = 0; jj < ld; ++jj) co[(size_t)i * ld + jj] = jj < k[i] ? C[(size_t)i * ldi + jj + 1] : double2{0, 0};
-    if (est_inner) est_inner[i] = ein[i];
-    if (rh_iters) rh_iters[i] = ri[i];
-    if (rs[i] != 0) worst = OV_ERR_RH_NOCONV;
+    if (est_inner) est_inner[i] = hb.ei[i];
+    if (rh_iters) rh_iters[i] = hb.rhit[i];
+    if (hb.rhst[i] != 0) worst = OV_ERR_RH_NOCONV;
   }
   return worst;
 }

@@ -1773,6 +1773,26 @@ __global__ void __launch_bounds__(kCombineThreads) k_estimate(const int* __restr
   if (threadIdx.x == 0) est_outer[prob] = kp > 0 && rh_status[prob] == 0 ? sqrt(no) / cnorm[prob] : INFINITY;
 }
 
+__global__ void k_check_setup(int rows, int n, CheckSteps cj, const int* __restrict__ status,
+                              const int* __restrict__ kbreak, const int* __restrict__ l_in, int* k_out, int* l_out,
+                              int* status_out, int* kbreak_out) {
+  for (int r = threadIdx.x; r < rows; r += blockDim.x) {
+    const int s = status[r], kb = kbreak[r];
+    status_out[r] = s;
+    kbreak_out[r] = kb;
+    for (int p = r; p < n; p += rows) {
+      const int j = cj.j[p / rows];
+      k_out[p] = s != kStOK && kb > 0 ? min(kb, j) : j;
+      l_out[p] = l_in[r];
+    }
+  }
+}
+cudaError_t launch_check_setup(int rows, int n, const CheckSteps& cj, const int* status, const int* kbreak, const int* l_in,
+                               int* k_out, int* l_out, int* status_out, int* kbreak_out, cudaStream_t st) {
+  k_check_setup<<<1, 128, 0, st>>>(rows, n, cj, status, kbreak, l_in, k_out, l_out, status_out, kbreak_out);
+  return cudaGetLastError();
+}
+
 size_t rh_col_scratch_bytes(int count) { return sizeof(float4) * 4 * (size_t)count * kMaxL * kColThreads; }
 
 static size_t inner_smem(int k) { return (size_t)13 * k * sizeof(double2) + 32 * sizeof(double) + k + 16; }

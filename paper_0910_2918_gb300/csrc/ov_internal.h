@@ -155,6 +155,17 @@ struct InnerWork {
   int arith;        // OV_INNER_DF64 / OV_INNER_FP64: arithmetic of the serial solves and inversions
   int rh_scale;     // 1: determinant-scaled Roberts-Higham steps in the inner level (DF64 arithmetic)
 };
+// A group of stopping checks of the same right-hand sides at outer steps j[0], j[1], ...
+constexpr int kMaxGroup = 8;
+struct CheckSteps {
+  int j[kMaxGroup];
+};
+// the problems of a group (i = check i / rows of right-hand side i % rows): k_out[i] = the check's
+// step, or the step of a breakdown at or before it; l_out[i] = l_in[i % rows]; and the breakdown
+// state of the right-hand sides as it is now
+cudaError_t launch_check_setup(int rows, int n, const CheckSteps& cj, const int* status, const int* kbreak, const int* l_in,
+                               int* k_out, int* l_out, int* status_out, int* kbreak_out, cudaStream_t st);
+
 // Inner level for `count` problems whose tridiagonal coefficients live in device
 // arrays alp/bet/gam with leading dimension ldc (index j = 1..k as in Coefs, so the
 // diagonal is alp[j], the subdiagonal H_{j,j-1} = bet[j] and the superdiagonal
