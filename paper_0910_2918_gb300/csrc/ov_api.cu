@@ -78,10 +78,14 @@ void release(Buf& b) {
 }  // namespace
 
 struct TuneKey {
-  int prec, mode, nprob, pad;
+  int prec, mode, nprob;
   bool operator<(const TuneKey& o) const {
     return prec != o.prec ? prec < o.prec : (mode != o.mode ? mode < o.mode : nprob < o.nprob);
   }
+};
+// threads per site block, and sites per block of the wide kernels (0: not used)
+struct Tuned {
+  int bs, wide;
 };
 
 // one gauge field with its operator parameters
@@ -120,7 +124,7 @@ struct ov_handle {
   Buf vptr;  // device array of basis slot pointers for recombination
   int inner_cap = 0, inner_ld = 0;
   ov_stats stats{};
-  std::map<TuneKey, int> tuned;  // autotuned block size per (precision, mode, problem count)
+  std::map<TuneKey, Tuned> tuned;  // autotuned kernels per (precision or relaxed, mode, problem count)
   // CUDA graph of graph_steps outer steps (captured on a private stream, replayed on st)
   Buf jstate, slot_tab;
   cudaStream_t cap_st = nullptr;
@@ -296,16 +300,23 @@ static int build_batch(ov_handle* h, const std::vector<int>& lat_of, int bs, Bat
   b->nblocks = blk;
   b->nprob = np;
   b->block = bs;
+  b->wide = 0;
   *pool = voff;
   return OV_OK;
 }
 
-// site blocks of a call at the smallest block size (sizes the partial-sum buffer)
+// site blocks of a call at the smallest block size, 16 sites of the wide kernels (sizes the
+// partial-sum buffer)
 static int max_blocks(const ov_handle* h, const std::vector<int>& lat_of) {
   int n = 0;
-  for (int q : lat_of) n += num_site_blocks(h->lat[q].g, 64);
+  for (int q : lat_of) n += 4 * num_site_blocks(h->lat[q].g, 64);
   return n;
 }
+// The wide kernels' sites per block: 16 while the blocks of both sides fit the SMs twice, so
+// that an SM holds few warps and each runs near its own latency, else 32. They are tried up to
+// kWideSites sites in all; above, the lattice fills the GPU with one thread a site.
+constexpr size_t kWideSites = 100000;
+static int wide_sites(int nblocks64) { return nblocks64 * 4 * 2 <= 2 * 152 ? 16 : 32; }
 
 static std::vector<int> lattices_of_call(const ov_handle* h, int nprob) {
   std::vector<int> v(nprob, 0);
@@ -724,16 +735,23 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
   size_t pool = 0;
   // block size: forced by opts.block_size, else the tuned one for this problem set, else
   // tuned below at the first step
-  const TuneKey key{h->prec, mode, nrhs, 0};
-  int bs = o.block_size;
+  const bool relaxing = !strict_only && o.relax > 0.0 && h->prec == OV_PREC_DF64;
+  const TuneKey key{relaxing ? kPrecDF64Relaxed : h->prec, mode, nrhs};
+  int bs = o.block_size, wide = 0;
   bool tune = false;
   if (bs == 0) {
     auto it = h->tuned.find(key);
-    if (it != h->tuned.end()) bs = it->second;
-    else { bs = kBlockDefault; tune = true; }
+    if (it != h->tuned.end()) {
+      bs = it->second.bs;
+      wide = it->second.wide;
+    } else {
+      bs = kBlockDefault;
+      tune = true;
+    }
   }
   int rc = build_batch(h, lat_of, bs, &bt, &pool, neg_mu);
   if (rc != OV_OK) return rc;
+  bt.wide = wide;
   rc = ensure_outer(h, nrhs, ld, pool, max_blocks(h, lat_of));
   if (rc != OV_OK) return rc;
   const int gcap = check_group_cap(h, nrhs, pool, o);
@@ -832,7 +850,6 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
   // hopping error, ~1e-7 of |A v| in every direction, puts back components along the
   // removed eigenvectors, whose eigenvalues lie inside the deflation gap that the
   // shortened Krylov space no longer resolves
-  const bool relaxing = !strict_only && o.relax > 0.0 && h->prec == OV_PREC_DF64;
   int relax_from = INT_MAX;
   if (relaxing) {
     if (o.k_fixed > 0) relax_from = std::max(1, (int)std::ceil(o.relax * o.k_fixed));
@@ -883,12 +900,19 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
         CK(cudaEventCreate(&e0));
         CK(cudaEventCreate(&e1));
         float best = 1e30f;
-        int best_bs = kBlockDefault;
-        for (int cand : {64, 128, 256}) {
+        Tuned best_t{kBlockDefault, 0};
+        std::vector<Tuned> cands = {{64, 0}, {128, 0}, {256, 0}};
+        if (h->prec == OV_PREC_DF64 && !relaxing && pool / 12 <= kWideSites) {
+          int nb64 = 0;
+          for (int q : lat_of) nb64 += num_site_blocks(h->lat[q].g, 64);
+          cands.push_back({64, wide_sites(nb64)});
+        }
+        for (const Tuned& cand : cands) {
           Batch bc;
           size_t pc = 0;
-          rc = build_batch(h, lat_of, cand, &bc, &pc, neg_mu);
+          rc = build_batch(h, lat_of, cand.bs, &bc, &pc, neg_mu);
           if (rc != OV_OK) return rc;
+          bc.wide = cand.wide;
           a.b = bc;
           float tmin = 1e30f;
           for (int rep = 0; rep < 2; ++rep) {
@@ -901,15 +925,16 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
             tmin = std::min(tmin, ms);
           }
           h->stats.launches += 2;
-          if (tmin < best) { best = tmin; best_bs = cand; }
+          if (tmin < best) { best = tmin; best_t = cand; }
         }
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
-        h->tuned[key] = best_bs;
-        rc = build_batch(h, lat_of, best_bs, &bt, &pool, neg_mu);
+        h->tuned[key] = best_t;
+        rc = build_batch(h, lat_of, best_t.bs, &bt, &pool, neg_mu);
         if (rc != OV_OK) return rc;
+        bt.wide = best_t.wide;
         a.b = bt;
-        if (h->trace) fprintf(stderr, "{\"ov_autotune\": %d, \"ms\": %.4f}\n", best_bs, best);
+        if (h->trace) fprintf(stderr, "{\"ov_autotune\": %d, \"wide\": %d, \"ms\": %.4f}\n", best_t.bs, best_t.wide, best);
       }
       h->stats.block_size = a.b.block;
       // steps jn..jto: whole graph units replayed, the rest launched one by one
@@ -1542,6 +1567,7 @@ int ov::apply_set_create(ov_handle* h, const std::vector<ApplyItem>& items, size
   a->bt.nblocks = blk;
   a->bt.nprob = np;
   a->bt.block = bs;
+  a->bt.wide = 0;
   a->pool = pool;
   a->nitems = np;
   a->maxblk = maxblk;
@@ -1797,8 +1823,13 @@ extern "C" int ov_wilson_apply(ov_handle* h, int nrhs, const void* x, void* y, i
   Batch bt;
   size_t pool = 0;
   const std::vector<int> lat_of = lattices_of_call(h, nrhs);
-  int rc = build_batch(h, lat_of, h->o.block_size ? h->o.block_size : kBlockDefault, &bt, &pool);
+  // (a small lattice: the wide kernel, as the tuner finds for its steps)
+  int nb64 = 0;
+  for (int q : lat_of) nb64 += num_site_blocks(h->lat[q].g, 64);
+  const bool wide = h->prec == OV_PREC_DF64 && !h->o.block_size && (size_t)nb64 * 64 <= kWideSites / 4;
+  int rc = build_batch(h, lat_of, h->o.block_size ? h->o.block_size : (wide ? 64 : kBlockDefault), &bt, &pool);
   if (rc != OV_OK) return rc;
+  if (wide) bt.wide = wide_sites(nb64);
   rc = ensure_outer(h, nrhs, std::max(h->cap_ld, 4), pool, max_blocks(h, lat_of));
   if (rc != OV_OK) return rc;
   const size_t canon = sizeof(double2) * pool;

@@ -62,6 +62,7 @@ struct Batch {
   const int2* blk_map;   // device [nblocks]: (problem, site block within the problem) of each block
   int nblocks, nprob;
   int block;             // threads per site block (64, 128 or 256)
+  int wide;              // 0, or sites per block (16 or 32) of the wide step and update kernels (block = 64)
 };
 
 // Arguments of one outer step (vector pointers are pools; problem r's vectors start at

@@ -667,6 +667,29 @@ constexpr int step_min_blocks() {
   return t / BS > 0 ? t / BS : 1;
 }
 
+// alpha_j from the total of its partial sums, and the update's scalars (one thread)
+template <class P, int MODE>
+__device__ __forceinline__ void finish_alpha(const StepArgs& a, int r, size_t co, const double (&tot)[2]) {
+  const double nvj = a.c.nv[co];
+  double ar, ai;
+  double2 nw = a.c.nw[co];
+  if (MODE == kModeLanczos) {
+    ar = tot[0] / nvj;
+    ai = 0.0;
+    nw = make_double2(nvj, 0.0);
+  } else {
+    // (tot) / nw_j
+    const double den = nw.x * nw.x + nw.y * nw.y;
+    ar = (tot[0] * nw.x + tot[1] * nw.y) / den;
+    ai = (tot[1] * nw.x - tot[0] * nw.y) / den;
+  }
+  a.c.alp[co] = make_double2(ar, ai);
+  // alpha_j / nv_j and conj(alpha_j) / conj(nw_j) = conj(alpha_j / nw_j)
+  st_scal<P>(a.scal, r, 4, ar / nvj, ai / nvj);
+  const double dw = nw.x * nw.x + nw.y * nw.y;
+  st_scal<P>(a.scal, r, 5, (ar * nw.x + ai * nw.y) / dw, -((ai * nw.x - ar * nw.y) / dw));
+}
+
 template <class P, int MODE, int BS>
 __global__ void __launch_bounds__(BS, step_min_blocks<P, BS>()) k_step(StepArgs a) {
   using R = typename P::R;
@@ -760,24 +783,7 @@ __global__ void __launch_bounds__(BS, step_min_blocks<P, BS>()) k_step(StepArgs 
   A v2[2] = {dot.re, dot.im};
   double tot[2];
   if (reduce_last<2, BS>(v2, a.partials, a.counters, r, d.block0, sr.bx, d.nblk, tot) && threadIdx.x == 0) {
-    const double nvj = a.c.nv[co];
-    double ar, ai;
-    double2 nw = a.c.nw[co];
-    if (MODE == kModeLanczos) {
-      ar = tot[0] / nvj;
-      ai = 0.0;
-      nw = make_double2(nvj, 0.0);
-    } else {
-      // (tot) / nw_j
-      const double den = nw.x * nw.x + nw.y * nw.y;
-      ar = (tot[0] * nw.x + tot[1] * nw.y) / den;
-      ai = (tot[1] * nw.x - tot[0] * nw.y) / den;
-    }
-    a.c.alp[co] = make_double2(ar, ai);
-    // alpha_j / nv_j and conj(alpha_j) / conj(nw_j) = conj(alpha_j / nw_j)
-    st_scal<P>(a.scal, r, 4, ar / nvj, ai / nvj);
-    const double dw = nw.x * nw.x + nw.y * nw.y;
-    st_scal<P>(a.scal, r, 5, (ar * nw.x + ai * nw.y) / dw, -((ai * nw.x - ar * nw.y) / dw));
+    finish_alpha<P, MODE>(a, r, co, tot);
   }
 }
 
@@ -794,6 +800,59 @@ __global__ void __launch_bounds__(BS, step_min_blocks<P, BS>()) k_step(StepArgs 
 #else
 #define OV_UPDATE_BOUNDS(BS) __launch_bounds__(BS)
 #endif
+// beta_{j+1} and the next step's scalars from ||t_{j+1}||^2 (one thread)
+template <class P>
+__device__ __forceinline__ void finish_lanczos(const StepArgs& a, int r, size_t co, int j, double tot) {
+  const double b = sqrt(tot);
+  const double bprev = fabs(a.c.bet[co].x);
+  const size_t cn = co + 1;
+  const bool broke = !(b > a.breakdown_tol * (fabs(a.c.alp[co].x) + bprev));
+  if (broke && a.c.status[r] == kStOK) {
+    a.c.status[r] = kStLucky;
+    a.c.kbreak[r] = j;
+  }
+  const bool dead = a.c.status[r] != kStOK;
+  a.c.nv[cn] = dead ? 1.0 : b;
+  a.c.nw[cn] = make_double2(dead ? 1.0 : b, 0.0);
+  a.c.bet[cn] = make_double2(dead ? 0.0 : b, 0.0);
+  a.c.gam[cn] = make_double2(dead ? 0.0 : b, 0.0);
+  set_step_scal<P>(a.scal, r, a.c.nv[cn], a.c.gam[cn], a.c.nw[cn], a.c.bet[cn], a.c.nv[co], a.c.nw[co]);
+}
+// beta_{j+1}, gamma_{j+1} and the next step's scalars from tw^dag t, ||t||^2, ||tw||^2 (one thread)
+template <class P>
+__device__ __forceinline__ void finish_two_sided(const StepArgs& a, int r, size_t co, int j, const double (&tot)[4]) {
+  const double dre = tot[0], dim = tot[1];
+  const double ad = sqrt(dre * dre + dim * dim);
+  const double b = sqrt(ad);
+  const size_t cn = co + 1;
+  const bool broke = !(ad > a.breakdown_tol * sqrt(tot[2]) * sqrt(tot[3])) || !(b > 0.0);
+  if (broke && a.c.status[r] == kStOK) {
+    a.c.status[r] = kStBreakdown;
+    a.c.kbreak[r] = j;
+  }
+  const bool dead = a.c.status[r] != kStOK;
+  a.c.nv[cn] = dead ? 1.0 : b;
+  a.c.nw[cn] = dead ? make_double2(1.0, 0.0) : make_double2(dre / b, dim / b);
+  a.c.bet[cn] = make_double2(dead ? 0.0 : b, 0.0);
+  a.c.gam[cn] = dead ? make_double2(0.0, 0.0) : make_double2(dre / b, dim / b);
+  set_step_scal<P>(a.scal, r, a.c.nv[cn], a.c.gam[cn], a.c.nw[cn], a.c.bet[cn], a.c.nv[co], a.c.nw[co]);
+}
+__device__ __forceinline__ void advance_step(const StepArgs& a, int j) {
+  // device-side step state: the last block of the launch advances j
+  if (a.jdev) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      __threadfence();
+      const unsigned t = atomicAdd(a.gticket, 1u);
+      if (t == gridDim.x - 1) {
+        *a.jdev = j + 1;
+        *a.gticket = 0u;
+        __threadfence();
+      }
+    }
+  }
+}
+
 template <class P, int MODE, int BS>
 __global__ void OV_UPDATE_BOUNDS(BS) k_update(StepArgs a) {
   using R = typename P::R;
@@ -843,55 +902,209 @@ __global__ void OV_UPDATE_BOUNDS(BS) k_update(StepArgs a) {
     A v1[1] = {nvv};
     double tot[1];
     if (reduce_last<1, BS>(v1, a.partials, a.counters, r, sr.d->block0, sr.bx, sr.d->nblk, tot) && threadIdx.x == 0) {
-      const double b = sqrt(tot[0]);
-      const double bprev = fabs(a.c.bet[co].x);
-      const size_t cn = co + 1;
-      const bool broke = !(b > a.breakdown_tol * (fabs(a.c.alp[co].x) + bprev));
-      if (broke && a.c.status[r] == kStOK) {
-        a.c.status[r] = kStLucky;
-        a.c.kbreak[r] = sp.j;
-      }
-      const bool dead = a.c.status[r] != kStOK;
-      a.c.nv[cn] = dead ? 1.0 : b;
-      a.c.nw[cn] = make_double2(dead ? 1.0 : b, 0.0);
-      a.c.bet[cn] = make_double2(dead ? 0.0 : b, 0.0);
-      a.c.gam[cn] = make_double2(dead ? 0.0 : b, 0.0);
-      set_step_scal<P>(a.scal, r, a.c.nv[cn], a.c.gam[cn], a.c.nw[cn], a.c.bet[cn], a.c.nv[co], a.c.nw[co]);
+      finish_lanczos<P>(a, r, co, sp.j, tot[0]);
     }
   } else {
     A v4[4] = {d.re, d.im, to_acc(nvl, A()), to_acc(nwl, A())};
     double tot[4];
     if (reduce_last<4, BS>(v4, a.partials, a.counters, r, sr.d->block0, sr.bx, sr.d->nblk, tot) && threadIdx.x == 0) {
-      const double dre = tot[0], dim = tot[1];
-      const double ad = sqrt(dre * dre + dim * dim);
-      const double b = sqrt(ad);
-      const size_t cn = co + 1;
-      const bool broke = !(ad > a.breakdown_tol * sqrt(tot[2]) * sqrt(tot[3])) || !(b > 0.0);
-      if (broke && a.c.status[r] == kStOK) {
-        a.c.status[r] = kStBreakdown;
-        a.c.kbreak[r] = sp.j;
-      }
-      const bool dead = a.c.status[r] != kStOK;
-      a.c.nv[cn] = dead ? 1.0 : b;
-      a.c.nw[cn] = dead ? make_double2(1.0, 0.0) : make_double2(dre / b, dim / b);
-      a.c.bet[cn] = make_double2(dead ? 0.0 : b, 0.0);
-      a.c.gam[cn] = dead ? make_double2(0.0, 0.0) : make_double2(dre / b, dim / b);
-      set_step_scal<P>(a.scal, r, a.c.nv[cn], a.c.gam[cn], a.c.nw[cn], a.c.bet[cn], a.c.nv[co], a.c.nw[co]);
+      finish_two_sided<P>(a, r, co, sp.j, tot);
     }
   }
-  // device-side step state: the last block of the launch advances j
-  if (a.jdev) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      __threadfence();
-      const unsigned t = atomicAdd(a.gticket, 1u);
-      if (t == gridDim.x - 1) {
-        *a.jdev = sp.j + 1;
-        *a.gticket = 0u;
-        __threadfence();
+  advance_step(a, sp.j);
+}
+
+// ------------------------------------------------------------ small lattices
+// One thread a site runs ~29 k instructions one after the other in a strict two-sided step, and
+// a lattice with fewer sites than the GPU has threads spends just that latency: 45 us a step on
+// 8^4. The wide kernels give a site twelve threads: the two sides of the step to different
+// blocks (blockIdx.y; alpha's partial sum moves to the v side, which reads tw_j), the three
+// colour rows of the result to different warps, the two upper spin components to the half
+// warps. A thread projects and multiplies its half-spinor's row (the projection is repeated by
+// the three colours: a third more work in all) and owns two of the twelve components, upper
+// spin `sp` and lower spin 2 + sp of its colour; the lower one takes its own or the other half
+// warp's product, by a shuffle. The sums of a component keep their order. A block takes WS
+// consecutive sites of a 64-site block of the map. MEASURED_WIDE
+__device__ __forceinline__ dfu shfl_half(dfu v) {
+  return {__shfl_xor_sync(0xffffffffu, v.hi, 16), __shfl_xor_sync(0xffffffffu, v.lo, 16)};
+}
+template <int WS>
+struct WideRef {
+  static constexpr int threads = 6 * WS, sub = 64 / WS;
+  int r, bx, s, col, sp;
+  bool active;
+  const ProbDesc* d;
+};
+template <int WS>
+__device__ __forceinline__ WideRef<WS> wide_ref(const Batch& b) {
+  constexpr int sub = WideRef<WS>::sub;
+  const int2 m = __ldg(&b.blk_map[blockIdx.x / sub]);
+  const ProbDesc* d = &b.desc[m.x];
+  const int warp = threadIdx.x >> 5, bx = m.y * sub + blockIdx.x % sub;
+  const int s = bx * WS + (warp / 3) * 16 + (threadIdx.x & 15);
+  return {m.x, bx, s, warp % 3, (int)(threadIdx.x >> 4) & 1, s < d->g.V, d};
+}
+
+// the hopping sum of hopping_df for components 3 sp + col (up) and 6 + 3 sp + col (lo)
+__device__ __forceinline__ void hopping_wide(cx<df64>& up, cx<df64>& lo, const float4* __restrict__ src,
+                                             const float2* __restrict__ links, const Geometry& g, int s,
+                                             const int (&xc)[4], df64 ef, df64 eb, int col, int sp) {
+  const int V = g.V;
+  const float2* __restrict__ links_lo = links + (size_t)36 * V;
+  cxu au = {{0.f, 0.f}, {0.f, 0.f}}, al = au;
+#pragma unroll 1
+  for (int hop = 0; hop < 8; ++hop) {
+    const int nu = hop >> 1;
+    const bool fwd = (hop & 1) == 0;
+    const int Ln = nu == 0 ? g.Lx : (nu == 1 ? g.Ly : (nu == 2 ? g.Lz : g.Lt));
+    const int st = nu == 0 ? 1 : (nu == 1 ? g.Lx : (nu == 2 ? g.Lx * g.Ly : g.Lx * g.Ly * g.Lz));
+    const int c = xc[0] * (nu == 0) + xc[1] * (nu == 1) + xc[2] * (nu == 2) + xc[3] * (nu == 3);
+    const int sn = fwd ? (c == Ln - 1 ? s - (Ln - 1) * st : s + st) : (c == 0 ? s + (Ln - 1) * st : s - st);
+    const int ls = fwd ? s : sn;
+    cx<float> u[3], ulo[3];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const int idx = fwd ? col * 3 + b : b * 3 + col;
+      u[b] = lconj(ld_link(links + (size_t)(nu * 9 + idx) * V + ls), !fwd);
+      ulo[b] = lconj(ld_link(links_lo + (size_t)(nu * 9 + idx) * V + ls), !fwd);
+    }
+    const int bs = c_bsrc[nu][sp], bq = (c_bph[nu][sp] + (fwd ? 2 : 0)) & 3;
+    cx<df64> h[3];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const cx<df64> p = ld_vec(src + (size_t)(3 * sp + b) * V + sn);
+      const cx<df64> q = rot(ld_vec(src + (size_t)(3 * bs + b) * V + sn), bq);
+      const dfu re = add_u(to_u(p.re), to_u(q.re)), im = add_u(to_u(p.im), to_u(q.im));
+      h[b] = {{re.hi, re.lo}, {im.hi, im.lo}};
+    }
+    cxu gs;
+    float cr = 0.f, ci = 0.f;
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      if (b == 0) {
+        set_u(gs.re, u[b].re, h[b].re);
+        set_u(gs.im, u[b].re, h[b].im);
+      } else {
+        madd_u(gs.re, u[b].re, h[b].re);
+        madd_u(gs.im, u[b].re, h[b].im);
+      }
+      madd_u(gs.re, -u[b].im, h[b].im);
+      madd_u(gs.im, u[b].im, h[b].re);
+      cr = __fmaf_rn(ulo[b].re, h[b].re.hi, __fmaf_rn(-ulo[b].im, h[b].im.hi, cr));
+      ci = __fmaf_rn(ulo[b].re, h[b].im.hi, __fmaf_rn(ulo[b].im, h[b].re.hi, ci));
+    }
+    gs.re.lo = __fadd_rn(gs.re.lo, cr);
+    gs.im.lo = __fadd_rn(gs.im.lo, ci);
+    if (nu == 3) {
+      const cx<df64> n = cscale(cx<df64>{norm_u(gs.re), norm_u(gs.im)}, fwd ? ef : eb);
+      gs = {to_u(n.re), to_u(n.im)};
+    }
+    const cxu go = {shfl_half(gs.re), shfl_half(gs.im)};
+    au = cadd_u(au, gs);
+    al = cadd_u(al, rot_u(c_dsrc[nu][sp] == sp ? gs : go, (c_dph[nu][sp] + (fwd ? 2 : 0)) & 3));
+  }
+  up = {norm_u(au.re), norm_u(au.im)};
+  lo = {norm_u(al.re), norm_u(al.im)};
+}
+
+template <int MODE, int WS>
+__global__ void __launch_bounds__(6 * WS) k_step_wide(StepArgs a) {
+  using P = PrecDF64;
+  const WideRef<WS> sr = wide_ref<WS>(a.b);
+  const ProbDesc& d = *sr.d;
+  const Geometry g = d.g;
+  const int r = sr.r, V = g.V;
+  const int ss = sr.active ? sr.s : 0;
+  const size_t vo = d.voff;
+  const df64 mass = {d.mass_hl[0], d.mass_hl[1]}, emu = {d.emu_hl[0], d.emu_hl[1]}, emui = {d.emui_hl[0], d.emui_hl[1]};
+  int xc[4];
+  site_coords(g, ss, xc[0], xc[1], xc[2], xc[3]);
+  const int k0 = 3 * sr.sp + sr.col, k1 = 6 + k0;  // this thread's components
+  cx<df64> up, lo;
+  if (MODE == kModeApply) {
+    const float4* tv = (const float4*)a.tv + vo;
+    hopping_wide(up, lo, tv, (const float2*)d.links, g, ss, xc, a.dagger ? emui : emu, a.dagger ? emu : emui, sr.col, sr.sp);
+    if (!sr.active) return;
+    float4* out = (float4*)a.p + vo + ss;
+    st_vec(out + (size_t)k0 * V, g5d(k0, ld_vec(tv + (size_t)k0 * V + ss), up, mass));
+    st_vec(out + (size_t)k1 * V, g5d(k1, ld_vec(tv + (size_t)k1 * V + ss), lo, mass));
+    return;
+  }
+  const StepPtrs sp = step_ptrs(a);
+  const size_t co = (size_t)r * a.c.ld + sp.j;
+  const int side = MODE == kModeTwoSided ? blockIdx.y : 0;
+  const cx<df64> scl = ld_scal<P>(a.scal, r, 2 * side), cf = ld_scal<P>(a.scal, r, 2 * side + 1);
+  const float4* src = (const float4*)(side == 0 ? sp.tc : sp.wc) + vo;
+  const float4* prv = (const float4*)(side == 0 ? sp.tp : sp.wp) + vo + ss;
+  float4* out = (float4*)(side == 0 ? a.p : a.r) + vo + ss;
+  hopping_wide(up, lo, src, (const float2*)d.links, g, ss, xc, side == 0 ? emu : emui, side == 0 ? emui : emu, sr.col, sr.sp);
+  cx<df64> dot = {df_zero(), df_zero()};
+  if (sr.active) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int k = q == 0 ? k0 : k1;
+      const cx<df64> psi = ld_vec(src + (size_t)k * V + ss), pv = ld_vec(prv + (size_t)k * V);
+      const cx<df64> h = g5d(k, psi, q == 0 ? up : lo, mass);
+      cx<df64> ok;
+      if (MODE == kModeLanczos) ok = smulsub<true, true>(scl, h, cf, pv);
+      else if (side == 0) ok = smulsub<true, false>(scl, h, cf, pv);
+      else ok = smulsub<false, false>(scl, h, cf, pv);
+      st_vec(out + (size_t)k * V, ok);
+      if (MODE == kModeLanczos) acc_dot(dot, psi, ok);
+      else if (side == 0) acc_dot(dot, ld_vec((const float4*)sp.wc + vo + (size_t)k * V + ss), ok);
+    }
+  }
+  if (side != 0) return;
+  df64 v2[2] = {dot.re, dot.im};
+  double tot[2];
+  constexpr int sub = WideRef<WS>::sub;
+  if (reduce_last<2, 6 * WS>(v2, a.partials, a.counters, r, d.block0 * sub, sr.bx, d.nblk * sub, tot) && threadIdx.x == 0)
+    finish_alpha<P, MODE>(a, r, co, tot);
+}
+
+template <int MODE, int WS>
+__global__ void __launch_bounds__(6 * WS) k_update_wide(StepArgs a) {
+  using P = PrecDF64;
+  const WideRef<WS> sr = wide_ref<WS>(a.b);
+  const int V = sr.d->g.V, r = sr.r;
+  const StepPtrs sp = step_ptrs(a);
+  const size_t co = (size_t)r * a.c.ld + sp.j;
+  const cx<df64> alp = ld_scal<P>(a.scal, r, 4), calp = ld_scal<P>(a.scal, r, 5);
+  cx<df64> d = {df_zero(), df_zero()};
+  df64 nvv = df_zero();
+  float nvl = 0.f, nwl = 0.f;
+  if (sr.active) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const size_t o = sr.d->voff + sr.s + (size_t)(6 * q + 3 * sr.sp + sr.col) * V;
+      const cx<df64> t = csubmul(ld_vec((const float4*)a.p + o), alp, ld_vec((const float4*)sp.tc + o));
+      if (MODE == kModeLanczos) {
+        st_vec((float4*)sp.tn + o, t);
+        acc_norm(nvv, t);
+      } else {
+        const cx<df64> u = csubmul(ld_vec((const float4*)a.r + o), calp, ld_vec((const float4*)sp.wc + o));
+        st_vec((float4*)sp.tn + o, t);
+        st_vec((float4*)sp.wn + o, u);
+        acc_dot(d, u, t);
+        acc_norm_lo(nvl, t);
+        acc_norm_lo(nwl, u);
       }
     }
   }
+  constexpr int sub = WideRef<WS>::sub;
+  const int part0 = sr.d->block0 * sub, nblk = sr.d->nblk * sub;
+  if (MODE == kModeLanczos) {
+    df64 v1[1] = {nvv};
+    double tot[1];
+    if (reduce_last<1, 6 * WS>(v1, a.partials, a.counters, r, part0, sr.bx, nblk, tot) && threadIdx.x == 0)
+      finish_lanczos<P>(a, r, co, sp.j, tot[0]);
+  } else {
+    df64 v4[4] = {d.re, d.im, {nvl, 0.f}, {nwl, 0.f}};
+    double tot[4];
+    if (reduce_last<4, 6 * WS>(v4, a.partials, a.counters, r, part0, sr.bx, nblk, tot) && threadIdx.x == 0)
+      finish_two_sided<P>(a, r, co, sp.j, tot);
+  }
+  advance_step(a, sp.j);
 }
 
 // ------------------------------------------------------------ recombination
@@ -1003,8 +1216,24 @@ cudaError_t launch_unpack(int prec, const Batch& b, const void* xi, double2* y, 
   if (prec == kPrecDF64Relaxed) { using P = PrecDF64R; CALL; }      \
   else { OV_DISPATCH(prec, CALL) }
 
+// the wide kernels (strict double-float steps; a.b.wide sites a block, within the map's blocks of 64)
+#define OV_WIDE_DISPATCH(ws, CALL)                        \
+  if (ws == 16) { constexpr int WS = 16; CALL; }          \
+  else { constexpr int WS = 32; CALL; }
+
 cudaError_t launch_step(int prec, int mode, const StepArgs& a, cudaStream_t st) {
   const int grid = a.b.nblocks;
+  if (a.b.wide && prec == OV_PREC_DF64 && mode != kModeRegen) {
+    const dim3 wg(grid * (64 / a.b.wide), mode == kModeTwoSided ? 2 : 1);
+    if (mode == kModeLanczos) {
+      OV_WIDE_DISPATCH(a.b.wide, (k_step_wide<kModeLanczos, WS><<<wg, 6 * WS, 0, st>>>(a)));
+    } else if (mode == kModeTwoSided) {
+      OV_WIDE_DISPATCH(a.b.wide, (k_step_wide<kModeTwoSided, WS><<<wg, 6 * WS, 0, st>>>(a)));
+    } else {
+      OV_WIDE_DISPATCH(a.b.wide, (k_step_wide<kModeApply, WS><<<wg, 6 * WS, 0, st>>>(a)));
+    }
+    return cudaGetLastError();
+  }
   switch (mode) {
     case kModeLanczos:
       OV_BS_DISPATCH(a.b.block, OV_STEP_DISPATCH(prec, (k_step<P, kModeLanczos, BS><<<grid, BS, 0, st>>>(a))));
@@ -1024,6 +1253,15 @@ cudaError_t launch_step(int prec, int mode, const StepArgs& a, cudaStream_t st) 
 
 cudaError_t launch_update(int prec, int mode, const StepArgs& a, cudaStream_t st) {
   const int grid = a.b.nblocks;
+  if (a.b.wide && prec == OV_PREC_DF64) {
+    const int wg = grid * (64 / a.b.wide);
+    if (mode == kModeLanczos) {
+      OV_WIDE_DISPATCH(a.b.wide, (k_update_wide<kModeLanczos, WS><<<wg, 6 * WS, 0, st>>>(a)));
+    } else {
+      OV_WIDE_DISPATCH(a.b.wide, (k_update_wide<kModeTwoSided, WS><<<wg, 6 * WS, 0, st>>>(a)));
+    }
+    return cudaGetLastError();
+  }
   if (mode == kModeLanczos) {
     OV_BS_DISPATCH(a.b.block, OV_DISPATCH(prec, (k_update<P, kModeLanczos, BS><<<grid, BS, 0, st>>>(a))));
   } else {
