@@ -94,27 +94,33 @@ template <class P>
 __device__ __forceinline__ void st_scal(void* scal, int r, int q, double re, double im) {
   st_vec((typename P::vec_t*)scal + (size_t)r * 8 + q, cd_to<typename P::R>(re, im));
 }
+// The scalars are formed by one warp, a quotient a lane: a double division is a chain of dozens
+// of instructions on a pipe that gives two lanes a cycle, and one thread doing a step's ~20
+// divisions and roots in turn held up the next kernel.
+__device__ __forceinline__ double bcast(double v, int lane) { return __shfl_sync(0xffffffffu, v, lane); }
 // scalars of step j from its coefficients nv_j, gamma_j, nw_j, beta_j and the previous
-// normalisations nv_{j-1}, nw_{j-1} (run by one thread):
+// normalisations nv_{j-1}, nw_{j-1} (run by a warp; the arguments are the same in every lane):
 //   1/nv_j, gamma_j/nv_{j-1}, 1/conj(nw_j), conj(beta_j)/conj(nw_{j-1})
 template <class P>
 __device__ __forceinline__ void set_step_scal(void* scal, int r, double nv, double2 gam, double2 nw, double2 bet,
                                               double nvp, double2 nwp) {
-  st_scal<P>(scal, r, 0, 1.0 / nv, 0.0);
-  st_scal<P>(scal, r, 1, gam.x / nvp, gam.y / nvp);
-  const double den = nw.x * nw.x + nw.y * nw.y;
-  st_scal<P>(scal, r, 2, nw.x / den, nw.y / den);  // 1/conj(nw) = nw/|nw|^2
+  const int lane = threadIdx.x & 31;
+  const double den = nw.x * nw.x + nw.y * nw.y;  // 1/conj(nw) = nw/|nw|^2
   // conj(beta)/conj(nwp) = conj(beta/nwp), beta/nwp = beta conj(nwp)/|nwp|^2
   const double dp = nwp.x * nwp.x + nwp.y * nwp.y;
-  const double qr = (bet.x * nwp.x + bet.y * nwp.y) / dp, qi = (bet.y * nwp.x - bet.x * nwp.y) / dp;
-  st_scal<P>(scal, r, 3, qr, -qi);
+  const double num = lane == 0 ? 1.0 : lane == 2 ? gam.x : lane == 3 ? gam.y : lane == 4 ? nw.x : lane == 5 ? nw.y
+                     : lane == 6 ? bet.x * nwp.x + bet.y * nwp.y : bet.y * nwp.x - bet.x * nwp.y;
+  const double dn = lane == 0 ? nv : lane < 4 ? nvp : lane < 6 ? den : dp;
+  const double q = lane == 1 ? 0.0 : lane < 8 ? num / dn : 0.0;
+  const double im = __shfl_down_sync(0xffffffffu, q, 1);
+  if (lane < 8 && !(lane & 1)) st_scal<P>(scal, r, lane >> 1, q, lane == 6 ? -im : im);
 }
 
 // ------------------------------------------------------------ block reductions
 // Each thread passes its values; the block's sums go to partials[(part0 + bx)*4 + q]
 // (part0: the problem's first slot, bx: the block's index within the problem, so the
 // slots do not depend on the launch order of the blocks). Returns true in the last block
-// to finish for this problem, where tot[] (valid in thread 0) holds the fixed-order total
+// to finish for this problem, where tot[] (valid in warp 0) holds the fixed-order total
 // over all its blocks.
 // The block's per-warp sums (thread 0 adds them in warp order).
 template <int NQ, int BS>
@@ -176,28 +182,32 @@ __device__ __forceinline__ bool reduce_last(T (&v)[NQ], double* partials, unsign
   __syncthreads();
   if (!s_last) return false;
   __threadfence();
-  double loc[NQ];
+  // the warps that have partials to add (the double pipe serves a warp's instruction in 16
+  // cycles: idle warps adding zeros would hold up the others)
+  const int nw = min(BS / 32, (nblk + 31) / 32);
+  if (warp < nw) {
+    double loc[NQ];
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) loc[q] = 0.0;
-  for (int b = tid; b < nblk; b += BS) {
+    for (int q = 0; q < NQ; ++q) loc[q] = 0.0;
+    for (int b = tid; b < nblk; b += BS) {
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) loc[q] += __ldcg(&partials[(size_t)(part0 + b) * 4 + q]);
+      for (int q = 0; q < NQ; ++q) loc[q] += __ldcg(&partials[(size_t)(part0 + b) * 4 + q]);
+    }
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      double w = warp_sum(loc[q]);
+      if (lane == 0) sred[warp][q] = w;
+    }
   }
   __syncthreads();
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    double w = warp_sum(loc[q]);
-    if (lane == 0) sred[warp][q] = w;
-  }
-  __syncthreads();
-  if (tid == 0) {
+  if (warp == 0) {
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
       double s = 0.0;
-      for (int w = 0; w < BS / 32; ++w) s += sred[w][q];
+      for (int w = 0; w < nw; ++w) s += sred[w][q];
       tot[q] = s;
     }
-    counters[r] = 0u;
+    if (lane == 0) counters[r] = 0u;
   }
   return true;
 }
@@ -247,16 +257,19 @@ __global__ void __launch_bounds__(BS) k_pack(Batch bt, const double2* __restrict
   }
   if (!want_norm) return;
   double v[1] = {n2}, tot[1];
-  if (reduce_last<1, BS>(v, partials, counters, r, sr.d->block0, sr.bx, sr.d->nblk, tot) && threadIdx.x == 0) {
-    double nrm = sqrt(tot[0]);
-    size_t o = (size_t)r * c.ld + 1;
-    c.nv[o] = nrm > 0.0 ? nrm : 1.0;
-    c.nw[o] = make_double2(nrm > 0.0 ? nrm : 1.0, 0.0);
-    c.bet[o] = make_double2(0.0, 0.0);
-    c.gam[o] = make_double2(0.0, 0.0);
-    c.status[r] = nrm > 0.0 ? kStOK : kStZero;
-    c.kbreak[r] = 0;
-    if (scal) set_step_scal<P>(scal, r, c.nv[o], c.gam[o], c.nw[o], c.bet[o], 1.0, make_double2(1.0, 0.0));
+  if (reduce_last<1, BS>(v, partials, counters, r, sr.d->block0, sr.bx, sr.d->nblk, tot) && threadIdx.x < 32) {
+    const double nrm = sqrt(tot[0]), n1 = nrm > 0.0 ? nrm : 1.0;
+    const double2 zero = make_double2(0.0, 0.0), w1 = make_double2(n1, 0.0);
+    if (threadIdx.x == 0) {
+      const size_t o = (size_t)r * c.ld + 1;
+      c.nv[o] = n1;
+      c.nw[o] = w1;
+      c.bet[o] = zero;
+      c.gam[o] = zero;
+      c.status[r] = nrm > 0.0 ? kStOK : kStZero;
+      c.kbreak[r] = 0;
+    }
+    if (scal) set_step_scal<P>(scal, r, n1, zero, w1, zero, 1.0, make_double2(1.0, 0.0));
   }
 }
 
@@ -667,9 +680,10 @@ constexpr int step_min_blocks() {
   return t / BS > 0 ? t / BS : 1;
 }
 
-// alpha_j from the total of its partial sums, and the update's scalars (one thread)
+// alpha_j from the total of its partial sums, and the update's scalars (one warp)
 template <class P, int MODE>
 __device__ __forceinline__ void finish_alpha(const StepArgs& a, int r, size_t co, const double (&tot)[2]) {
+  const int lane = threadIdx.x & 31;
   const double nvj = a.c.nv[co];
   double ar, ai;
   double2 nw = a.c.nw[co];
@@ -680,14 +694,20 @@ __device__ __forceinline__ void finish_alpha(const StepArgs& a, int r, size_t co
   } else {
     // (tot) / nw_j
     const double den = nw.x * nw.x + nw.y * nw.y;
-    ar = (tot[0] * nw.x + tot[1] * nw.y) / den;
-    ai = (tot[1] * nw.x - tot[0] * nw.y) / den;
+    const double q = (lane == 0 ? tot[0] * nw.x + tot[1] * nw.y : tot[1] * nw.x - tot[0] * nw.y) / den;
+    ar = bcast(q, 0);
+    ai = bcast(q, 1);
   }
-  a.c.alp[co] = make_double2(ar, ai);
   // alpha_j / nv_j and conj(alpha_j) / conj(nw_j) = conj(alpha_j / nw_j)
-  st_scal<P>(a.scal, r, 4, ar / nvj, ai / nvj);
   const double dw = nw.x * nw.x + nw.y * nw.y;
-  st_scal<P>(a.scal, r, 5, (ar * nw.x + ai * nw.y) / dw, -((ai * nw.x - ar * nw.y) / dw));
+  const double num = lane == 0 ? ar : lane == 1 ? ai : lane == 2 ? ar * nw.x + ai * nw.y : ai * nw.x - ar * nw.y;
+  const double q = num / (lane < 2 ? nvj : dw);
+  const double im = __shfl_down_sync(0xffffffffu, q, 1);
+  if (lane == 0) {
+    a.c.alp[co] = make_double2(ar, ai);
+    st_scal<P>(a.scal, r, 4, q, im);
+  }
+  if (lane == 2) st_scal<P>(a.scal, r, 5, q, -im);
 }
 
 template <class P, int MODE, int BS>
@@ -782,9 +802,8 @@ __global__ void __launch_bounds__(BS, step_min_blocks<P, BS>()) k_step(StepArgs 
   }
   A v2[2] = {dot.re, dot.im};
   double tot[2];
-  if (reduce_last<2, BS>(v2, a.partials, a.counters, r, d.block0, sr.bx, d.nblk, tot) && threadIdx.x == 0) {
+  if (reduce_last<2, BS>(v2, a.partials, a.counters, r, d.block0, sr.bx, d.nblk, tot) && threadIdx.x < 32)
     finish_alpha<P, MODE>(a, r, co, tot);
-  }
 }
 
 // ------------------------------------------------------------ vector update
@@ -800,42 +819,64 @@ __global__ void __launch_bounds__(BS, step_min_blocks<P, BS>()) k_step(StepArgs 
 #else
 #define OV_UPDATE_BOUNDS(BS) __launch_bounds__(BS)
 #endif
-// beta_{j+1} and the next step's scalars from ||t_{j+1}||^2 (one thread)
+// beta_{j+1} and the next step's scalars from ||t_{j+1}||^2 (one warp)
 template <class P>
 __device__ __forceinline__ void finish_lanczos(const StepArgs& a, int r, size_t co, int j, double tot) {
+  const int lane = threadIdx.x & 31;
+  const double nvp = a.c.nv[co];
+  const double2 nwp = a.c.nw[co];
+  const int status = a.c.status[r];
   const double b = sqrt(tot);
   const double bprev = fabs(a.c.bet[co].x);
   const size_t cn = co + 1;
   const bool broke = !(b > a.breakdown_tol * (fabs(a.c.alp[co].x) + bprev));
-  if (broke && a.c.status[r] == kStOK) {
-    a.c.status[r] = kStLucky;
-    a.c.kbreak[r] = j;
+  const bool dead = broke || status != kStOK;
+  const double nv = dead ? 1.0 : b;
+  const double2 nw = make_double2(nv, 0.0), bg = make_double2(dead ? 0.0 : b, 0.0);
+  __syncwarp();
+  if (lane == 0) {
+    if (broke && status == kStOK) {
+      a.c.status[r] = kStLucky;
+      a.c.kbreak[r] = j;
+    }
+    a.c.nv[cn] = nv;
+    a.c.nw[cn] = nw;
+    a.c.bet[cn] = bg;
+    a.c.gam[cn] = bg;
   }
-  const bool dead = a.c.status[r] != kStOK;
-  a.c.nv[cn] = dead ? 1.0 : b;
-  a.c.nw[cn] = make_double2(dead ? 1.0 : b, 0.0);
-  a.c.bet[cn] = make_double2(dead ? 0.0 : b, 0.0);
-  a.c.gam[cn] = make_double2(dead ? 0.0 : b, 0.0);
-  set_step_scal<P>(a.scal, r, a.c.nv[cn], a.c.gam[cn], a.c.nw[cn], a.c.bet[cn], a.c.nv[co], a.c.nw[co]);
+  set_step_scal<P>(a.scal, r, nv, bg, nw, bg, nvp, nwp);
 }
-// beta_{j+1}, gamma_{j+1} and the next step's scalars from tw^dag t, ||t||^2, ||tw||^2 (one thread)
+// beta_{j+1}, gamma_{j+1} and the next step's scalars from tw^dag t, ||t||^2, ||tw||^2 (one warp)
 template <class P>
 __device__ __forceinline__ void finish_two_sided(const StepArgs& a, int r, size_t co, int j, const double (&tot)[4]) {
+  const int lane = threadIdx.x & 31;
+  const double nvp = a.c.nv[co];
+  const double2 nwp = a.c.nw[co];
+  const int status = a.c.status[r];
   const double dre = tot[0], dim = tot[1];
-  const double ad = sqrt(dre * dre + dim * dim);
+  const double root = sqrt(lane == 0 ? dre * dre + dim * dim : lane == 1 ? tot[2] : tot[3]);
+  const double ad = bcast(root, 0), nt = bcast(root, 1), nu = bcast(root, 2);
   const double b = sqrt(ad);
   const size_t cn = co + 1;
-  const bool broke = !(ad > a.breakdown_tol * sqrt(tot[2]) * sqrt(tot[3])) || !(b > 0.0);
-  if (broke && a.c.status[r] == kStOK) {
-    a.c.status[r] = kStBreakdown;
-    a.c.kbreak[r] = j;
+  const bool broke = !(ad > a.breakdown_tol * nt * nu) || !(b > 0.0);
+  const bool dead = broke || status != kStOK;
+  const double q = (lane == 0 ? dre : dim) / b;
+  const double2 g = make_double2(bcast(q, 0), bcast(q, 1));
+  const double nv = dead ? 1.0 : b;
+  const double2 nw = dead ? make_double2(1.0, 0.0) : g, be = make_double2(dead ? 0.0 : b, 0.0);
+  const double2 ga = dead ? make_double2(0.0, 0.0) : g;
+  __syncwarp();
+  if (lane == 0) {
+    if (broke && status == kStOK) {
+      a.c.status[r] = kStBreakdown;
+      a.c.kbreak[r] = j;
+    }
+    a.c.nv[cn] = nv;
+    a.c.nw[cn] = nw;
+    a.c.bet[cn] = be;
+    a.c.gam[cn] = ga;
   }
-  const bool dead = a.c.status[r] != kStOK;
-  a.c.nv[cn] = dead ? 1.0 : b;
-  a.c.nw[cn] = dead ? make_double2(1.0, 0.0) : make_double2(dre / b, dim / b);
-  a.c.bet[cn] = make_double2(dead ? 0.0 : b, 0.0);
-  a.c.gam[cn] = dead ? make_double2(0.0, 0.0) : make_double2(dre / b, dim / b);
-  set_step_scal<P>(a.scal, r, a.c.nv[cn], a.c.gam[cn], a.c.nw[cn], a.c.bet[cn], a.c.nv[co], a.c.nw[co]);
+  set_step_scal<P>(a.scal, r, nv, ga, nw, be, nvp, nwp);
 }
 __device__ __forceinline__ void advance_step(const StepArgs& a, int j) {
   // device-side step state: the last block of the launch advances j
@@ -901,15 +942,13 @@ __global__ void OV_UPDATE_BOUNDS(BS) k_update(StepArgs a) {
   if (MODE == kModeLanczos) {
     A v1[1] = {nvv};
     double tot[1];
-    if (reduce_last<1, BS>(v1, a.partials, a.counters, r, sr.d->block0, sr.bx, sr.d->nblk, tot) && threadIdx.x == 0) {
+    if (reduce_last<1, BS>(v1, a.partials, a.counters, r, sr.d->block0, sr.bx, sr.d->nblk, tot) && threadIdx.x < 32)
       finish_lanczos<P>(a, r, co, sp.j, tot[0]);
-    }
   } else {
     A v4[4] = {d.re, d.im, to_acc(nvl, A()), to_acc(nwl, A())};
     double tot[4];
-    if (reduce_last<4, BS>(v4, a.partials, a.counters, r, sr.d->block0, sr.bx, sr.d->nblk, tot) && threadIdx.x == 0) {
+    if (reduce_last<4, BS>(v4, a.partials, a.counters, r, sr.d->block0, sr.bx, sr.d->nblk, tot) && threadIdx.x < 32)
       finish_two_sided<P>(a, r, co, sp.j, tot);
-    }
   }
   advance_step(a, sp.j);
 }
@@ -952,31 +991,43 @@ __device__ __forceinline__ void hopping_wide(cx<df64>& up, cx<df64>& lo, const f
   const int V = g.V;
   const float2* __restrict__ links_lo = links + (size_t)36 * V;
   cxu au = {{0.f, 0.f}, {0.f, 0.f}}, al = au;
-#pragma unroll 1
-  for (int hop = 0; hop < 8; ++hop) {
+  // the next hop's operands are loaded while this one is computed
+  cx<float> un[3], uln[3];
+  cx<df64> pn[3], qn[3];
+  auto load = [&](int hop) {
     const int nu = hop >> 1;
     const bool fwd = (hop & 1) == 0;
     const int Ln = nu == 0 ? g.Lx : (nu == 1 ? g.Ly : (nu == 2 ? g.Lz : g.Lt));
     const int st = nu == 0 ? 1 : (nu == 1 ? g.Lx : (nu == 2 ? g.Lx * g.Ly : g.Lx * g.Ly * g.Lz));
     const int c = xc[0] * (nu == 0) + xc[1] * (nu == 1) + xc[2] * (nu == 2) + xc[3] * (nu == 3);
     const int sn = fwd ? (c == Ln - 1 ? s - (Ln - 1) * st : s + st) : (c == 0 ? s + (Ln - 1) * st : s - st);
-    const int ls = fwd ? s : sn;
-    cx<float> u[3], ulo[3];
+    const int ls = fwd ? s : sn, bs = c_bsrc[nu][sp];
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
       const int idx = fwd ? col * 3 + b : b * 3 + col;
-      u[b] = lconj(ld_link(links + (size_t)(nu * 9 + idx) * V + ls), !fwd);
-      ulo[b] = lconj(ld_link(links_lo + (size_t)(nu * 9 + idx) * V + ls), !fwd);
+      un[b] = ld_link(links + (size_t)(nu * 9 + idx) * V + ls);
+      uln[b] = ld_link(links_lo + (size_t)(nu * 9 + idx) * V + ls);
+      pn[b] = ld_vec(src + (size_t)(3 * sp + b) * V + sn);
+      qn[b] = ld_vec(src + (size_t)(3 * bs + b) * V + sn);
     }
-    const int bs = c_bsrc[nu][sp], bq = (c_bph[nu][sp] + (fwd ? 2 : 0)) & 3;
+  };
+  load(0);
+#pragma unroll 1
+  for (int hop = 0; hop < 8; ++hop) {
+    const int nu = hop >> 1;
+    const bool fwd = (hop & 1) == 0;
+    const int bq = (c_bph[nu][sp] + (fwd ? 2 : 0)) & 3;
+    cx<float> u[3], ulo[3];
     cx<df64> h[3];
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
-      const cx<df64> p = ld_vec(src + (size_t)(3 * sp + b) * V + sn);
-      const cx<df64> q = rot(ld_vec(src + (size_t)(3 * bs + b) * V + sn), bq);
+      u[b] = lconj(un[b], !fwd);
+      ulo[b] = lconj(uln[b], !fwd);
+      const cx<df64> p = pn[b], q = rot(qn[b], bq);
       const dfu re = add_u(to_u(p.re), to_u(q.re)), im = add_u(to_u(p.im), to_u(q.im));
       h[b] = {{re.hi, re.lo}, {im.hi, im.lo}};
     }
+    if (hop < 7) load(hop + 1);
     cxu gs;
     float cr = 0.f, ci = 0.f;
 #pragma unroll
@@ -1058,7 +1109,7 @@ __global__ void __launch_bounds__(6 * WS) k_step_wide(StepArgs a) {
   df64 v2[2] = {dot.re, dot.im};
   double tot[2];
   constexpr int sub = WideRef<WS>::sub;
-  if (reduce_last<2, 6 * WS>(v2, a.partials, a.counters, r, d.block0 * sub, sr.bx, d.nblk * sub, tot) && threadIdx.x == 0)
+  if (reduce_last<2, 6 * WS>(v2, a.partials, a.counters, r, d.block0 * sub, sr.bx, d.nblk * sub, tot) && threadIdx.x < 32)
     finish_alpha<P, MODE>(a, r, co, tot);
 }
 
@@ -1096,12 +1147,12 @@ __global__ void __launch_bounds__(6 * WS) k_update_wide(StepArgs a) {
   if (MODE == kModeLanczos) {
     df64 v1[1] = {nvv};
     double tot[1];
-    if (reduce_last<1, 6 * WS>(v1, a.partials, a.counters, r, part0, sr.bx, nblk, tot) && threadIdx.x == 0)
+    if (reduce_last<1, 6 * WS>(v1, a.partials, a.counters, r, part0, sr.bx, nblk, tot) && threadIdx.x < 32)
       finish_lanczos<P>(a, r, co, sp.j, tot[0]);
   } else {
     df64 v4[4] = {d.re, d.im, {nvl, 0.f}, {nwl, 0.f}};
     double tot[4];
-    if (reduce_last<4, 6 * WS>(v4, a.partials, a.counters, r, part0, sr.bx, nblk, tot) && threadIdx.x == 0)
+    if (reduce_last<4, 6 * WS>(v4, a.partials, a.counters, r, part0, sr.bx, nblk, tot) && threadIdx.x < 32)
       finish_two_sided<P>(a, r, co, sp.j, tot);
   }
   advance_step(a, sp.j);
