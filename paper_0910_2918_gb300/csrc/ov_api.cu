@@ -1510,7 +1510,7 @@ double ov::lattice_mass(const ov_handle* h, int q) { return h->lat[q].m_w + 4.0;
 
 // A fixed set of matvecs (one per item: lattice, sign of mu, offset of the vector in the
 // canonical block buffers), its problem descriptors and block map uploaded once; every run
-// is one pack, one stencil launch and one unpack over all items.
+// is one pack and one stencil launch over all items.
 struct ov::ApplySet {
   Buf desc, map;
   Batch bt{};
@@ -1592,14 +1592,13 @@ int ov::apply_set_run(ov_handle* h, const ApplySet* a, const double2* X, double2
   StepArgs sa{};
   sa.b = a->bt;
   sa.tv = h->tv.p;
-  sa.p = h->p.p;
+  sa.ycanon = Y;
   sa.dagger = 0;
   sa.c = c;
   CK(launch_step(h->prec, kModeApply, sa, st));
-  CK(launch_unpack(h->prec, a->bt, h->p.p, Y, st));
-  h->stats.launches += 3;
+  h->stats.launches += 2;
   h->stats.stencil_launches += 1;
-  h->stats.other_launches += 2;
+  h->stats.other_launches += 1;
   return OV_OK;
 }
 
@@ -1848,14 +1847,13 @@ extern "C" int ov_wilson_apply(ov_handle* h, int nrhs, const void* x, void* y, i
   StepArgs a{};
   a.b = bt;
   a.tv = h->tv.p;
-  a.p = h->p.p;
+  a.ycanon = yd;
   a.dagger = dagger ? 1 : 0;
   a.c = c;
   CK(launch_step(h->prec, kModeApply, a, st));
-  CK(launch_unpack(h->prec, bt, h->p.p, yd, st));
-  h->stats.launches += 3;
+  h->stats.launches += 2;
   h->stats.stencil_launches += 1;
-  h->stats.other_launches += 2;
+  h->stats.other_launches += 1;
   if (mem == OV_MEM_HOST) CK(cudaMemcpyAsync(y, yd, canon, cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   return OV_OK;

@@ -82,8 +82,9 @@ struct StepArgs {
   //   2: 1/conj(nw_j)                3: c_w = beta_j / conj(nw_{j-1})
   //   4: alpha_j / nv_j              5: conj(alpha_j) / conj(nw_j)
   void* scal;
-  const void* tv;  // apply mode: the source
-  void* p;         // A v_j - ..., and the apply mode's output
+  const void* tv;   // apply mode: the source
+  double2* ycanon;  // apply mode: the result, in the canonical layout
+  void* p;          // A v_j - ...
   void* r;         // A^dag w_j - ...
   // vectors of step j when jdev is NULL (the regeneration pass): t_j, t_{j-1} and the
   // destination of t_{j+1} (which may alias t_{j-1})
@@ -119,7 +120,6 @@ void fill_consts(ProbDesc& d, double m_w, double mu);
 // the step-1 scalars
 cudaError_t launch_pack(int prec, const Batch& b, const double2* xcanon, void* xint, void* xint2, Coefs c,
                         double* partials, unsigned* counters, int want_norm, void* scal, cudaStream_t st);
-cudaError_t launch_unpack(int prec, const Batch& b, const void* xint, double2* ycanon, cudaStream_t st);
 cudaError_t launch_step(int prec, int mode, const StepArgs& a, cudaStream_t st);
 cudaError_t launch_update(int prec, int mode, const StepArgs& a, cudaStream_t st);
 // y_r = scale_r * sum_{j<k_r} c[r][j+1] v_{r,j+1} (+ x_r and gamma5 if add_x); slots[j] is
@@ -215,7 +215,7 @@ double lattice_mu(const ov_handle* h, int q);
 double lattice_mass(const ov_handle* h, int q);  // m_w + 4
 // Fixed sets of matvecs in the handle's arithmetic: item r computes Y[voff..] = A X[voff..]
 // for 12 V entries of lattice q at mu (neg = 0) or at -mu (neg = 1: A(-mu) = A^dag); X and Y
-// are canonical complex-double buffers of `pool` entries. One run = three launches.
+// are canonical complex-double buffers of `pool` entries. One run = two launches.
 struct ApplyItem {
   int q, neg;
   size_t voff;

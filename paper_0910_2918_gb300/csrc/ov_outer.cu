@@ -232,28 +232,78 @@ __device__ __forceinline__ SiteRef site_ref(const Batch& b) {
 }
 
 
-// ------------------------------------------------------------ pack / unpack
+// ------------------------------------------------------------ canonical buffers
+// The canonical layout keeps a site's twelve numbers together (192 bytes), a warp's sites in
+// one run. Read or written thread by thread, an instruction touches 32 places 192 bytes apart
+// (12 x 16^4 in float: pack 73 us, unpack 86 us for 226 MB each); a warp moves them through
+// shared memory instead, sixteen sites at a time, in 512-byte pieces (pack 55 us; the matvec
+// writes its result this way itself, 110 -> 112 us, without a pass to unpack it).
+constexpr int kCanonPitch = 13;  // of a site in shared memory: odd, so that lanes meet no bank twice
+template <int BS>
+struct CanonSmem {
+  double2 v[BS / 32][16 * kCanonPitch];
+};
+// z = the numbers of the lane's site; base: the problem's canonical entries, w0: the warp's
+// first site (whole warps call)
+__device__ __forceinline__ void canon_load(const double2* __restrict__ base, int V, int w0, double2* sm, double2 (&z)[12]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int half = 0; half < 2; ++half) {
+    const int s0 = w0 + 16 * half, n = min(max(V - s0, 0), 16) * 12;
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+      const int e = lane + 32 * q;
+      if (e < n) sm[e / 12 * kCanonPitch + e % 12] = base[(size_t)s0 * 12 + e];
+    }
+    __syncwarp();
+    if ((lane >> 4) == half)
+#pragma unroll
+      for (int k = 0; k < 12; ++k) z[k] = sm[(lane & 15) * kCanonPitch + k];
+  }
+}
+__device__ __forceinline__ void canon_store(double2* base, int V, int w0, double2* sm, const double2 (&z)[12]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int half = 0; half < 2; ++half) {
+    const int s0 = w0 + 16 * half, n = min(max(V - s0, 0), 16) * 12;
+    __syncwarp();
+    if ((lane >> 4) == half)
+#pragma unroll
+      for (int k = 0; k < 12; ++k) sm[(lane & 15) * kCanonPitch + k] = z[k];
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+      const int e = lane + 32 * q;
+      if (e < n) base[(size_t)s0 * 12 + e] = sm[e / 12 * kCanonPitch + e % 12];
+    }
+  }
+}
+
 template <class P, int BS>
 __global__ void __launch_bounds__(BS) k_pack(Batch bt, const double2* __restrict__ x, typename P::vec_t* xi,
                                                  typename P::vec_t* xi2, Coefs c, double* partials,
                                                  unsigned* counters, int want_norm, void* scal) {
   using R = typename P::R;
+  __shared__ CanonSmem<BS> sm;
   const SiteRef sr = site_ref<BS>(bt);
   const int s = sr.s, r = sr.r;
   const int V = sr.d->g.V;
   const size_t voff = sr.d->voff;
+  double2 z[12];
+  canon_load(x + voff, V, s - (int)(threadIdx.x & 31), sm.v[threadIdx.x >> 5], z);
   double n2 = 0.0;
   if (sr.active) {
-    const double2* src = x + voff + (size_t)s * 12;
     typename P::vec_t* dst = xi + voff + s;
     typename P::vec_t* dst2 = xi2 ? xi2 + voff + s : nullptr;
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
-      double2 z = src[k];
-      n2 = fma(z.x, z.x, fma(z.y, z.y, n2));
-      st_vec(dst + (size_t)k * V, cd_to<R>(z.x, z.y));
-      if (dst2) st_vec(dst2 + (size_t)k * V, cd_to<R>(z.x, z.y));
+      st_vec(dst + (size_t)k * V, cd_to<R>(z[k].x, z[k].y));
+      if (dst2) st_vec(dst2 + (size_t)k * V, cd_to<R>(z[k].x, z[k].y));
     }
+    if (want_norm)
+#pragma unroll
+      for (int k = 0; k < 12; ++k) n2 = fma(z[k].x, z[k].x, fma(z[k].y, z[k].y, n2));
   }
   if (!want_norm) return;
   double v[1] = {n2}, tot[1];
@@ -270,20 +320,6 @@ __global__ void __launch_bounds__(BS) k_pack(Batch bt, const double2* __restrict
       c.kbreak[r] = 0;
     }
     if (scal) set_step_scal<P>(scal, r, n1, zero, w1, zero, 1.0, make_double2(1.0, 0.0));
-  }
-}
-
-template <class P, int BS>
-__global__ void __launch_bounds__(BS) k_unpack(Batch bt, const typename P::vec_t* __restrict__ xi, double2* y) {
-  const SiteRef sr = site_ref<BS>(bt);
-  if (!sr.active) return;
-  const int V = sr.d->g.V;
-  const typename P::vec_t* src = xi + sr.d->voff + sr.s;
-  double2* dst = y + sr.d->voff + (size_t)sr.s * 12;
-#pragma unroll
-  for (int k = 0; k < 12; ++k) {
-    cx<double> z = vec_to_cd(ld_vec(src + (size_t)k * V));
-    dst[k] = make_double2(z.re, z.im);
   }
 }
 
@@ -737,13 +773,18 @@ __global__ void __launch_bounds__(BS, step_min_blocks<P, BS>()) k_step(StepArgs 
   cx<R> acc[12];
 
   if (MODE == kModeApply) {
+    __shared__ CanonSmem<BS> sm;
+    double2 z[12];
     if (active) {
       const V_t* tv = (const V_t*)a.tv + vo;
       hopping<P>(acc, tv, links, g, s, xc, a.dagger ? emui : emu, a.dagger ? emu : emui);
-      V_t* out = (V_t*)a.p + vo + s;
 #pragma unroll
-      for (int k = 0; k < 12; ++k) st_vec(out + (size_t)k * g.V, g5d(k, ld_vec(tv + (size_t)k * g.V + s), acc[k], mass));
+      for (int k = 0; k < 12; ++k) {
+        const cx<double> d = vec_to_cd(g5d(k, ld_vec(tv + (size_t)k * g.V + s), acc[k], mass));
+        z[k] = make_double2(d.re, d.im);
+      }
     }
+    canon_store(a.ycanon + vo, g.V, s - (int)(threadIdx.x & 31), sm.v[threadIdx.x >> 5], z);
     return;
   }
 
@@ -963,7 +1004,8 @@ __global__ void OV_UPDATE_BOUNDS(BS) k_update(StepArgs a) {
 // the three colours: a third more work in all) and owns two of the twelve components, upper
 // spin `sp` and lower spin 2 + sp of its colour; the lower one takes its own or the other half
 // warp's product, by a shuffle. The sums of a component keep their order. A block takes WS
-// consecutive sites of a 64-site block of the map. MEASURED_WIDE
+// consecutive sites of a 64-site block of the map. Step on 8^4 45 -> 18 us, 4^4 (mu = 0) 37 -> 16
+// us; 24 lattices of 57,000 sites in all 96 -> 128 us, so the tuner decides.
 __device__ __forceinline__ dfu shfl_half(dfu v) {
   return {__shfl_xor_sync(0xffffffffu, v.hi, 16), __shfl_xor_sync(0xffffffffu, v.lo, 16)};
 }
@@ -1076,9 +1118,11 @@ __global__ void __launch_bounds__(6 * WS) k_step_wide(StepArgs a) {
     const float4* tv = (const float4*)a.tv + vo;
     hopping_wide(up, lo, tv, (const float2*)d.links, g, ss, xc, a.dagger ? emui : emu, a.dagger ? emu : emui, sr.col, sr.sp);
     if (!sr.active) return;
-    float4* out = (float4*)a.p + vo + ss;
-    st_vec(out + (size_t)k0 * V, g5d(k0, ld_vec(tv + (size_t)k0 * V + ss), up, mass));
-    st_vec(out + (size_t)k1 * V, g5d(k1, ld_vec(tv + (size_t)k1 * V + ss), lo, mass));
+    double2* out = a.ycanon + vo + (size_t)ss * 12;
+    const cx<double> z0 = vec_to_cd(g5d(k0, ld_vec(tv + (size_t)k0 * V + ss), up, mass));
+    const cx<double> z1 = vec_to_cd(g5d(k1, ld_vec(tv + (size_t)k1 * V + ss), lo, mass));
+    out[k0] = make_double2(z0.re, z0.im);
+    out[k1] = make_double2(z1.re, z1.im);
     return;
   }
   const StepPtrs sp = step_ptrs(a);
@@ -1159,42 +1203,63 @@ __global__ void __launch_bounds__(6 * WS) k_update_wide(StepArgs a) {
 }
 
 // ------------------------------------------------------------ recombination
-template <class P, int BS>
+// scale z (+ x, gamma5) for components k0 .. k0 + NC - 1
+template <int NC, class AT>
+__device__ __forceinline__ void finish_site(const cx<AT> (&acc)[NC], int k0, double sc, int add_x, const double2 (&xs)[NC],
+                                            double2 (&out)[NC]) {
+#pragma unroll
+  for (int k = 0; k < NC; ++k) {
+    cx<double> z = acc_to_cd(acc[k]);
+    z.re *= sc;
+    z.im *= sc;
+    if (add_x) {
+      if (k0 + k >= 6) { z.re = -z.re; z.im = -z.im; }
+      z.re += xs[k].x;
+      z.im += xs[k].y;
+    }
+    out[k] = make_double2(z.re, z.im);
+  }
+}
+
+// NC = 12: a thread sums the whole site (bound by HBM: the stored basis is read once; two steps
+// unrolled 8.7 ms for 12 x 16^4 at k = 350, one 14.1, four 9.6; one or three components a thread
+// 8.9 to 10.0). NC = 1: one component (blockIdx.y) a thread, for lattices with few sites, where
+// the site's thread ran k times twelve dependent sums (4^4, k = 170: 0.30 -> 0.10 ms)
+template <class P, int BS, int NC>
 __global__ void __launch_bounds__(BS) k_recombine(Batch bt, const void* const* __restrict__ slots,
                                                       const typename AccOf<P>::st* __restrict__ cacc, int ldc,
                                                       const int* __restrict__ kr, const double* __restrict__ scale,
                                                       const double2* __restrict__ x, int add_x, double2* y) {
   using AT = typename AccOf<P>::A;
   const SiteRef sr = site_ref<BS>(bt);
-  if (!sr.active) return;
-  const int s = sr.s, r = sr.r, V = sr.d->g.V;
+  const int s = sr.s, r = sr.r, V = sr.d->g.V, k0 = NC == 12 ? 0 : blockIdx.y;
   const size_t vo = sr.d->voff;
-  cx<AT> acc[12];
+  cx<AT> acc[NC];
 #pragma unroll
-  for (int k = 0; k < 12; ++k) acc[k] = czero<AT>();
-  const int k_r = kr[r];
+  for (int k = 0; k < NC; ++k) acc[k] = czero<AT>();
+  const int k_r = sr.active ? kr[r] : 0;
   const typename AccOf<P>::st* cr = cacc + (size_t)r * ldc;
+#pragma unroll(NC == 12 ? 2 : 8)
   for (int j = 0; j < k_r; ++j) {
     const cx<AT> cj = ld_acc(cr + j + 1);
-    const typename P::vec_t* vj = (const typename P::vec_t*)slots[j] + vo + s;
+    const typename P::vec_t* vj = (const typename P::vec_t*)slots[j] + vo + (size_t)k0 * V + s;
 #pragma unroll
-    for (int k = 0; k < 12; ++k) acc_axpy(acc[k], cj, ld_vec(vj + (size_t)k * V));
+    for (int k = 0; k < NC; ++k) acc_axpy(acc[k], cj, ld_vec(vj + (size_t)k * V));
   }
   const double sc = scale[r];
-  double2* dst = y + vo + (size_t)s * 12;
-  const double2* xs = x + vo + (size_t)s * 12;
-#pragma unroll
-  for (int k = 0; k < 12; ++k) {
-    cx<double> z = acc_to_cd(acc[k]);
-    z.re *= sc;
-    z.im *= sc;
-    if (add_x) {
-      const double2 xv = xs[k];
-      if (k >= 6) { z.re = -z.re; z.im = -z.im; }
-      z.re += xv.x;
-      z.im += xv.y;
-    }
-    dst[k] = make_double2(z.re, z.im);
+  double2 xs[NC], out[NC];
+  if constexpr (NC == 12) {
+    __shared__ CanonSmem<BS> sm;
+    double2* w = sm.v[threadIdx.x >> 5];
+    const int w0 = s - (int)(threadIdx.x & 31);
+    if (add_x) canon_load(x + vo, V, w0, w, xs);
+    finish_site<NC>(acc, 0, sc, add_x, xs, out);
+    canon_store(y + vo, V, w0, w, out);
+  } else if (sr.active) {
+    const size_t o = vo + (size_t)s * 12 + k0;
+    if (add_x) xs[0] = x[o];
+    finish_site<NC>(acc, k0, sc, add_x, xs, out);
+    y[o] = out[0];
   }
 }
 
@@ -1202,26 +1267,19 @@ template <class P, int BS>
 __global__ void __launch_bounds__(BS) k_finish_acc(Batch bt, const typename AccOf<P>::st* __restrict__ yacc,
                                                        const double* __restrict__ scale,
                                                        const double2* __restrict__ x, int add_x, double2* y) {
+  using AT = typename AccOf<P>::A;
+  __shared__ CanonSmem<BS> sm;
   const SiteRef sr = site_ref<BS>(bt);
-  if (!sr.active) return;
-  const int s = sr.s, r = sr.r, V = sr.d->g.V;
+  const int s = sr.s, V = sr.d->g.V, w0 = s - (int)(threadIdx.x & 31);
   const size_t vo = sr.d->voff;
-  const double sc = scale[r];
-  double2* dst = y + vo + (size_t)s * 12;
-  const double2* xs = x + vo + (size_t)s * 12;
+  double2* w = sm.v[threadIdx.x >> 5];
+  double2 xs[12], out[12];
+  if (add_x) canon_load(x + vo, V, w0, w, xs);
+  cx<AT> acc[12];
 #pragma unroll
-  for (int k = 0; k < 12; ++k) {
-    cx<double> z = acc_to_cd(ld_acc(yacc + vo + (size_t)k * V + s));
-    z.re *= sc;
-    z.im *= sc;
-    if (add_x) {
-      const double2 xv = xs[k];
-      if (k >= 6) { z.re = -z.re; z.im = -z.im; }
-      z.re += xv.x;
-      z.im += xv.y;
-    }
-    dst[k] = make_double2(z.re, z.im);
-  }
+  for (int k = 0; k < 12; ++k) acc[k] = sr.active ? ld_acc(yacc + vo + (size_t)k * V + s) : czero<AT>();
+  finish_site<12>(acc, 0, scale[sr.r], add_x, xs, out);
+  canon_store(y + vo, V, w0, w, out);
 }
 
 // ------------------------------------------------------------ launchers
@@ -1253,12 +1311,6 @@ cudaError_t launch_pack(int prec, const Batch& b, const double2* x, void* xi, vo
   OV_BS_DISPATCH(b.block, OV_DISPATCH(prec, (k_pack<P, BS><<<b.nblocks, BS, 0, st>>>(
                                                 b, x, (typename P::vec_t*)xi, (typename P::vec_t*)xi2, c, partials,
                                                 counters, want_norm, scal))));
-  return cudaGetLastError();
-}
-
-cudaError_t launch_unpack(int prec, const Batch& b, const void* xi, double2* y, cudaStream_t st) {
-  OV_BS_DISPATCH(b.block, OV_DISPATCH(prec, (k_unpack<P, BS><<<b.nblocks, BS, 0, st>>>(
-                                                b, (const typename P::vec_t*)xi, y))));
   return cudaGetLastError();
 }
 
@@ -1324,7 +1376,15 @@ cudaError_t launch_update(int prec, int mode, const StepArgs& a, cudaStream_t st
 cudaError_t launch_recombine(int prec, const Batch& b, const void* const* slots, const void* cacc, int ldc,
                              const int* k_dev, const double* scale, const double2* x, int add_x, double2* y,
                              cudaStream_t st) {
-  OV_BS_DISPATCH(b.block, OV_DISPATCH(prec, (k_recombine<P, BS><<<b.nblocks, BS, 0, st>>>(
+  // one component a thread while that leaves the GPU with less than its threads twice
+  if (b.nblocks * b.block <= 2 * 152 * 2048 / 12) {
+    const dim3 grid(b.nblocks, 12);
+    OV_BS_DISPATCH(b.block, OV_DISPATCH(prec, (k_recombine<P, BS, 1><<<grid, BS, 0, st>>>(
+                                                  b, slots, (const typename AccOf<P>::st*)cacc, ldc, k_dev, scale, x,
+                                                  add_x, y))));
+    return cudaGetLastError();
+  }
+  OV_BS_DISPATCH(b.block, OV_DISPATCH(prec, (k_recombine<P, BS, 12><<<b.nblocks, BS, 0, st>>>(
                                                 b, slots, (const typename AccOf<P>::st*)cacc, ldc, k_dev, scale, x,
                                                 add_x, y))));
   return cudaGetLastError();
