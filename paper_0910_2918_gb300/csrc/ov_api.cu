@@ -83,9 +83,10 @@ struct TuneKey {
     return prec != o.prec ? prec < o.prec : (mode != o.mode ? mode < o.mode : nprob < o.nprob);
   }
 };
-// threads per site block, and sites per block of the wide kernels (0: not used)
+// threads per site block, sites per block of the wide kernels (0: not used), and whether runs
+// of steps go to k_steps in one launch
 struct Tuned {
-  int bs, wide;
+  int bs, wide, coop;
 };
 
 // one gauge field with its operator parameters
@@ -127,6 +128,7 @@ struct ov_handle {
   std::map<TuneKey, Tuned> tuned;  // autotuned kernels per (precision or relaxed, mode, problem count)
   // CUDA graph of graph_steps outer steps (captured on a private stream, replayed on st)
   Buf jstate, slot_tab;
+  Buf bars;  // k_steps: a barrier counter per problem, then the word that reports a wait that ran out
   cudaStream_t cap_st = nullptr;
   // stopping checks overlapped with speculative outer steps: a high-priority stream and
   // the events that order it against the handle's stream
@@ -507,6 +509,7 @@ extern "C" void ov_destroy(ov_handle* h) {
   if (h->chk_host) cudaFreeHost(h->chk_host);
   release(h->jstate);
   release(h->slot_tab);
+  release(h->bars);
   delete h;
 }
 
@@ -527,7 +530,7 @@ static int ensure_outer(ov_handle* h, int nrhs, int ld, size_t pool, int nblocks
   CK(grow(h->coef_nv, sizeof(double) * (size_t)nrhs * ld));
   CK(grow(h->coef_status, sizeof(int) * nrhs));
   CK(grow(h->coef_kbreak, sizeof(int) * nrhs));
-  CK(grow(h->partials, sizeof(double) * 4 * (size_t)nblocks));
+  CK(grow(h->partials, sizeof(double) * 8 * (size_t)nblocks));
   if (h->counters.bytes < sizeof(unsigned) * nrhs) {
     CK(grow(h->counters, sizeof(unsigned) * nrhs));
     CK(cudaMemsetAsync(h->counters.p, 0, sizeof(unsigned) * nrhs, h->st));
@@ -737,13 +740,14 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
   // tuned below at the first step
   const bool relaxing = !strict_only && o.relax > 0.0 && h->prec == OV_PREC_DF64;
   const TuneKey key{relaxing ? kPrecDF64Relaxed : h->prec, mode, nrhs};
-  int bs = o.block_size, wide = 0;
+  int bs = o.block_size, wide = 0, coop = 0;
   bool tune = false;
   if (bs == 0) {
     auto it = h->tuned.find(key);
     if (it != h->tuned.end()) {
       bs = it->second.bs;
       wide = it->second.wide;
+      coop = it->second.coop;
     } else {
       bs = kBlockDefault;
       tune = true;
@@ -837,6 +841,8 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
     CK(grow(h->jstate, sizeof(int) * 2));
     CK(cudaMemcpyAsync(h->jstate.p, init, sizeof(int) * 2, cudaMemcpyHostToDevice, st));
     CK(grow(h->slot_tab, sizeof(void*) * (size_t)(ktarget + 2)));
+    CK(grow(h->bars, sizeof(unsigned) * (nrhs + 1)));
+    CK(cudaMemsetAsync(h->bars.p, 0, sizeof(unsigned) * (nrhs + 1), st));
   }
   a.jdev = (int*)h->jstate.p;
   a.gticket = (unsigned*)((int*)h->jstate.p + 1);
@@ -900,12 +906,12 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
         CK(cudaEventCreate(&e0));
         CK(cudaEventCreate(&e1));
         float best = 1e30f;
-        Tuned best_t{kBlockDefault, 0};
-        std::vector<Tuned> cands = {{64, 0}, {128, 0}, {256, 0}};
+        Tuned best_t{kBlockDefault, 0, 0};
+        std::vector<Tuned> cands = {{64, 0, 0}, {128, 0, 0}, {256, 0, 0}};
         if (h->prec == OV_PREC_DF64 && !relaxing && pool / 12 <= kWideSites) {
           int nb64 = 0;
           for (int q : lat_of) nb64 += num_site_blocks(h->lat[q].g, 64);
-          cands.push_back({64, wide_sites(nb64)});
+          cands.push_back({64, wide_sites(nb64), 4 * nb64 <= steps_capacity(mode) ? 1 : 0});
         }
         for (const Tuned& cand : cands) {
           Batch bc;
@@ -933,11 +939,22 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
         rc = build_batch(h, lat_of, best_t.bs, &bt, &pool, neg_mu);
         if (rc != OV_OK) return rc;
         bt.wide = best_t.wide;
+        coop = best_t.coop;
         a.b = bt;
-        if (h->trace) fprintf(stderr, "{\"ov_autotune\": %d, \"wide\": %d, \"ms\": %.4f}\n", best_t.bs, best_t.wide, best);
+        if (h->trace) fprintf(stderr, "{\"ov_autotune\": %d, \"wide\": %d, \"one_launch\": %d, \"ms\": %.4f}\n", best_t.bs, best_t.wide, best_t.coop, best);
       }
       h->stats.block_size = a.b.block;
       // steps jn..jto: whole graph units replayed, the rest launched one by one
+      if (coop && gU > 0) {
+        // every block fits the GPU at once: the whole span in one launch
+        const int nst = jto - jn + 1;
+        CK(launch_steps(mode, a, nst, (unsigned*)h->bars.p, (int*)h->bars.p + nrhs, st));
+        h->stats.launches += 1;
+        h->stats.stencil_launches += nst;
+        h->stats.update_launches += nst;
+        h->stats.outer_steps += nst;
+        jn = jto + 1;
+      }
       while (jn <= jto) {
         const int sp = step_prec(jn);
         // a graph unit holds steps of one precision
@@ -1392,7 +1409,9 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
   tstop(h, tr);
   tstop(h, t_total);
   if (mem == OV_MEM_HOST) CK(cudaMemcpyAsync(y, yd, canon, cudaMemcpyDeviceToHost, st));
+  if (coop) CK(cudaMemcpyAsync(h->chk_host, (int*)h->bars.p + nrhs, sizeof(int), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
+  if (coop && *(const int*)h->chk_host != 0) return OV_ERR_CUDA;
   tcollect(h);
   int worst = OV_OK;
   for (int r = 0; r < nrhs; ++r) {

@@ -121,6 +121,11 @@ void fill_consts(ProbDesc& d, double m_w, double mu);
 cudaError_t launch_pack(int prec, const Batch& b, const double2* xcanon, void* xint, void* xint2, Coefs c,
                         double* partials, unsigned* counters, int want_norm, void* scal, cudaStream_t st);
 cudaError_t launch_step(int prec, int mode, const StepArgs& a, cudaStream_t st);
+// nsteps outer steps in one cooperative launch (strict double-float, a.b.block = 64; bars: a zeroed
+// counter per problem that all launches of an apply share, *err: set if a wait ran out); it must
+// not have more blocks (four per site block) than steps_capacity(mode)
+int steps_capacity(int mode);
+cudaError_t launch_steps(int mode, const StepArgs& a, int nsteps, unsigned* bars, int* err, cudaStream_t st);
 cudaError_t launch_update(int prec, int mode, const StepArgs& a, cudaStream_t st);
 // y_r = scale_r * sum_{j<k_r} c[r][j+1] v_{r,j+1} (+ x_r and gamma5 if add_x); slots[j] is
 // the device address of basis slot j (a vector pool)

@@ -1026,7 +1026,14 @@ __device__ __forceinline__ WideRef<WS> wide_ref(const Batch& b) {
   return {m.x, bx, s, warp % 3, (int)(threadIdx.x >> 4) & 1, s < d->g.V, d};
 }
 
-// the hopping sum of hopping_df for components 3 sp + col (up) and 6 + 3 sp + col (lo)
+// the hopping sum of hopping_df for components 3 sp + col (up) and 6 + 3 sp + col (lo). CG: the
+// vector is read past the L1 cache (other blocks of the same launch write it)
+template <bool CG>
+__device__ __forceinline__ cx<df64> ld_vec_wide(const float4* p) {
+  const float4 v = CG ? __ldcg(p) : *p;
+  return ld_vec(&v);
+}
+template <bool CG = false>
 __device__ __forceinline__ void hopping_wide(cx<df64>& up, cx<df64>& lo, const float4* __restrict__ src,
                                              const float2* __restrict__ links, const Geometry& g, int s,
                                              const int (&xc)[4], df64 ef, df64 eb, int col, int sp) {
@@ -1049,8 +1056,8 @@ __device__ __forceinline__ void hopping_wide(cx<df64>& up, cx<df64>& lo, const f
       const int idx = fwd ? col * 3 + b : b * 3 + col;
       un[b] = ld_link(links + (size_t)(nu * 9 + idx) * V + ls);
       uln[b] = ld_link(links_lo + (size_t)(nu * 9 + idx) * V + ls);
-      pn[b] = ld_vec(src + (size_t)(3 * sp + b) * V + sn);
-      qn[b] = ld_vec(src + (size_t)(3 * bs + b) * V + sn);
+      pn[b] = ld_vec_wide<CG>(src + (size_t)(3 * sp + b) * V + sn);
+      qn[b] = ld_vec_wide<CG>(src + (size_t)(3 * bs + b) * V + sn);
     }
   };
   load(0);
@@ -1200,6 +1207,284 @@ __global__ void __launch_bounds__(6 * WS) k_update_wide(StepArgs a) {
       finish_two_sided<P>(a, r, co, sp.j, tot);
   }
   advance_step(a, sp.j);
+}
+
+// ------------------------------------------------------------ runs of steps in one launch
+// On lattices whose blocks all fit the SMs at once, two launches a step cost more than the
+// step's work (4^4: 20 us a step, of which the launches, the pointers read from memory, the
+// tickets and the coefficients' finishing took most). k_steps runs `nsteps` outer steps in one
+// cooperative launch: a block of the wide layout holds both sides of its sites (threads 0 .. 95
+// the v side, the rest the w side), keeps its own entries of t_j, t_{j-1}, p (and r) in
+// registers and exchanges what the dot products need through shared memory; only the new
+// vectors go to memory, for the neighbours. The two reductions of a step are barriers over the
+// problem's blocks, after which every block adds the partial sums itself, in the same order, and
+// forms the coefficients (block 0 of the problem stores them). A barrier's wait is bounded: when
+// it runs out the block sets *err and returns, and so do the others. A step on 4^4 (mu = 0) 20 ->
+// 15 us, on 8^4 (mu = 0.3) 25 -> 23 us, half of it the two barriers and the double arithmetic of
+// the coefficients between them.
+constexpr int kBarSpins = 1 << 22;  // polls of one barrier, a second or so
+__device__ __forceinline__ bool problem_barrier(unsigned* bar, unsigned nblk, int* err, int* s_fail) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const unsigned t = atomicAdd(bar, 1u), target = (t / nblk + 1u) * nblk;
+    int n = 0;
+    for (;;) {
+      unsigned v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+      if ((int)(v - target) >= 0) break;
+      if (++n > kBarSpins) {
+        *err = 1;
+        *s_fail = 1;
+        break;
+      }
+    }
+    __threadfence();
+  }
+  __syncthreads();
+  return *s_fail == 0;
+}
+// the problem's total of NQ partial sums a block, in warp 0, in block order by lanes
+template <int NQ>
+__device__ __forceinline__ void problem_total(const double* part, int nblk, double (&tot)[NQ]) {
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) tot[q] = 0.0;
+  for (int b = threadIdx.x; b < nblk; b += 32)
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) tot[q] += __ldcg(part + (size_t)b * 4 + q);
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) tot[q] = warp_sum(tot[q]);
+}
+// a block's sums of NQ values over warps [w0, w1), stored as its partial sums (all threads call)
+template <int NQ>
+__device__ __forceinline__ void block_partial(df64 (&v)[NQ], int w1, double* out) {
+  __shared__ float2 s[6][4];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    v[q] = warp_sum(v[q]);
+    if (lane == 0) s[warp][q] = make_float2(v[q].hi, v[q].lo);
+  }
+  __syncthreads();
+  if (threadIdx.x < NQ) {
+    df64 t = df_zero();
+    for (int w = 0; w < w1; ++w) t = t + df64{s[w][threadIdx.x].x, s[w][threadIdx.x].y};
+    __stcg(out + threadIdx.x, df_to_double(t));
+  }
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(MODE == kModeTwoSided ? 192 : 96) k_steps(StepArgs a, int nsteps, unsigned* bars, int* err) {
+  constexpr bool TWO = MODE == kModeTwoSided;
+  constexpr int WS = 16, sub = 4, NW = TWO ? 6 : 3;
+  __shared__ float4 s_x[96 * 2];          // the w side's entries, for the v side's dot products
+  __shared__ float4 s_scal[6];            // the step scalars of StepArgs::scal
+  __shared__ int s_fail;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int side = TWO ? tid / 96 : 0, t96 = tid % 96;
+  const int2 m = __ldg(&a.b.blk_map[blockIdx.x / sub]);
+  const int r = m.x, bx = m.y * sub + blockIdx.x % sub;
+  const ProbDesc& d = a.b.desc[r];
+  const Geometry g = d.g;
+  const int V = g.V, s = bx * WS + (lane & 15), sp2 = (lane >> 4) & 1, col = warp % 3;
+  const bool active = s < V;
+  const int ss = active ? s : 0;
+  const size_t vo = d.voff;
+  const int nblk = d.nblk * sub;
+  const bool lead = bx == 0;
+  double* const pa = a.partials + (size_t)d.block0 * sub * 4;                       // alpha's partial sums
+  double* const pd = pa + (size_t)a.b.nblocks * sub * 4;                            // beta's and gamma's
+  const df64 mass = {d.mass_hl[0], d.mass_hl[1]}, emu = {d.emu_hl[0], d.emu_hl[1]}, emui = {d.emui_hl[0], d.emui_hl[1]};
+  const df64 ef = side == 0 ? emu : emui, eb = side == 0 ? emui : emu;
+  int xc[4];
+  site_coords(g, ss, xc[0], xc[1], xc[2], xc[3]);
+  const int kk[2] = {3 * sp2 + col, 6 + 3 * sp2 + col};  // this thread's components
+  const int j0 = __ldcg(a.jdev);
+  if (tid == 0) s_fail = 0;
+  if (tid < 4) s_scal[tid] = __ldcg((const float4*)a.scal + (size_t)r * 8 + tid);
+  size_t co = (size_t)r * a.c.ld + j0;
+  double nvj = a.c.nv[co];
+  double2 nwj = a.c.nw[co], betj = a.c.bet[co];
+  int status = a.c.status[r];
+  StepPtrs sp = step_ptrs(a);
+  const float4* src = (const float4*)(side == 0 ? sp.tc : sp.wc) + vo;
+  cx<df64> cur[2], prv[2];
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const size_t o = (size_t)kk[q] * V + ss;
+    cur[q] = ld_vec_wide<true>(src + o);
+    prv[q] = ld_vec_wide<true>((const float4*)(side == 0 ? sp.tp : sp.wp) + vo + o);
+  }
+  for (int i = 0; i < nsteps; ++i, ++co) {
+    const int j = j0 + i;
+    // the destination of t_{j+1} (the w side's ring: tw_{j+1} over tw_{j-1})
+    float4* dst;
+    if (side == 1) dst = (float4*)((char*)a.wring + a.pool_bytes * ((j + 1) & 1)) + vo;
+    else dst = (a.slot_tab ? (float4*)a.slot_tab[j] : (float4*)((char*)a.vring + a.pool_bytes * ((j + 1) & 1))) + vo;
+    if (TWO && side == 1) {
+      st_vec(&s_x[t96], cur[0]);
+      st_vec(&s_x[96 + t96], cur[1]);
+    }
+    __syncthreads();  // s_x, s_scal
+    const cx<df64> scl = ld_vec(&s_scal[2 * side]), cf = ld_vec(&s_scal[2 * side + 1]);
+    cx<df64> up, lo, ok[2];
+    hopping_wide<true>(up, lo, src, (const float2*)d.links, g, ss, xc, ef, eb, col, sp2);
+    cx<df64> dot = {df_zero(), df_zero()};
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const cx<df64> h = g5d(kk[q], cur[q], q == 0 ? up : lo, mass);
+      if (!TWO) ok[q] = smulsub<true, true>(scl, h, cf, prv[q]);
+      else if (side == 0) ok[q] = smulsub<true, false>(scl, h, cf, prv[q]);
+      else ok[q] = smulsub<false, false>(scl, h, cf, prv[q]);
+      if (active && side == 0) acc_dot(dot, TWO ? ld_vec(&s_x[96 * q + t96]) : cur[q], ok[q]);
+    }
+    {
+      df64 v[2] = {dot.re, dot.im};
+      block_partial(v, 3, pa + (size_t)bx * 4);
+    }
+    if (!problem_barrier(&bars[r], nblk, err, &s_fail)) return;
+    if (warp == 0) {
+      double tot[2];
+      problem_total<2>(pa, nblk, tot);
+      // as finish_alpha
+      double ar, ai = 0.0;
+      double2 nw = nwj;
+      if (!TWO) {
+        ar = tot[0] / nvj;
+        nw = make_double2(nvj, 0.0);
+      } else {
+        const double den = nw.x * nw.x + nw.y * nw.y;
+        const double q = (lane == 0 ? tot[0] * nw.x + tot[1] * nw.y : tot[1] * nw.x - tot[0] * nw.y) / den;
+        ar = bcast(q, 0);
+        ai = bcast(q, 1);
+      }
+      const double dw = nw.x * nw.x + nw.y * nw.y;
+      const double num = lane == 0 ? ar : lane == 1 ? ai : lane == 2 ? ar * nw.x + ai * nw.y : ai * nw.x - ar * nw.y;
+      const double q = num / (lane < 2 ? nvj : dw);
+      const double im = __shfl_down_sync(0xffffffffu, q, 1);
+      if (lane == 0) {
+        if (lead) a.c.alp[co] = make_double2(ar, ai);
+        st_vec(&s_scal[4], cd_to<df64>(q, im));
+      }
+      if (lane == 2) st_vec(&s_scal[5], cd_to<df64>(q, -im));
+      betj.y = ar;  // (Lanczos' breakdown test reads alpha_j; bet is real)
+    }
+    __syncthreads();
+    const cx<df64> al = ld_vec(&s_scal[4 + side]);
+    df64 nvv = df_zero();
+    cx<df64> del = {df_zero(), df_zero()};
+    float nl = 0.f;
+    cx<df64> nxt[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      nxt[q] = csubmul(ok[q], al, cur[q]);
+      if (active) {
+        __stcg(dst + (size_t)kk[q] * V + ss, make_float4(nxt[q].re.hi, nxt[q].re.lo, nxt[q].im.hi, nxt[q].im.lo));
+        if (!TWO) acc_norm(nvv, nxt[q]);
+        else acc_norm_lo(nl, nxt[q]);
+      }
+      if (TWO && side == 1) st_vec(&s_x[96 * q + t96], nxt[q]);
+    }
+    if (TWO) {
+      __syncthreads();
+      if (active && side == 0) {
+        acc_dot(del, ld_vec(&s_x[t96]), nxt[0]);
+        acc_dot(del, ld_vec(&s_x[96 + t96]), nxt[1]);
+      }
+      df64 v[4] = {del.re, del.im, {side == 0 ? nl : 0.f, 0.f}, {side == 1 ? nl : 0.f, 0.f}};
+      block_partial(v, NW, pd + (size_t)bx * 4);
+    } else {
+      df64 v[1] = {nvv};
+      block_partial(v, NW, pd + (size_t)bx * 4);
+    }
+    __threadfence();  // the new vector, before the barrier's arrival
+    if (!problem_barrier(&bars[r], nblk, err, &s_fail)) return;
+    if (warp == 0) {
+      double nv;
+      double2 nw, be, ga;
+      bool broke;
+      if (!TWO) {
+        double tot[1];
+        problem_total<1>(pd, nblk, tot);
+        // as finish_lanczos
+        const double bb = sqrt(tot[0]);
+        broke = !(bb > a.breakdown_tol * (fabs(betj.y) + fabs(betj.x)));
+        const bool dead = broke || status != kStOK;
+        nv = dead ? 1.0 : bb;
+        nw = make_double2(nv, 0.0);
+        be = ga = make_double2(dead ? 0.0 : bb, 0.0);
+      } else {
+        double tot[4];
+        problem_total<4>(pd, nblk, tot);
+        // as finish_two_sided
+        const double dre = tot[0], dim = tot[1];
+        const double root = sqrt(lane == 0 ? dre * dre + dim * dim : lane == 1 ? tot[2] : tot[3]);
+        const double ad = bcast(root, 0), nt = bcast(root, 1), nu = bcast(root, 2);
+        const double bb = sqrt(ad);
+        broke = !(ad > a.breakdown_tol * nt * nu) || !(bb > 0.0);
+        const bool dead = broke || status != kStOK;
+        const double q = (lane == 0 ? dre : dim) / bb;
+        const double2 gg = make_double2(bcast(q, 0), bcast(q, 1));
+        nv = dead ? 1.0 : bb;
+        nw = dead ? make_double2(1.0, 0.0) : gg;
+        be = make_double2(dead ? 0.0 : bb, 0.0);
+        ga = dead ? make_double2(0.0, 0.0) : gg;
+      }
+      if (lead && lane == 0) {
+        if (broke && status == kStOK) {
+          a.c.status[r] = TWO ? kStBreakdown : kStLucky;
+          a.c.kbreak[r] = j;
+        }
+        a.c.nv[co + 1] = nv;
+        a.c.nw[co + 1] = nw;
+        a.c.bet[co + 1] = be;
+        a.c.gam[co + 1] = ga;
+      }
+      if (broke && status == kStOK) status = TWO ? kStBreakdown : kStLucky;
+      set_step_scal<PrecDF64>(s_scal, 0, nv, ga, nw, be, nvj, nwj);
+      if (lead && i + 1 == nsteps) set_step_scal<PrecDF64>(a.scal, r, nv, ga, nw, be, nvj, nwj);
+      nvj = nv;
+      nwj = nw;
+      betj = be;
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      prv[q] = cur[q];
+      cur[q] = nxt[q];
+    }
+    src = dst;
+  }
+  // the last problem to finish advances the step index
+  if (lead && tid == 0) {
+    __threadfence();
+    if (atomicAdd(a.gticket, 1u) == (unsigned)(a.b.nprob - 1)) {
+      *a.gticket = 0u;
+      *a.jdev = j0 + nsteps;
+      __threadfence();
+    }
+  }
+}
+
+// blocks of k_steps that run at the same time
+int steps_capacity(int mode) {
+  int per = 0, dev = 0, sms = 0;
+  cudaError_t e = mode == kModeTwoSided
+                      ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_steps<kModeTwoSided>, 192, 0)
+                      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_steps<kModeLanczos>, 96, 0);
+  if (e != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return per * sms;
+}
+cudaError_t launch_steps(int mode, const StepArgs& a, int nsteps, unsigned* bars, int* err, cudaStream_t st) {
+  StepArgs args = a;
+  void* p[] = {&args, &nsteps, &bars, &err};
+  const dim3 grid(a.b.nblocks * 4);
+  if (mode == kModeTwoSided)
+    return cudaLaunchCooperativeKernel((const void*)k_steps<kModeTwoSided>, grid, dim3(192), p, 0, st);
+  return cudaLaunchCooperativeKernel((const void*)k_steps<kModeLanczos>, grid, dim3(96), p, 0, st);
 }
 
 // ------------------------------------------------------------ recombination

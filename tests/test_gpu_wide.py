@@ -1,5 +1,6 @@
 """The wide step and update kernels (twelve threads a site, for lattices with fewer sites than
-the GPU has threads) against the kernels with one thread a site, at ragged volumes (V not a
+the GPU has threads) and the runs of steps in one cooperative launch against the kernels with
+one thread a site, at ragged volumes (V not a
 multiple of the 16, 32 or 64 sites of a block). The two differ in the grouping of the partial
 sums only, like two block sizes, so the bar is the one of test_block_sizes: 1e-11."""
 import numpy as np
@@ -18,20 +19,22 @@ def ov():
     return ov
 
 
+# (the last lattice has more blocks than run at once: two launches a step)
+@pytest.mark.parametrize("recomb", [0, 1])
 @pytest.mark.parametrize("mu", [0.0, 0.3])
-@pytest.mark.parametrize("dims,nrhs,sites", [((5, 4, 7, 6), 1, 16), ((3, 2, 2, 3), 2, 16), ((9, 7, 8, 6), 3, 32)])
-def test_wide_equals_narrow(ov, monkeypatch, capfd, dims, nrhs, sites, mu):
+@pytest.mark.parametrize("dims,nrhs,sites,one", [((5, 4, 7, 6), 1, 16, 1), ((3, 2, 2, 3), 2, 16, 1), ((9, 7, 8, 6), 6, 32, 0)])
+def test_wide_equals_narrow(ov, monkeypatch, capfd, dims, nrhs, sites, one, mu, recomb):
     monkeypatch.setenv("OV_TRACE", "1")
     U = oi.gauge_field(dims, "near_unit", 3, eps=0.35)
     x = np.stack([oi.gaussian_source(dims, 10 + r) for r in range(nrhs)])
     ys = {}
     for bs in (0, 64):
         y = np.zeros_like(x)
-        with ov.Overlap(dims, U, -1.5, mu, "df64", opts=ov.make_opts(k_fixed=60, block_size=bs)) as op:
+        with ov.Overlap(dims, U, -1.5, mu, "df64", opts=ov.make_opts(k_fixed=60, block_size=bs, recombination=recomb)) as op:
             rc, _ = op.sign_apply(x, y, 1e-8, 60, 60)
         assert rc == 0
         ys[bs] = y
-    assert f'"wide": {sites},' in capfd.readouterr().err  # the tuner took the wide kernels
+    assert f'"wide": {sites}, "one_launch": {one},' in capfd.readouterr().err  # what the tuner took
     for r in range(nrhs):
         assert rel(ys[0][r], ys[64][r]) < 1e-11
 
