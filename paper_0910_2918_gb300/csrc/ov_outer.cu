@@ -376,8 +376,8 @@ __device__ __forceinline__ void hopping_df(cx<df64> (&accn)[12], const float4* _
 __device__ __forceinline__ cx<double> ld_hop(const double2* p) { return ld_vec(p); }
 __device__ __forceinline__ cx<float> ld_hop(const float2* p) { return ld_vec(p); }
 __device__ __forceinline__ cx<float> ld_hop(const float4* p) {
-  const float4 v = *p;
-  return {v.x, v.z};
+  const float2 v = *(const float2*)p;
+  return {v.x, v.y};
 }
 
 // acc = sum over the 8 hops of the hopping term for source `src` at site s in arithmetic
@@ -509,14 +509,77 @@ __device__ __forceinline__ cxu rot_u(cxu z, int q) {
   return {nre ? neg_u(r.re) : r.re, nim ? neg_u(r.im) : r.im};
 }
 
+// One thread a site: the real and the imaginary part of every number are the two halves of a
+// packed register, as they lie in memory (hi pair, lo pair), so that an instruction serves both
+// (two passes of the float pipe, one issue slot: the sums are then bound by the pipe, ~1100 of
+// its cycles a hop and side, more than by issue slots). The operations and their order are those
+// of the scalar form (another order moved results with relaxed steps by 1.6e-9). Strict step of
+// 12 x 16^4 0.843 -> 0.756 ms; a column of the link at a time instead of all loads first 0.814.
+struct pcx {  // unnormalised complex pair: hi + lo
+  f32x2 hi, lo;
+};
+__device__ __forceinline__ pcx ld_pcx(const float4* p) {
+  const ulonglong2 v = *(const ulonglong2*)p;
+  return {v.x, v.y};
+}
+__device__ __forceinline__ pcx add_p(pcx a, pcx b) {
+  const f32x2 s = add2(a.hi, b.hi), bb = sub2(s, a.hi);
+  const f32x2 err = add2(sub2(a.hi, sub2(s, bb)), sub2(b.hi, bb));
+  return {s, add2(add2(a.lo, b.lo), err)};
+}
+// acc = u h and acc += u h (u: one link word in both halves of the register, or (-u, u))
+__device__ __forceinline__ void set_p(pcx& acc, f32x2 u, pcx h) {
+  acc.hi = mul2(u, h.hi);
+  acc.lo = fma2(u, h.lo, fma2(u, h.hi, neg2(acc.hi)));
+}
+__device__ __forceinline__ void madd_p(pcx& acc, f32x2 u, pcx h) {
+  const f32x2 p = mul2(u, h.hi);
+  const f32x2 e = fma2(u, h.lo, fma2(u, h.hi, neg2(p)));
+  const f32x2 s = add2(acc.hi, p), bb = sub2(s, acc.hi);
+  const f32x2 err = add2(sub2(acc.hi, sub2(s, bb)), sub2(p, bb));
+  acc.hi = s;
+  acc.lo = add2(acc.lo, add2(e, err));
+}
+__device__ __forceinline__ f32x2 swap_p(f32x2 a) {
+  const float2 v = upk(a);
+  return pk(v.y, v.x);
+}
+// acc (+)= u h for the complex link u (hi words), c += ul h.hi for its lo words: the term of u.re,
+// then that of u.im with (i h) = (-h.im, h.re) as (-u.im, u.im) times hs = (h.im, h.re)
+template <bool SET>
+__device__ __forceinline__ void cmadd_p(pcx& acc, f32x2& c, cx<float> u, cx<float> ul, pcx h, pcx hs) {
+  if (SET) set_p(acc, pk(u.re, u.re), h);
+  else madd_p(acc, pk(u.re, u.re), h);
+  madd_p(acc, pk(-u.im, u.im), hs);
+  c = fma2(pk(ul.re, ul.re), h.hi, fma2(pk(-ul.im, ul.im), hs.hi, c));
+}
+// i^q a, with the signs of the two halves as masks
+struct Phase4 {
+  bool sw;
+  unsigned mre, mim;
+};
+__device__ __forceinline__ Phase4 phase_of(int q) {
+  return {(q & 1) != 0, q == 1 || q == 2 ? 0x80000000u : 0u, q >= 2 ? 0x80000000u : 0u};
+}
+__device__ __forceinline__ f32x2 rot_p(f32x2 a, Phase4 f) {
+  const float2 v = upk(a);
+  const float x = f.sw ? v.y : v.x, y = f.sw ? v.x : v.y;
+  return pk(__uint_as_float(__float_as_uint(x) ^ f.mre), __uint_as_float(__float_as_uint(y) ^ f.mim));
+}
+__device__ __forceinline__ pcx rot_p(pcx a, Phase4 f) { return {rot_p(a.hi, f), rot_p(a.lo, f)}; }
+__device__ __forceinline__ cx<df64> norm_p(pcx a) {
+  const float2 h = upk(a.hi), l = upk(a.lo);
+  return {df_fast_two_sum(h.x, l.x), df_fast_two_sum(h.y, l.y)};
+}
+
 __device__ __forceinline__ void hopping_df(cx<df64> (&accn)[12], const float4* __restrict__ src,
                                            const float2* __restrict__ links, const Geometry& g, int s,
                                            const int (&xc)[4], df64 ef, df64 eb) {
   const int V = g.V;
   const float2* __restrict__ links_lo = links + (size_t)36 * V;
-  cxu acc[12];
+  pcx acc[12];
 #pragma unroll
-  for (int k = 0; k < 12; ++k) acc[k] = {{0.f, 0.f}, {0.f, 0.f}};
+  for (int k = 0; k < 12; ++k) acc[k] = {0ull, 0ull};
 #pragma unroll 1
   for (int hop = 0; hop < 8; ++hop) {
     const int nu = hop >> 1;
@@ -534,75 +597,49 @@ __device__ __forceinline__ void hopping_df(cx<df64> (&accn)[12], const float4* _
       ulo[e] = lconj(ld_link(links_lo + (size_t)(nu * 9 + idx) * V + ls), !fwd);
     }
     const int b0s = c_bsrc[nu][0], b1s = c_bsrc[nu][1];
-    const int b0q = (c_bph[nu][0] + (fwd ? 2 : 0)) & 3, b1q = (c_bph[nu][1] + (fwd ? 2 : 0)) & 3;
-    cx<df64> h0[3], h1[3];
+    const Phase4 b0f = phase_of((c_bph[nu][0] + (fwd ? 2 : 0)) & 3), b1f = phase_of((c_bph[nu][1] + (fwd ? 2 : 0)) & 3);
+    pcx h0[3], h1[3];
 #pragma unroll
     for (int col = 0; col < 3; ++col) {
-      const cx<df64> p0 = ld_vec(src + (size_t)(0 + col) * V + sn);
-      const cx<df64> p1 = ld_vec(src + (size_t)(3 + col) * V + sn);
-      const cx<df64> q0 = rot(ld_vec(src + (size_t)(3 * b0s + col) * V + sn), b0q);
-      const cx<df64> q1 = rot(ld_vec(src + (size_t)(3 * b1s + col) * V + sn), b1q);
       // projections, unnormalised (their low words only enter through FMAs below)
-      const dfu r0 = add_u(to_u(p0.re), to_u(q0.re)), i0 = add_u(to_u(p0.im), to_u(q0.im));
-      const dfu r1 = add_u(to_u(p1.re), to_u(q1.re)), i1 = add_u(to_u(p1.im), to_u(q1.im));
-      h0[col] = {{r0.hi, r0.lo}, {i0.hi, i0.lo}};
-      h1[col] = {{r1.hi, r1.lo}, {i1.hi, i1.lo}};
+      h0[col] = add_p(ld_pcx(src + (size_t)(0 + col) * V + sn), rot_p(ld_pcx(src + (size_t)(3 * b0s + col) * V + sn), b0f));
+      h1[col] = add_p(ld_pcx(src + (size_t)(3 + col) * V + sn), rot_p(ld_pcx(src + (size_t)(3 * b1s + col) * V + sn), b1f));
     }
     const bool sc = nu == 3;
     const df64 fac = fwd ? ef : eb;
     const int d0s = c_dsrc[nu][0], d1s = c_dsrc[nu][1];
-    const int d0q = (c_dph[nu][0] + (fwd ? 2 : 0)) & 3, d1q = (c_dph[nu][1] + (fwd ? 2 : 0)) & 3;
+    const Phase4 d0f = phase_of((c_dph[nu][0] + (fwd ? 2 : 0)) & 3), d1f = phase_of((c_dph[nu][1] + (fwd ? 2 : 0)) & 3);
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      cxu g0, g1;
+      pcx g0, g1;
+      f32x2 c0 = 0ull, c1 = 0ull;  // U.lo row a times h.hi
 #pragma unroll
       for (int b = 0; b < 3; ++b) {
-        const cx<float> ub = u[a * 3 + b];
-        // (u.re + i u.im)(h.re + i h.im); the first product of each sum sets it
+        const cx<float> uh = u[a * 3 + b], ul = ulo[a * 3 + b];
+        const pcx s0 = {swap_p(h0[b].hi), swap_p(h0[b].lo)}, s1 = {swap_p(h1[b].hi), swap_p(h1[b].lo)};
         if (b == 0) {
-          set_u(g0.re, ub.re, h0[b].re);
-          set_u(g0.im, ub.re, h0[b].im);
-          set_u(g1.re, ub.re, h1[b].re);
-          set_u(g1.im, ub.re, h1[b].im);
+          cmadd_p<true>(g0, c0, uh, ul, h0[b], s0);
+          cmadd_p<true>(g1, c1, uh, ul, h1[b], s1);
         } else {
-          madd_u(g0.re, ub.re, h0[b].re);
-          madd_u(g0.im, ub.re, h0[b].im);
-          madd_u(g1.re, ub.re, h1[b].re);
-          madd_u(g1.im, ub.re, h1[b].im);
+          cmadd_p<false>(g0, c0, uh, ul, h0[b], s0);
+          cmadd_p<false>(g1, c1, uh, ul, h1[b], s1);
         }
-        madd_u(g0.re, -ub.im, h0[b].im);
-        madd_u(g0.im, ub.im, h0[b].re);
-        madd_u(g1.re, -ub.im, h1[b].im);
-        madd_u(g1.im, ub.im, h1[b].re);
       }
-      // U.lo row a times h.hi, into the low words
-      float c0r = 0.f, c0i = 0.f, c1r = 0.f, c1i = 0.f;
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        const cx<float> ul = ulo[a * 3 + b];
-        c0r = __fmaf_rn(ul.re, h0[b].re.hi, __fmaf_rn(-ul.im, h0[b].im.hi, c0r));
-        c0i = __fmaf_rn(ul.re, h0[b].im.hi, __fmaf_rn(ul.im, h0[b].re.hi, c0i));
-        c1r = __fmaf_rn(ul.re, h1[b].re.hi, __fmaf_rn(-ul.im, h1[b].im.hi, c1r));
-        c1i = __fmaf_rn(ul.re, h1[b].im.hi, __fmaf_rn(ul.im, h1[b].re.hi, c1i));
-      }
-      g0.re.lo = __fadd_rn(g0.re.lo, c0r);
-      g0.im.lo = __fadd_rn(g0.im.lo, c0i);
-      g1.re.lo = __fadd_rn(g1.re.lo, c1r);
-      g1.im.lo = __fadd_rn(g1.im.lo, c1i);
+      g0.lo = add2(g0.lo, c0);
+      g1.lo = add2(g1.lo, c1);
       if (sc) {
-        const cx<df64> n0 = cscale(cx<df64>{norm_u(g0.re), norm_u(g0.im)}, fac);
-        const cx<df64> n1 = cscale(cx<df64>{norm_u(g1.re), norm_u(g1.im)}, fac);
-        g0 = {to_u(n0.re), to_u(n0.im)};
-        g1 = {to_u(n1.re), to_u(n1.im)};
+        const cx<df64> n0 = cscale(norm_p(g0), fac), n1 = cscale(norm_p(g1), fac);
+        g0 = {pk(n0.re.hi, n0.im.hi), pk(n0.re.lo, n0.im.lo)};
+        g1 = {pk(n1.re.hi, n1.im.hi), pk(n1.re.lo, n1.im.lo)};
       }
-      acc[0 + a] = cadd_u(acc[0 + a], g0);
-      acc[3 + a] = cadd_u(acc[3 + a], g1);
-      acc[6 + a] = cadd_u(acc[6 + a], rot_u(d0s == 0 ? g0 : g1, d0q));
-      acc[9 + a] = cadd_u(acc[9 + a], rot_u(d1s == 0 ? g0 : g1, d1q));
+      acc[0 + a] = add_p(acc[0 + a], g0);
+      acc[3 + a] = add_p(acc[3 + a], g1);
+      acc[6 + a] = add_p(acc[6 + a], rot_p(d0s == 0 ? g0 : g1, d0f));
+      acc[9 + a] = add_p(acc[9 + a], rot_p(d1s == 0 ? g0 : g1, d1f));
     }
   }
 #pragma unroll
-  for (int k = 0; k < 12; ++k) accn[k] = {norm_u(acc[k].re), norm_u(acc[k].im)};
+  for (int k = 0; k < 12; ++k) accn[k] = norm_p(acc[k]);
 }
 
 // (gamma5 D psi)_k at the centre site from the hopping sum: mass*psi - hop/2, lower spins negated.
@@ -1379,7 +1416,7 @@ __global__ void __launch_bounds__(MODE == kModeTwoSided ? 192 : 96) k_steps(Step
     for (int q = 0; q < 2; ++q) {
       nxt[q] = csubmul(ok[q], al, cur[q]);
       if (active) {
-        __stcg(dst + (size_t)kk[q] * V + ss, make_float4(nxt[q].re.hi, nxt[q].re.lo, nxt[q].im.hi, nxt[q].im.lo));
+        __stcg(dst + (size_t)kk[q] * V + ss, vec_of(nxt[q]));
         if (!TWO) acc_norm(nvv, nxt[q]);
         else acc_norm_lo(nl, nxt[q]);
       }

@@ -117,6 +117,46 @@ template <class R, class L> __device__ __forceinline__ cx<R> lcmulc(cx<L> u, cx<
   return {lmul(v.re, u.re) + lmul(v.im, u.im), lmul(v.im, u.re) - lmul(v.re, u.im)};
 }
 
+// ----------------------------------------------------------------- packed pairs of floats
+// Two floats in a 64-bit register, handled by one instruction (add, sub, mul, fma .f32x2, each
+// half rounded as the scalar instruction would). The packed forms take two passes of the float
+// pipe and one issue slot.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pk(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 upk(f32x2 a) {
+  float2 v;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(a));
+  return v;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f32x2 neg2(f32x2 a) {  // folded into the instruction that takes it
+  const float2 v = upk(a);
+  return pk(-v.x, -v.y);
+}
+
 // ----------------------------------------------------------------- precision policies
 // vec_t: storage of one complex vector element; link_t: storage of one complex link
 // element; R: arithmetic of the stencil; L: link arithmetic; A: per-thread accumulator of
@@ -141,7 +181,7 @@ struct PrecDF64 {
   using R = df64;
   using L = float;
   using A = df64;
-  using vec_t = float4;  // (re.hi, re.lo, im.hi, im.lo)
+  using vec_t = float4;  // (re.hi, im.hi, re.lo, im.lo)
   using link_t = float2;
   static constexpr int id = 2;
 };
@@ -168,13 +208,12 @@ __device__ __forceinline__ cx<float> ld_vec(const float2* p) {
 }
 __device__ __forceinline__ cx<df64> ld_vec(const float4* p) {
   float4 v = *p;
-  return {{v.x, v.y}, {v.z, v.w}};
+  return {{v.x, v.z}, {v.y, v.w}};
 }
 __device__ __forceinline__ void st_vec(double2* p, cx<double> a) { *p = make_double2(a.re, a.im); }
 __device__ __forceinline__ void st_vec(float2* p, cx<float> a) { *p = make_float2(a.re, a.im); }
-__device__ __forceinline__ void st_vec(float4* p, cx<df64> a) {
-  *p = make_float4(a.re.hi, a.re.lo, a.im.hi, a.im.lo);
-}
+__device__ __forceinline__ float4 vec_of(cx<df64> a) { return make_float4(a.re.hi, a.im.hi, a.re.lo, a.im.lo); }
+__device__ __forceinline__ void st_vec(float4* p, cx<df64> a) { *p = vec_of(a); }
 __device__ __forceinline__ cx<double> ld_link(const double2* p) {
   double2 v = __ldg(p);
   return {v.x, v.y};
