@@ -104,8 +104,8 @@ typedef struct {
                            estimate reaches tol (at least check_interval and at most
                            4 * check_interval steps later) [0] */
   int block_size;       /* threads per block of the site kernels: 64, 128, 256, or 0 = autotune
-                           (time the first outer step at each size once per handle and problem
-                           set, keep the fastest) [0] */
+                           (time the first outer step at each size, and with the kernels for small
+                           lattices, once per handle and problem set, keep the fastest) [0] */
   int graph_steps;      /* outer steps per CUDA graph: runs of steps between checks replay a graph of
                            this many steps captured once per handle (0: plain launches; timing = 1
                            also uses plain launches) [8] */
@@ -132,10 +132,13 @@ typedef struct {
                            48-lattice batch 13 of 48 lattices then stop converging [0] */
   int overlap_checks;   /* 1: a stopping check runs on a second, high-priority stream while up to
                            24 further outer steps (fewer than check_interval) run speculatively;
-                           a run that stops at the check uses k = the check's step, so results
-                           are those of the serial order (not used where the previous check's
-                           largest outer estimate was within 8 tol, where a stop is likely);
-                           0: checks block the outer steps [1] */
+                           where an interval of outer steps takes less time than a check, the steps
+                           of up to 8 intervals run first and their checks are evaluated together
+                           and judged in order (not with check_schedule 1 or learned sizing). A run
+                           that stops at a check uses k = the check's step, so results are those of
+                           the serial order (no speculation where the previous check's largest outer
+                           estimate was within 8 tol, where a stop is likely); 0: checks block the
+                           outer steps [1] */
   int nested;           /* 1: the nested method (Sec. 3); 0: the non-nested method (Sec. 2): every
                            stopping check takes c = sgn(H_k) e_1 by Roberts-Higham on the full
                            k x k Ritz matrix (FP64 Gauss-Jordan inversions over global memory,
