@@ -1098,11 +1098,13 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
       }
       CK(cudaMemcpyAsync(h->cl.p, lreq.data(), sizeof(int) * nrhs, cudaMemcpyHostToDevice, st));
       // (at most one interval before k_max, so that the check at k_max has a baseline)
-      // at an even k: the spectrum is indefinite and nearly symmetric about zero, and an odd
-      // number of Ritz values leaves one close to zero, which upsets the estimates of every
-      // check of the run (24^3 x 48, first check at k = 199: stops at 249)
+      // at an even k where the interval is even too: the spectrum is indefinite and nearly
+      // symmetric about zero, and an odd number of Ritz values leaves one close to zero, which
+      // upsets the estimates of a grid of odd k (24^3 x 48, checks every 10 steps: from k = 199 on
+      // the run stops at 249, from 198 on at 238; with an odd interval the parity alternates)
+      const int odd = o.check_interval % 2 == 0 ? 1 : 0;
       if (kmax_pred > 0.0)
-        next_check = std::max(j + 1, std::min((int)std::floor(std::min(kmax_pred, (double)ktarget)) & ~1,
+        next_check = std::max(j + 1, std::min((int)std::floor(std::min(kmax_pred, (double)ktarget)) & ~odd,
                                               ktarget - o.check_interval));
       if (relaxing && kmax_pred > 0.0)
         relax_from = std::max(j + 1, (int)std::ceil(o.relax * std::min(kmax_pred, (double)ktarget)));
