@@ -920,8 +920,8 @@ __device__ bool tri_factor_df(const InnerSmemDf<St>& S, int k, const St* ia) {
 //    1000: the errors of the serial sweeps).
 // 3 + 5 + 3 dependent multiply-adds replace 333 at k = 333; 12 problems, l = 120: 8.72 -> 1.44 ms
 // (two-sided); at mu = 0, in real arithmetic, the whole inner level 11.0 -> 1.31 ms (1.87 in
-// complex arithmetic). With the chains gone the two-sided step is bound by the
-// float pipe of its SM (48% issue, ~6000 instructions a warp and step). 32 or 64 lanes a side do
+// complex arithmetic). With the chains gone the two-sided step is spent on the instructions and
+// latency of its SM (issue 49%, float pipe 38%, ~6000 instructions a warp and step). 32 or 64 lanes a side do
 // less work in the scans but run longer chunks: slower from k = 333 on.
 constexpr int kSideLanes = 128;  // lanes of one side (v: threads 0.., w: the rest)
 constexpr int kSideWarps = kSideLanes / 32;
