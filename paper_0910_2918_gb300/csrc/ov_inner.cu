@@ -1658,6 +1658,9 @@ __global__ void __cluster_dims__(kCombineCtas, 1, 1) __launch_bounds__(kCombineT
   __shared__ float4 s_ds[kMaxL];
   __shared__ double s_red[kCombineThreads / 32][2];
   __shared__ double s_tot[kCombineCtas][2];
+  // a CTA's shared memory may be written by another once it is known to run: all arrive here, and
+  // wait before the one remote write (the sums over Q lie between, so the wait costs nothing)
+  cluster.barrier_arrive();
   const int rank = (int)cluster.block_rank(), prob = blockIdx.x / kCombineCtas, row0 = prob % w.rows;
   const int k = k_dev[prob];
   const int le = w.leff[prob];
@@ -1726,6 +1729,7 @@ __global__ void __cluster_dims__(kCombineCtas, 1, 1) __launch_bounds__(kCombineT
   nd = warp_sum(nd);
   if ((tid & 31) == 0) { s_red[tid >> 5][0] = nc; s_red[tid >> 5][1] = nd; }
   __syncthreads();
+  cluster.barrier_wait();
   if (tid < 2) {
     double t = 0.0;
     for (int q = 0; q < kCombineThreads / 32; ++q) t += s_red[q][tid];
