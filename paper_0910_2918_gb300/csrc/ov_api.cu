@@ -150,6 +150,7 @@ struct ov_handle {
   int last_steps = 0, last_ld = 0, last_nrhs = 0;
   int trace = 0;  // OV_TRACE set in the environment: one JSON line per check on stderr
   size_t basis_cap = 0;  // OV_BASIS_CAP_BYTES: bytes the stored basis may take (0: no cap)
+  int bar_polls = kBarPolls;  // OV_BARRIER_POLLS: the bound of a wait in k_steps
   Buf nn_scratch;        // the non-nested check's dense H_k, iterates and elimination buffers
   // deflation (Sec. 2): per lattice the critical eigenvalues and right / left eigenvectors
   // (canonical complex doubles, [m][12 V]; L = R at mu = 0)
@@ -375,10 +376,16 @@ static int check_opts(const ov_opts& o) {
   return OV_OK;
 }
 
+static int env_polls() {
+  const char* v = getenv("OV_BARRIER_POLLS");
+  return v ? std::max(0, atoi(v)) : kBarPolls;
+}
+
 extern "C" int ov_set_opts(ov_handle* h, const ov_opts* opts) {
   if (!h || !opts) return OV_ERR_ARG;
   if (check_opts(*opts) != OV_OK) return OV_ERR_ARG;
   h->o = *opts;
+  h->bar_polls = env_polls();
   return OV_OK;
 }
 
@@ -451,6 +458,7 @@ extern "C" int ov_create(ov_handle** hp, const ov_geom* geom, const void* links,
   h->o = o;
   h->trace = getenv("OV_TRACE") != nullptr;
   if (const char* cap = getenv("OV_BASIS_CAP_BYTES")) h->basis_cap = (size_t)strtoull(cap, nullptr, 10);
+  h->bar_polls = env_polls();
   const size_t canon = sizeof(double2) * 36 * (size_t)V;
   const double2* src = (const double2*)links;
   Buf tmp;
@@ -548,8 +556,9 @@ static int ensure_outer(ov_handle* h, int nrhs, int ld, size_t pool, int nblocks
 struct CheckBuf {
   double *eo, *ei;
   int *rhst, *rhit, *leff, *k, *l, *status, *kbreak;
+  int* err;  // one word: a wait of k_steps ran out
 };
-static size_t check_bytes(int cap) { return (size_t)cap * (2 * sizeof(double) + 7 * sizeof(int)); }
+static size_t check_bytes(int cap) { return (size_t)cap * (2 * sizeof(double) + 7 * sizeof(int)) + sizeof(int); }
 static CheckBuf check_buf(void* base, int cap) {
   CheckBuf b;
   b.eo = (double*)base;
@@ -562,6 +571,7 @@ static CheckBuf check_buf(void* base, int cap) {
   b.l = i + 4 * (size_t)cap;
   b.status = i + 5 * (size_t)cap;
   b.kbreak = i + 6 * (size_t)cap;
+  b.err = i + 7 * (size_t)cap;
   return b;
 }
 // the breakdown state of right-hand side r as the check at step j sees it: one recorded by a
@@ -949,7 +959,7 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
       if (coop && gU > 0) {
         // every block fits the GPU at once: the whole span in one launch
         const int nst = jto - jn + 1;
-        CK(launch_steps(mode, a, nst, (unsigned*)h->bars.p, (int*)h->bars.p + nrhs, st));
+        CK(launch_steps(mode, a, nst, (unsigned*)h->bars.p, h->bar_polls, (int*)h->bars.p + nrhs, st));
         h->stats.launches += 1;
         h->stats.stencil_launches += nst;
         h->stats.update_launches += nst;
@@ -1159,7 +1169,8 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
     if (gcap > 1) CK(cudaEventRecord(h->ev_time[2], cs));
     const CheckBuf db = check_buf(h->chk.p, h->inner_cap);
     const CheckBuf hb = check_buf(h->chk_host, h->inner_cap);
-    CK(launch_check_setup(nrhs, n, cj, c.status, c.kbreak, (const int*)h->cl.p, db.k, db.l, db.status, db.kbreak, cs));
+    CK(launch_check_setup(nrhs, n, cj, c.status, c.kbreak, (const int*)h->cl.p, (const int*)h->bars.p + nrhs, db.k, db.l,
+                          db.status, db.kbreak, db.err, cs));
     const int ti = tstart(h, kClsInner, cs);
     // the double-float inner level takes both Roberts-Higham sets at once (they run side by
     // side); in FP64 the inner estimate's set runs where it is wanted, or where a stop is
@@ -1196,6 +1207,11 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
       }
     }
     CK(cudaStreamSynchronize(cs));
+    if (*hb.err != 0) {
+      // a wait of k_steps ran out: the coefficients end somewhere before these checks
+      CK(cudaStreamSynchronize(st));
+      return OV_ERR_CUDA;
+    }
     // the inner estimate is needed only where the run may stop at this check
     bool have_ei = phase == 0 && !fixed;
     if (!have_ei && !fixed) {

@@ -1778,8 +1778,9 @@ __global__ void __launch_bounds__(kCombineThreads) k_estimate(const int* __restr
 }
 
 __global__ void k_check_setup(int rows, int n, CheckSteps cj, const int* __restrict__ status,
-                              const int* __restrict__ kbreak, const int* __restrict__ l_in, int* k_out, int* l_out,
-                              int* status_out, int* kbreak_out) {
+                              const int* __restrict__ kbreak, const int* __restrict__ l_in, const int* err, int* k_out,
+                              int* l_out, int* status_out, int* kbreak_out, int* err_out) {
+  if (threadIdx.x == 0) *err_out = *err;
   for (int r = threadIdx.x; r < rows; r += blockDim.x) {
     const int s = status[r], kb = kbreak[r];
     status_out[r] = s;
@@ -1792,8 +1793,9 @@ __global__ void k_check_setup(int rows, int n, CheckSteps cj, const int* __restr
   }
 }
 cudaError_t launch_check_setup(int rows, int n, const CheckSteps& cj, const int* status, const int* kbreak, const int* l_in,
-                               int* k_out, int* l_out, int* status_out, int* kbreak_out, cudaStream_t st) {
-  k_check_setup<<<1, 128, 0, st>>>(rows, n, cj, status, kbreak, l_in, k_out, l_out, status_out, kbreak_out);
+                               const int* err, int* k_out, int* l_out, int* status_out, int* kbreak_out, int* err_out,
+                               cudaStream_t st) {
+  k_check_setup<<<1, 128, 0, st>>>(rows, n, cj, status, kbreak, l_in, err, k_out, l_out, status_out, kbreak_out, err_out);
   return cudaGetLastError();
 }
 

@@ -122,10 +122,12 @@ cudaError_t launch_pack(int prec, const Batch& b, const double2* xcanon, void* x
                         double* partials, unsigned* counters, int want_norm, void* scal, cudaStream_t st);
 cudaError_t launch_step(int prec, int mode, const StepArgs& a, cudaStream_t st);
 // nsteps outer steps in one cooperative launch (strict double-float, a.b.block = 64; bars: a zeroed
-// counter per problem that all launches of an apply share, *err: set if a wait ran out); it must
-// not have more blocks (four per site block) than steps_capacity(mode)
+// counter per problem that all launches of an apply share, *err: set if a wait took more than
+// `polls` looks at its counter; nothing runs while it is set); it must not have more blocks (four
+// per site block) than steps_capacity(mode)
+constexpr int kBarPolls = 1 << 22;  // of one barrier's wait: a second or so
 int steps_capacity(int mode);
-cudaError_t launch_steps(int mode, const StepArgs& a, int nsteps, unsigned* bars, int* err, cudaStream_t st);
+cudaError_t launch_steps(int mode, const StepArgs& a, int nsteps, unsigned* bars, int polls, int* err, cudaStream_t st);
 cudaError_t launch_update(int prec, int mode, const StepArgs& a, cudaStream_t st);
 // y_r = scale_r * sum_{j<k_r} c[r][j+1] v_{r,j+1} (+ x_r and gamma5 if add_x); slots[j] is
 // the device address of basis slot j (a vector pool)
@@ -168,9 +170,10 @@ struct CheckSteps {
 };
 // the problems of a group (i = check i / rows of right-hand side i % rows): k_out[i] = the check's
 // step, or the step of a breakdown at or before it; l_out[i] = l_in[i % rows]; and the breakdown
-// state of the right-hand sides as it is now
+// state of the right-hand sides and the error word of launch_steps as they are now
 cudaError_t launch_check_setup(int rows, int n, const CheckSteps& cj, const int* status, const int* kbreak, const int* l_in,
-                               int* k_out, int* l_out, int* status_out, int* kbreak_out, cudaStream_t st);
+                               const int* err, int* k_out, int* l_out, int* status_out, int* kbreak_out, int* err_out,
+                               cudaStream_t st);
 
 // Inner level for `count` problems whose tridiagonal coefficients live in device
 // arrays alp/bet/gam with leading dimension ldc (index j = 1..k as in Coefs, so the

@@ -1256,22 +1256,22 @@ __global__ void __launch_bounds__(6 * WS) k_update_wide(StepArgs a) {
 // vectors go to memory, for the neighbours. The two reductions of a step are barriers over the
 // problem's blocks, after which every block adds the partial sums itself, in the same order, and
 // forms the coefficients (block 0 of the problem stores them). A barrier's wait is bounded: when
-// it runs out the block sets *err and returns, and so do the others. A step on 4^4 (mu = 0) 20 ->
-// 15 us, on 8^4 (mu = 0.3) 25 -> 23 us, half of it the two barriers and the double arithmetic of
-// the coefficients between them.
-constexpr int kBarSpins = 1 << 22;  // polls of one barrier, a second or so
-__device__ __forceinline__ bool problem_barrier(unsigned* bar, unsigned nblk, int* err, int* s_fail) {
+// it runs out the block sets *err and returns; the others look at *err while they wait, and a
+// launch that finds it set returns at once (the counters are off their grid from then on). The
+// host reads the word with every group of checks and at the end, and gives the apply up. A step
+// on 4^4 (mu = 0) 20 -> 15 us, on 8^4 (mu = 0.3) 25 -> 23 us, half of it the two barriers and the
+// double arithmetic of the coefficients between them.
+__device__ __forceinline__ bool problem_barrier(unsigned* bar, unsigned nblk, int polls, int* err, int* s_fail) {
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
     const unsigned t = atomicAdd(bar, 1u), target = (t / nblk + 1u) * nblk;
-    int n = 0;
-    for (;;) {
+    for (int n = 0;; ++n) {
       unsigned v;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
       if ((int)(v - target) >= 0) break;
-      if (++n > kBarSpins) {
-        *err = 1;
+      if (n >= polls || ((n & 1023) == 1023 && *(volatile int*)err != 0)) {
+        *(volatile int*)err = 1;
         *s_fail = 1;
         break;
       }
@@ -1311,7 +1311,7 @@ __device__ __forceinline__ void block_partial(df64 (&v)[NQ], int w1, double* out
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(MODE == kModeTwoSided ? 192 : 96) k_steps(StepArgs a, int nsteps, unsigned* bars, int* err) {
+__global__ void __launch_bounds__(MODE == kModeTwoSided ? 192 : 96) k_steps(StepArgs a, int nsteps, unsigned* bars, int polls, int* err) {
   constexpr bool TWO = MODE == kModeTwoSided;
   constexpr int WS = 16, sub = 4, NW = TWO ? 6 : 3;
   __shared__ float4 s_x[96 * 2];          // the w side's entries, for the v side's dot products
@@ -1337,7 +1337,9 @@ __global__ void __launch_bounds__(MODE == kModeTwoSided ? 192 : 96) k_steps(Step
   site_coords(g, ss, xc[0], xc[1], xc[2], xc[3]);
   const int kk[2] = {3 * sp2 + col, 6 + 3 * sp2 + col};  // this thread's components
   const int j0 = __ldcg(a.jdev);
-  if (tid == 0) s_fail = 0;
+  if (tid == 0) s_fail = *(volatile int*)err;
+  __syncthreads();
+  if (s_fail) return;
   if (tid < 4) s_scal[tid] = __ldcg((const float4*)a.scal + (size_t)r * 8 + tid);
   size_t co = (size_t)r * a.c.ld + j0;
   double nvj = a.c.nv[co];
@@ -1379,7 +1381,7 @@ __global__ void __launch_bounds__(MODE == kModeTwoSided ? 192 : 96) k_steps(Step
       df64 v[2] = {dot.re, dot.im};
       block_partial(v, 3, pa + (size_t)bx * 4);
     }
-    if (!problem_barrier(&bars[r], nblk, err, &s_fail)) return;
+    if (!problem_barrier(&bars[r], nblk, polls, err, &s_fail)) return;
     if (warp == 0) {
       double tot[2];
       problem_total<2>(pa, nblk, tot);
@@ -1435,7 +1437,7 @@ __global__ void __launch_bounds__(MODE == kModeTwoSided ? 192 : 96) k_steps(Step
       block_partial(v, NW, pd + (size_t)bx * 4);
     }
     __threadfence();  // the new vector, before the barrier's arrival
-    if (!problem_barrier(&bars[r], nblk, err, &s_fail)) return;
+    if (!problem_barrier(&bars[r], nblk, polls, err, &s_fail)) return;
     if (warp == 0) {
       double nv;
       double2 nw, be, ga;
@@ -1515,9 +1517,9 @@ int steps_capacity(int mode) {
   }
   return per * sms;
 }
-cudaError_t launch_steps(int mode, const StepArgs& a, int nsteps, unsigned* bars, int* err, cudaStream_t st) {
+cudaError_t launch_steps(int mode, const StepArgs& a, int nsteps, unsigned* bars, int polls, int* err, cudaStream_t st) {
   StepArgs args = a;
-  void* p[] = {&args, &nsteps, &bars, &err};
+  void* p[] = {&args, &nsteps, &bars, &polls, &err};
   const dim3 grid(a.b.nblocks * 4);
   if (mode == kModeTwoSided)
     return cudaLaunchCooperativeKernel((const void*)k_steps<kModeTwoSided>, grid, dim3(192), p, 0, st);
