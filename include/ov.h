@@ -44,7 +44,10 @@
  * Environment, read by ov_create: OV_TRACE (set: one JSON line per stopping check on
  * stderr); OV_BASIS_CAP_BYTES (a byte count: the stored Krylov basis of the handle may
  * not grow beyond it, as if device memory ran out there; with OV_RECOMB_AUTO the run then
- * continues in the double pass; meant for testing that fall-back). Also read by ov_set_opts:
+ * continues in the double pass; meant for testing that fall-back); OV_ONE_LAUNCH_BLOCKS (the
+ * blocks up to which the outer steps of a small lattice are asked for in one cooperative launch,
+ * in place of what the device reports to fit; a launch that the device refuses becomes two
+ * launches a step; meant for testing that fall-back). Also read by ov_set_opts:
  * OV_BARRIER_POLLS (how often a block of the one-launch outer steps of small lattices looks for
  * the others before it gives up and the apply returns OV_ERR_CUDA; 2^22 looks, a second or so,
  * without it; meant for testing that return). Phases of an apply

@@ -151,6 +151,7 @@ struct ov_handle {
   int trace = 0;  // OV_TRACE set in the environment: one JSON line per check on stderr
   size_t basis_cap = 0;  // OV_BASIS_CAP_BYTES: bytes the stored basis may take (0: no cap)
   int bar_polls = kBarPolls;  // OV_BARRIER_POLLS: the bound of a wait in k_steps
+  int step_blocks = 0;        // OV_ONE_LAUNCH_BLOCKS: blocks k_steps is asked to run (0: as the device says)
   Buf nn_scratch;        // the non-nested check's dense H_k, iterates and elimination buffers
   // deflation (Sec. 2): per lattice the critical eigenvalues and right / left eigenvectors
   // (canonical complex doubles, [m][12 V]; L = R at mu = 0)
@@ -459,6 +460,7 @@ extern "C" int ov_create(ov_handle** hp, const ov_geom* geom, const void* links,
   h->trace = getenv("OV_TRACE") != nullptr;
   if (const char* cap = getenv("OV_BASIS_CAP_BYTES")) h->basis_cap = (size_t)strtoull(cap, nullptr, 10);
   h->bar_polls = env_polls();
+  if (const char* nb = getenv("OV_ONE_LAUNCH_BLOCKS")) h->step_blocks = atoi(nb);
   const size_t canon = sizeof(double2) * 36 * (size_t)V;
   const double2* src = (const double2*)links;
   Buf tmp;
@@ -874,6 +876,7 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
   }
   auto step_prec = [&](int jj) { return jj >= relax_from ? kPrecDF64Relaxed : h->prec; };
   int jdone = 0;
+  bool ran_coop = false;  // some span ran in one launch
   size_t slots_on_device = 0;  // entries of the device slot table written so far
   // outer steps jfrom+1 .. jto: basis slots (stored mode), the autotuned block size at
   // step 1, whole graph units replayed and the rest launched one by one
@@ -922,7 +925,7 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
         if (h->prec == OV_PREC_DF64 && !relaxing && pool / 12 <= kWideSites) {
           int nb64 = 0;
           for (int q : lat_of) nb64 += num_site_blocks(h->lat[q].g, 64);
-          cands.push_back({64, wide_sites(nb64), 4 * nb64 <= steps_capacity(mode) ? 1 : 0});
+          cands.push_back({64, wide_sites(nb64), 4 * nb64 <= (h->step_blocks > 0 ? h->step_blocks : steps_capacity(mode)) ? 1 : 0});
         }
         for (const Tuned& cand : cands) {
           Batch bc;
@@ -959,12 +962,23 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
       if (coop && gU > 0) {
         // every block fits the GPU at once: the whole span in one launch
         const int nst = jto - jn + 1;
-        CK(launch_steps(mode, a, nst, (unsigned*)h->bars.p, h->bar_polls, (int*)h->bars.p + nrhs, st));
-        h->stats.launches += 1;
-        h->stats.stencil_launches += nst;
-        h->stats.update_launches += nst;
-        h->stats.outer_steps += nst;
-        jn = jto + 1;
+        const cudaError_t e = launch_steps(mode, a, nst, (unsigned*)h->bars.p, h->bar_polls, (int*)h->bars.p + nrhs, st);
+        if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+          // refused (fewer SMs than the device has, as under a partition or a stream limited to
+          // some of them): nothing ran, and the wide kernels take the same step state
+          cudaGetLastError();
+          coop = 0;
+          auto it = h->tuned.find(key);
+          if (it != h->tuned.end()) it->second.coop = 0;
+        } else {
+          CK(e);
+          ran_coop = true;
+          h->stats.launches += 1;
+          h->stats.stencil_launches += nst;
+          h->stats.update_launches += nst;
+          h->stats.outer_steps += nst;
+          jn = jto + 1;
+        }
       }
       while (jn <= jto) {
         const int sp = step_prec(jn);
@@ -1428,9 +1442,9 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
   tstop(h, tr);
   tstop(h, t_total);
   if (mem == OV_MEM_HOST) CK(cudaMemcpyAsync(y, yd, canon, cudaMemcpyDeviceToHost, st));
-  if (coop) CK(cudaMemcpyAsync(h->chk_host, (int*)h->bars.p + nrhs, sizeof(int), cudaMemcpyDeviceToHost, st));
+  if (ran_coop) CK(cudaMemcpyAsync(h->chk_host, (int*)h->bars.p + nrhs, sizeof(int), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
-  if (coop && *(const int*)h->chk_host != 0) return OV_ERR_CUDA;
+  if (ran_coop && *(const int*)h->chk_host != 0) return OV_ERR_CUDA;
   tcollect(h);
   int worst = OV_OK;
   for (int r = 0; r < nrhs; ++r) {

@@ -1,5 +1,5 @@
 """Outer steps in one cooperative launch (small double-float lattices): what the host does when
-a wait inside the launch runs out."""
+a wait inside the launch runs out, and where the device refuses the launch."""
 import time
 
 import numpy as np
@@ -46,3 +46,28 @@ def test_a_wait_that_runs_out_ends_the_apply(ov, monkeypatch, capfd, mu, k_fixed
         op.set_opts(**opts)
         assert op.sign_apply(x, after, 1e-9, 600, 100)[0] == 0
         assert np.array_equal(after, good)
+
+
+# (750 and 384 blocks; a GB300's 152 SMs hold four of the one-sided ones each, two of the two-sided)
+@pytest.mark.parametrize("dims,mu,recomb", [((10, 10, 10, 12), 0.0, 0), ((8, 8, 8, 12), 0.3, 0), ((8, 8, 8, 12), 0.3, 1)])
+def test_a_refused_launch_becomes_two_launches_a_step(ov, monkeypatch, capfd, dims, mu, recomb):
+    """Asked for more blocks than run at once, the device refuses the cooperative launch; the
+    steps go on with the wide kernels, here at a size where the tuner takes them, and the answer
+    is the one-thread-a-site kernels' to rounding (the bar of the block sizes, 1e-11)."""
+    monkeypatch.setenv("OV_TRACE", "1")
+    monkeypatch.setenv("OV_ONE_LAUNCH_BLOCKS", "1000000")
+    k = 60
+    U = oi.gauge_field(dims, "near_unit", 3, eps=0.35)
+    x = oi.gaussian_source(dims, 10).reshape(1, -1)
+    ys = {}
+    for bs in (0, 64):
+        ys[bs] = np.zeros_like(x)
+        with ov.Overlap(dims, U, -1.5, mu, "df64",
+                        opts=ov.make_opts(k_fixed=k, block_size=bs, recombination=recomb)) as op:
+            for _ in range(2):
+                op.reset_stats()
+                assert op.sign_apply(x, ys[bs], 1e-8, k, 60)[0] == 0
+            if bs == 0 and '"one_launch": 1' not in capfd.readouterr().err:
+                pytest.skip("the tuner took one thread a site")
+            assert op.stats()["outer_steps"] == k and op.stats()["graph_launches"] > 0
+    assert np.linalg.norm(ys[0] - ys[64]) < 1e-11 * np.linalg.norm(ys[64])
