@@ -729,6 +729,18 @@ static int graph_for(ov_handle* h, const StepArgs& a, int prec, int mode, int U,
   return OV_OK;
 }
 
+// An early return leaves nothing in flight: a check or a span still running would meet the next
+// apply's use of the same coefficients and check buffers, which it is not ordered against.
+struct Drain {
+  ov_handle* h;
+  bool armed = true;
+  ~Drain() {
+    if (!armed) return;
+    if (h->chk_st) cudaStreamSynchronize(h->chk_st);
+    cudaStreamSynchronize(h->st);
+  }
+};
+
 // ---------------------------------------------------------------- sign apply
 static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int mem, double tol, int k_max, int l,
                            ov_info* info, int add_x, int neg_mu = 0, int strict_only = 0) {
@@ -742,6 +754,7 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
   CK(cudaSetDevice(h->dev));
   cudaStream_t st = h->st;
   if (h->is_batch && nrhs != (int)h->lat.size()) return OV_ERR_ARG;
+  Drain drain{h};
   const std::vector<int> lat_of = lattices_of_call(h, nrhs);
   bool herm = true;
   for (int q : lat_of) herm = herm && h->lat[q].mu == 0.0;
@@ -1083,6 +1096,11 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
       js.push_back(std::min(js.back() + o.check_interval, ktarget));
     if (js.back() > jdone) {
       rc = steps_to(js.back(), gcap > 1 ? target : 0);
+      // (no basis memory for all of the group's steps: the checks of those that ran may end the run)
+      if (rc == OV_ERR_NOMEM && jdone >= target) {
+        while (js.back() > jdone) js.pop_back();
+        rc = OV_OK;
+      }
       if (rc != OV_OK) return rc;
     }
     j = target;
@@ -1217,15 +1235,14 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
       spec_run = true;
       if (jlast + spec > jdone) {
         rc = steps_to(jlast + spec, g > 1 ? jlast + o.check_interval : 0);
-        if (rc != OV_OK) return rc;
+        // no basis memory for steps that the run may not need: the check decides, and where the
+        // run goes on they fail again
+        if (rc != OV_OK && rc != OV_ERR_NOMEM) return rc;
       }
     }
     CK(cudaStreamSynchronize(cs));
-    if (*hb.err != 0) {
-      // a wait of k_steps ran out: the coefficients end somewhere before these checks
-      CK(cudaStreamSynchronize(st));
-      return OV_ERR_CUDA;
-    }
+    // a wait of k_steps ran out: the coefficients end somewhere before these checks
+    if (*hb.err != 0) return OV_ERR_CUDA;
     // the inner estimate is needed only where the run may stop at this check
     bool have_ei = phase == 0 && !fixed;
     if (!have_ei && !fixed) {
@@ -1444,6 +1461,7 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
   if (mem == OV_MEM_HOST) CK(cudaMemcpyAsync(y, yd, canon, cudaMemcpyDeviceToHost, st));
   if (ran_coop) CK(cudaMemcpyAsync(h->chk_host, (int*)h->bars.p + nrhs, sizeof(int), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
+  drain.armed = false;
   if (ran_coop && *(const int*)h->chk_host != 0) return OV_ERR_CUDA;
   tcollect(h);
   int worst = OV_OK;
