@@ -1643,9 +1643,9 @@ __global__ void __launch_bounds__(kColThreads) k_rh_col(int count, int hermitian
 // ------------------------------------------------------------ combine
 // c = Q_l s and the inner estimate, a cluster of kCombineCtas CTAs a problem (the sums over l
 // are in double, whose pipe gives two multiply-adds a cycle and SM: one CTA a problem took
-// 0.26 ms at k = 333, l = 120, the cluster 0.067). Eight lanes share a row of Q. The difference
-// to the c of the leading l - dl block, c - c' = Q (s - [s'; 0]), only feeds the estimate: in
-// float pairs.
+// 0.26 ms for 12 of k = 333, l = 120, the cluster 0.048). Eight lanes share a row of Q. The
+// difference to the c of the leading l - dl block is summed as c - c' = Q (s - [s'; 0]), in double
+// like c (in float pairs it took longer, 0.067 ms, for 1e-15 in place of 1e-16 in the estimate).
 constexpr int kCombineCtas = 8, kCombineThreads = 128;
 
 __global__ void __cluster_dims__(kCombineCtas, 1, 1) __launch_bounds__(kCombineThreads)
@@ -1655,7 +1655,7 @@ __global__ void __cluster_dims__(kCombineCtas, 1, 1) __launch_bounds__(kCombineT
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   __shared__ double2 s_s[kMaxL];
-  __shared__ float4 s_ds[kMaxL];
+  __shared__ double2 s_ds[kMaxL];
   __shared__ double s_red[kCombineThreads / 32][2];
   __shared__ double s_tot[kCombineCtas][2];
   // a CTA's shared memory may be written by another once it is known to run: all arrive here, and
@@ -1675,7 +1675,7 @@ __global__ void __cluster_dims__(kCombineCtas, 1, 1) __launch_bounds__(kCombineT
     const double2 v = s1[i];
     const double2 v2 = have_est && i < le2 ? s2[i] : make_double2(0.0, 0.0);
     s_s[i] = v;
-    e_store(&s_ds[i], e_from2(make_double2(v.x - v2.x, v.y - v2.y), cdf{}));
+    s_ds[i] = zsub(v, v2);
   }
   __syncthreads();
   // the double-float inner level keeps Q as float pairs in the doubles' bytes
@@ -1701,28 +1701,26 @@ __global__ void __cluster_dims__(kCombineCtas, 1, 1) __launch_bounds__(kCombineT
   for (int m0 = rank * (kCombineThreads / 8); m0 < k; m0 += kCombineCtas * (kCombineThreads / 8)) {
     const int m = m0 + rl;
     double2 v = make_double2(0.0, 0.0);
-    cdf d = {df_zero(), df_zero()};
+    double2 d = make_double2(0.0, 0.0);
     if (!bad && m < k) {
       for (int i = sub; i < le; i += 8) {
         const double2* qp = &Q[(size_t)m * kMaxL + i];
-        const cdf qe = pairs ? e_load((const float4*)qp) : e_from2(*qp, cdf{});
-        const double2 qv = pairs ? e_to2(qe) : *qp;
+        const double2 qv = pairs ? e_to2(e_load((const float4*)qp)) : *qp;
         v = zadd(v, zmul(qv, s_s[i]));
-        if (have_est) d = e_addmul(d, qe, e_load(&s_ds[i]));
+        if (have_est) d = zadd(d, zmul(qv, s_ds[i]));
       }
     }
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) {
       v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
       v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
-      d.re = d.re + shfl_lane(d.re, (tid & 31) ^ o);
-      d.im = d.im + shfl_lane(d.im, (tid & 31) ^ o);
+      d.x += __shfl_xor_sync(0xffffffffu, d.x, o);
+      d.y += __shfl_xor_sync(0xffffffffu, d.y, o);
     }
     if (sub == 0 && m < k) {
       put(m, v);
       nc += zabs2(v);
-      const double2 dv = e_to2(d);
-      nd += zabs2(dv);
+      nd += zabs2(d);
     }
   }
   nc = warp_sum(nc);
