@@ -331,8 +331,9 @@ int ov_mlp_train(float* theta, int n, const float* X, const float* Y, int epochs
                  const float* Yv, float* val_history);
 /* Attach a trained network to a handle (theta NULL detaches). With it, ov_sign_apply runs
  * 16 outer steps, predicts (k*, l*) per right-hand side on the device, places the first
- * stopping check at the smallest predicted k* and uses the predicted l (rounded up to a
- * multiple of 8, clamped to [l_min, min(l_max, l)]). The a-posteriori estimates still
+ * stopping check at the largest predicted k* (rounded down to an integer, and to an even one
+ * where check_interval is even; at most check_interval before k_max) and uses the predicted l
+ * (rounded up to a multiple of 8, clamped to [l_min, min(l_max, l)]). The a-posteriori estimates still
  * decide: checks continue past a short prediction, and an inner estimate above tol grows
  * l by 16 and repeats the check. */
 int ov_set_sizer(ov_handle* h, const float* theta, int l_min, int l_max);
