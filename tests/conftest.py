@@ -1,3 +1,4 @@
+import gc
 import os
 import sys
 
@@ -13,6 +14,18 @@ def pytest_configure(config):
     config.addinivalue_line("markers", "gpu: needs a CUDA GPU (GB300) and the built libov")
     config.addinivalue_line("markers", "slow: long CPU test")
     config.addinivalue_line("markers", "dense: large dense linear algebra (all BLAS threads)")
+
+
+@pytest.hookimpl(hookwrapper=True)
+def pytest_runtest_call(item):
+    """Some GPU tests compare wall times of some 50 ms; a full collection of the imported modules'
+    objects takes as long, so none starts inside such a test."""
+    on = item.get_closest_marker("gpu") is not None and gc.isenabled()
+    if on:
+        gc.disable()
+    yield
+    if on:
+        gc.enable()
 
 
 @pytest.fixture(scope="session")
