@@ -118,7 +118,7 @@ struct ov_handle {
   Buf partials, counters, scale, scal;
   int cap_rhs = 0, cap_ld = 0;
   // inner level
-  Buf iQ, iT, iS, is, irh_its, irh_ok, iperm, ifail, irx, icn;
+  Buf iQ, iT, iS, is, irh_its, irh_ok, iperm, ifail, icn;
   Buf ck, cl, ckprev, cc_cur, cacc_cur, cacc_fin;
   Buf chk;  // what a group of checks reports (CheckBuf), with its copy in pinned host memory
   void* chk_host = nullptr;
@@ -498,7 +498,7 @@ extern "C" void ov_destroy(ov_handle* h) {
   Buf* all[] = {&h->desc, &h->blkmap, &h->xcanon, &h->ycanon, &h->tv, &h->tw, &h->p, &h->r, &h->vring, &h->wring, &h->yacc,
                 &h->coef_alp, &h->coef_bet, &h->coef_gam, &h->coef_nv, &h->coef_nw, &h->coef_status,
                 &h->coef_kbreak, &h->partials, &h->counters, &h->scale, &h->scal, &h->iQ, &h->iT, &h->iS, &h->is,
-                &h->irh_its, &h->irh_ok, &h->iperm, &h->ifail, &h->irx, &h->icn, &h->ck, &h->cl, &h->ckprev, &h->cc_cur,
+                &h->irh_its, &h->irh_ok, &h->iperm, &h->ifail, &h->icn, &h->ck, &h->cl, &h->ckprev, &h->cc_cur,
                 &h->cacc_cur, &h->cacc_fin, &h->chk,
                 &h->vptr, &h->sizer_theta, &h->sizer_feat, &h->sizer_pred, &h->nn_scratch, &h->dx, &h->dy,
                 &h->dpart, &h->dG};
@@ -596,18 +596,18 @@ static int check_group_cap(const ov_handle* h, int nrhs, size_t pool, const ov_o
   return std::max(1, std::min(kMaxGroup, 64 / nrhs));
 }
 
-static int ensure_inner(ov_handle* h, int count, int ld) {
-  // ld: leading dimension of the per-problem k-vectors (>= k + 2)
+static int ensure_inner(ov_handle* h, int count, int ld, bool dense = false) {
+  // ld: leading dimension of the per-problem k-vectors (>= k + 2); dense: for run_rh_dense on up to
+  // 2 count matrices
   CK(grow(h->iQ, sizeof(double2) * (size_t)count * ld * kMaxL));
   CK(grow(h->iT, sizeof(double2) * (size_t)count * kMaxL * 3));
-  CK(grow(h->iS, sizeof(double2) * (size_t)2 * count * kMaxL * kMaxL));
+  CK(grow(h->iS, rh_scratch_bytes(2 * count, h->o.inner_arith, dense)));
   CK(grow(h->is, sizeof(double2) * (size_t)2 * count * kMaxL));
   CK(grow(h->irh_its, sizeof(int) * 2 * count));
   CK(grow(h->irh_ok, sizeof(int) * 2 * count));
   CK(grow(h->iperm, sizeof(int) * 2 * (size_t)count * kMaxL));
   CK(grow(h->ifail, sizeof(int) * count));
   CK(grow(h->icn, sizeof(double) * count));
-  if (h->o.inner_arith == OV_INNER_DF64) CK(grow(h->irx, rh_col_scratch_bytes(count)));
   const size_t cb = sizeof(double2) * (size_t)count * ld;
   CK(grow(h->ck, sizeof(int) * count));
   CK(grow(h->cl, sizeof(int) * count));
@@ -642,7 +642,6 @@ static InnerWork inner_work(ov_handle* h, int rows) {
   w.rh_ok = (int*)h->irh_ok.p;
   w.perm = (int*)h->iperm.p;
   w.fail = (int*)h->ifail.p;
-  w.rx = (float4*)h->irx.p;
   w.ld = h->inner_ld;  // Q rows per problem, as allocated by ensure_inner
   w.arith = h->o.inner_arith;
   w.rh_scale = h->o.rh_scaling;
@@ -1227,8 +1226,9 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
     CK(e);
     tstop(h, ti);
     // the check's step kernel, k_inner, k_rh, k_combine, k_estimate; the double-float inner level
-    // has two Roberts-Higham kernels
-    const int rh_kernels = o.nested && o.inner_arith == OV_INNER_DF64 ? 2 : 1;
+    // has two Roberts-Higham kernels, run on so many matrices at a time
+    const int rh_kernels =
+        o.nested && o.inner_arith == OV_INNER_DF64 ? 2 * (((phase == 0 ? 2 * n : n) + kRhWave - 1) / kRhWave) : 1;
     h->stats.launches += 4 + rh_kernels;
     h->stats.inner_launches += 4 + rh_kernels;
     h->stats.checks += g;
@@ -2106,7 +2106,7 @@ extern "C" int ov_rh_sign(ov_handle* h, int count, int m, const void* T, void* S
     }
     return worst;
   }
-  int rc = ensure_inner(h, (count + 1) / 2, std::max(h->inner_ld, 4));
+  int rc = ensure_inner(h, (count + 1) / 2, std::max(h->inner_ld, 4), true);
   if (rc != OV_OK) return rc;
   const size_t mb = sizeof(double2) * (size_t)count * m * m;
   Buf dT, dS, dI;

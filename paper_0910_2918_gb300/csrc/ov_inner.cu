@@ -605,7 +605,7 @@ __global__ void __launch_bounds__(1024) k_rh_df(int count, int dense_m, const do
   __shared__ float s_logdet;  // log |det S_n| from the pivots (high words)
   // global S_n (row-major, leading dim m) in the float-pair storage, in the problem's
   // double2 slot (16 bytes per element)
-  St* Sg = (St*)(w.S + (size_t)mid * kMaxL * kMaxL);
+  St* Sg = (St*)(w.S + (size_t)blockIdx.x * kMaxL * kMaxL);
   int* perm = w.perm + (size_t)mid * kMaxL;
   const E ez = e_zero(E{});
   for (int e = tid; e < m * m; e += nth) {
@@ -791,7 +791,7 @@ __global__ void __launch_bounds__(1024) k_rh_df(int count, int dense_m, const do
   if (CPLX && dense_m > 0) {
     // the caller reads S as double2: convert in place (same 16-byte slot per element)
     __syncthreads();
-    double2* Sd = w.S + (size_t)mid * kMaxL * kMaxL;
+    double2* Sd = w.S + (size_t)blockIdx.x * kMaxL * kMaxL;
     for (int e = tid; e < m * m; e += nth) {
       const E v = e_load(&Sg[e]);
       Sd[e] = e_to2(v);
@@ -1453,7 +1453,8 @@ __global__ void __launch_bounds__(kColThreads) k_rh_col(int count, int hermitian
     __syncthreads();
   }
   // this thread's two rows of numbers per eliminated row; the solution overwrites the first
-  float4* const u1 = w.rx + (size_t)mid * 2 * kMaxL * kColThreads + t;
+  float4* const rx = (float4*)w.S + (size_t)blockIdx.x * 2 * kMaxL * kColThreads;
+  float4* const u1 = rx + t;
   float4* const u2 = u1 + (size_t)kMaxL * kColThreads;
   // (T - z) x = e_1 for pole idx (the zeros of S_b are idx = 2^b .. 2^{b+1} - 1), times its
   // weight; idx = 0: weight zero
@@ -1565,7 +1566,7 @@ __global__ void __launch_bounds__(kColThreads) k_rh_col(int count, int hermitian
     return fine;
   };
   // sum over threads [a, b) of row t's solutions (thread t: row t of T)
-  const float4* const row = w.rx + (size_t)mid * 2 * kMaxL * kColThreads + (size_t)t * kColThreads;
+  const float4* const row = rx + (size_t)t * kColThreads;
   auto rowsum = [&](int a, int b) {
     cdf s0 = zero, s1 = zero, s2 = zero, s3 = zero;
     int i = a;
@@ -1797,7 +1798,11 @@ cudaError_t launch_check_setup(int rows, int n, const CheckSteps& cj, const int*
   return cudaGetLastError();
 }
 
-size_t rh_col_scratch_bytes(int count) { return sizeof(float4) * 4 * (size_t)count * kMaxL * kColThreads; }
+size_t rh_scratch_bytes(int nmat, int arith, bool dense) {
+  const size_t it = sizeof(double2) * (size_t)kMaxL * kMaxL, col = sizeof(float4) * 2 * (size_t)kMaxL * kColThreads;
+  static_assert(sizeof(float4) * 2 * kMaxL * kColThreads >= sizeof(double2) * kMaxL * kMaxL, "a slot holds either");
+  return arith == OV_INNER_DF64 && !dense ? std::min(nmat, kRhWave) * col : nmat * it;
+}
 
 static size_t inner_smem(int k) { return (size_t)13 * k * sizeof(double2) + 32 * sizeof(double) + k + 16; }
 static size_t inner_smem_real(int k) { return (size_t)13 * k * sizeof(float2) + 32 * sizeof(double) + k + 16; }
@@ -1836,17 +1841,18 @@ cudaError_t run_inner(int count, const int* k_dev, const int* l_dev, int hermiti
   // matrix + column buffer (which also holds the 64-double reduction scratch)
   const size_t rsm = (size_t)kMaxL * kMaxL * esz + std::max<size_t>(kMaxL * esz, 512);
   if (w.arith == OV_INNER_DF64) {
-    k_rh_col<<<nmat, kColThreads, 0, st>>>(count, hermitian, w, inner_dl, rh_tol, rh_maxit, mid0, w.rh_scale);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    // the matrices it left; float pairs take the bytes of the double elements they replace
-    if (hermitian) {
-      e = cudaFuncSetAttribute(k_rh_df<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm);
-      if (e != cudaSuccess) return e;
-      k_rh_df<false><<<nmat, 1024, rsm, st>>>(count, 0, nullptr, w, inner_dl, rh_tol, rh_maxit, mid0, w.rh_scale);
-    } else {
-      e = cudaFuncSetAttribute(k_rh_df<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm);
-      if (e != cudaSuccess) return e;
-      k_rh_df<true><<<nmat, 1024, rsm, st>>>(count, 0, nullptr, w, inner_dl, rh_tol, rh_maxit, mid0, w.rh_scale);
+    if (hermitian) e = cudaFuncSetAttribute(k_rh_df<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm);
+    else e = cudaFuncSetAttribute(k_rh_df<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm);
+    if (e != cudaSuccess) return e;
+    for (int m0 = mid0; m0 < mid0 + nmat; m0 += kRhWave) {
+      const int nm = std::min(kRhWave, mid0 + nmat - m0);
+      k_rh_col<<<nm, kColThreads, 0, st>>>(count, hermitian, w, inner_dl, rh_tol, rh_maxit, m0, w.rh_scale);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      // the matrices it left (in the same scratch); float pairs take the bytes of the double
+      // elements they replace
+      if (hermitian) k_rh_df<false><<<nm, 1024, rsm, st>>>(count, 0, nullptr, w, inner_dl, rh_tol, rh_maxit, m0, w.rh_scale);
+      else k_rh_df<true><<<nm, 1024, rsm, st>>>(count, 0, nullptr, w, inner_dl, rh_tol, rh_maxit, m0, w.rh_scale);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
   } else if (hermitian) {
     e = cudaFuncSetAttribute(k_rh<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsm);

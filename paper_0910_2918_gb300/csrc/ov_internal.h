@@ -149,14 +149,13 @@ struct InnerWork {
   double2* Q;       // [count][ld][kMaxL]  (row-major k x l_eff, leading dim kMaxL)
   double2* T;       // [count][kMaxL][3]  inner alpha, beta, gamma
   int* leff;        // [count]
-  double2* S;       // [2*count][kMaxL*kMaxL] Roberts-Higham scratch (global copy of S_n)
+  double2* S;       // rh_scratch_bytes(2*count, arith, dense): Roberts-Higham scratch
   double2* s;       // [2*count][kMaxL]  first column of sgn(T)
   int* rh_its;      // [2*count]
   int* rh_ok;       // [2*count]
   int* perm;        // [2*count][kMaxL]
   int* fail;        // [count] singular H_k
   double* cnorm;    // [count] ||c||
-  float4* rx;       // rh_col_scratch_bytes(count): the shifted systems of k_rh_col
   int ld;
   int rows;         // rows of the coefficient arrays: problem i reads row i % rows (several checks of
                     // the same right-hand sides in one call: problem i is check i / rows)
@@ -191,7 +190,11 @@ cudaError_t run_inner(int count, const int* k_dev, const int* l_dev, int hermiti
                       double rh_tol, int rh_maxit, int inner_dl, double2* c, int ldo, void* cacc, int prec,
                       double* est_inner, const double2* cprev, int ldp, const int* kprev_dev,
                       double* est_outer, int* rh_status, int* rh_iters, int phase, cudaStream_t st);
-size_t rh_col_scratch_bytes(int count);
+// InnerWork::S for nmat matrices: the iterates of the l x l iteration, one slot a matrix; in
+// double-float arithmetic also the systems of k_rh_col, in turn, for kRhWave matrices at a time
+// (two rounds of the four CTAs that an SM holds; 600 MB) unless they are dense
+constexpr int kRhWave = 8 * 152;
+size_t rh_scratch_bytes(int nmat, int arith, bool dense);
 cudaError_t run_rh_dense(int count, int m, const double2* T, double2* S, int* iters, int* ok,
                          double rh_tol, int rh_maxit, InnerWork& w, cudaStream_t st);
 
