@@ -1563,7 +1563,7 @@ __global__ void __launch_bounds__(kColThreads) k_rh_col(int count, int hermitian
       }
     }
     if (m > 1) e_store(&u1[(size_t)(m - 1) * kColThreads], keep);
-    return fine;
+    return fine || idx == 0;
   };
   // sum over threads [a, b) of row t's solutions (thread t: row t of T)
   const float4* const row = rx + (size_t)t * kColThreads;
@@ -1630,7 +1630,7 @@ __global__ void __launch_bounds__(kColThreads) k_rh_col(int count, int hermitian
   }
   const bool good = was && its <= rh_maxit;
   const bool finite = t >= m || (isfinite(f.re.hi) && isfinite(f.im.hi));
-  const int all = __syncthreads_and((fine || t == 0) && finite && good);
+  const int all = __syncthreads_and(fine && finite && good);
   if (t == 0) {
     w.rh_ok[mid] = all ? 1 : kRhLeft;
     w.rh_its[mid] = its;
