@@ -321,6 +321,10 @@ static int max_blocks(const ov_handle* h, const std::vector<int>& lat_of) {
 // that an SM holds few warps and each runs near its own latency, else 32. They are tried up to
 // kWideSites sites in all; above, the lattice fills the GPU with one thread a site.
 constexpr size_t kWideSites = 100000;
+// A matvec is not tuned: it takes the wide kernel up to kWideApplySites sites. The whole call, wide
+// against one thread a site at the default block size: 4^4 30 / 50 us, 8^4 34 / 52, 13,824 sites 46 /
+// 54, 16,384 45 / 53; 20,736 58 / 55, 24,192 60 / 56 (sixteen-byte stores at a stride of a site).
+constexpr size_t kWideApplySites = 18000;
 static int wide_sites(int nblocks64) { return nblocks64 * 4 * 2 <= 2 * 152 ? 16 : 32; }
 
 static std::vector<int> lattices_of_call(const ov_handle* h, int nprob) {
@@ -934,6 +938,9 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
         float best = 1e30f;
         Tuned best_t{kBlockDefault, 0, 0};
         std::vector<Tuned> cands = {{64, 0, 0}, {128, 0, 0}, {256, 0, 0}};
+        // (one launch a span wherever its blocks fit and the wide kernels win: it was the faster
+        // form of the two at every size tried, 14.8 us a step against 20.1 on 4^4 and 25.3 / 27.3 on
+        // 9^3 x 13 at mu = 0, 16.5 / 21.8 on 4^4 and 25.6 / 28.5 on 7 x 7 x 9 x 11 at mu = 0.3)
         if (h->prec == OV_PREC_DF64 && !relaxing && pool / 12 <= kWideSites) {
           int nb64 = 0;
           for (int q : lat_of) nb64 += num_site_blocks(h->lat[q].g, 64);
@@ -1896,10 +1903,9 @@ extern "C" int ov_wilson_apply(ov_handle* h, int nrhs, const void* x, void* y, i
   Batch bt;
   size_t pool = 0;
   const std::vector<int> lat_of = lattices_of_call(h, nrhs);
-  // (a small lattice: the wide kernel, as the tuner finds for its steps)
   int nb64 = 0;
   for (int q : lat_of) nb64 += num_site_blocks(h->lat[q].g, 64);
-  const bool wide = h->prec == OV_PREC_DF64 && !h->o.block_size && (size_t)nb64 * 64 <= kWideSites / 4;
+  const bool wide = h->prec == OV_PREC_DF64 && !h->o.block_size && (size_t)nb64 * 64 <= kWideApplySites;
   int rc = build_batch(h, lat_of, h->o.block_size ? h->o.block_size : (wide ? 64 : kBlockDefault), &bt, &pool);
   if (rc != OV_OK) return rc;
   if (wide) bt.wide = wide_sites(nb64);
