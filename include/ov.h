@@ -32,7 +32,11 @@
  * (OV_MEM_HOST / OV_MEM_DEVICE). Host buffers are copied synchronously inside the call;
  * device buffers must stay valid until the call returns. The caller owns x, y and the
  * links; the handle owns everything it allocates (converted links, Krylov bases,
- * coefficients, inner-level scratch) and frees it in ov_destroy. All device work runs
+ * coefficients, inner-level scratch) and frees it in ov_destroy. The inner level holds, for
+ * each problem that a check evaluates at a time, (k_max + 2) x 120 complex doubles of basis
+ * and two Roberts-Higham systems of 0.49 MB, at most 600 MB of those; where checks are
+ * evaluated in groups (overlap_checks) that is up to 8 problems for one source and up to 64
+ * in all: 23 MB for one source at k_max = 1000. All device work runs
  * on the stream given to ov_create (NULL = legacy default stream); every entry point
  * returns after that stream has finished the call's work.
  *

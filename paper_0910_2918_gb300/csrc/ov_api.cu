@@ -1038,7 +1038,7 @@ static int sign_apply_core(ov_handle* h, int nrhs, const void* x, void* y, int m
   // steps already reached ktarget (then no step is run, only the check).
   //
   // Checks are evaluated in groups. Where an interval of outer steps takes less time than a
-  // check (small lattices: a step of one 8^4 source takes 27 us, a check ~1.5 ms on one SM), the
+  // check (small lattices: a step of one 8^4 source takes 23 us, a check ~1.5 ms on one SM), the
   // steps of several intervals run first and their checks go to the inner level together, on
   // SMs that a single check leaves idle; their results are judged in the order of the serial
   // run, which they equal, and what lies behind the one that stops it is dropped. The group

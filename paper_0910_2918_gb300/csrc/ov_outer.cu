@@ -14,8 +14,11 @@
 //
 // Reductions: every block writes its partial sums (double) to a partials array; the
 // last block of each right-hand side (atomic ticket, no spin-wait) adds the partials in
-// a fixed order and writes the Krylov coefficient. Results are therefore bitwise
-// reproducible run to run.
+// a fixed order and writes the Krylov coefficient. Where whole runs of steps go in one
+// launch (k_steps, small lattices) a right-hand side's blocks wait for one another instead,
+// with a bound, and each adds the partials in the same order. Results are therefore bitwise
+// reproducible run to run with the same kernels and block size (the first apply of a handle
+// tunes them, and forms the source's norm with the block size it starts from).
 #include "ov_internal.h"
 #include "ov_types.cuh"
 
