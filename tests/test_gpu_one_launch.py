@@ -1,5 +1,6 @@
 """Outer steps in one cooperative launch (small double-float lattices): what the host does when
-a wait inside the launch runs out, and where the device refuses the launch."""
+a wait inside the launch runs out, and where the device refuses the launch; two threads at once."""
+import threading
 import time
 
 import numpy as np
@@ -48,8 +49,8 @@ def test_a_wait_that_runs_out_ends_the_apply(ov, monkeypatch, capfd, mu, k_fixed
         assert np.array_equal(after, good)
 
 
-# (750 and 384 blocks; a GB300's 152 SMs hold four of the one-sided ones each, two of the two-sided)
-@pytest.mark.parametrize("dims,mu,recomb", [((10, 10, 10, 12), 0.0, 0), ((8, 8, 8, 12), 0.3, 0), ((8, 8, 8, 12), 0.3, 1)])
+# (628 and 384 blocks; a GB300's 152 SMs hold four of the one-sided ones each, two of the two-sided)
+@pytest.mark.parametrize("dims,mu,recomb", [((10, 10, 10, 10), 0.0, 0), ((8, 8, 8, 12), 0.3, 0), ((8, 8, 8, 12), 0.3, 1)])
 def test_a_refused_launch_becomes_two_launches_a_step(ov, monkeypatch, capfd, dims, mu, recomb):
     """Asked for more blocks than run at once, the device refuses the cooperative launch; the
     steps go on with the wide kernels, here at a size where the tuner takes them, and the answer
@@ -71,3 +72,38 @@ def test_a_refused_launch_becomes_two_launches_a_step(ov, monkeypatch, capfd, di
                 pytest.skip("the tuner took one thread a site")
             assert op.stats()["outer_steps"] == k and op.stats()["graph_launches"] > 0
     assert np.linalg.norm(ys[0] - ys[64]) < 1e-11 * np.linalg.norm(ys[64])
+
+
+def test_two_handles_in_two_threads(ov):
+    """Two threads, each with its own handle and stream, on lattices whose launches do not fit the
+    GPU together (256 of 304 blocks each): the same answers, bitwise, as one after the other."""
+    import torch
+
+    dims = (8, 8, 8, 8)
+    ops, xs, want = [], [], []
+    for i in range(2):
+        U = oi.gauge_field(dims, "near_unit", i, eps=0.35)
+        stream = torch.cuda.Stream()
+        ops.append((ov.Overlap(dims, U, -1.5, 0.3, "df64", opts=ov.make_opts(check_interval=10), stream=stream.cuda_stream), stream))
+        xs.append(oi.gaussian_source(dims, 5 + i).reshape(1, -1))
+        for _ in range(2):  # the first apply tunes
+            y = np.zeros_like(xs[i])
+            assert ops[i][0].sign_apply(xs[i], y, 1e-9, 800, 100)[0] == 0
+        want.append(y)
+    bad = []
+
+    def work(i):
+        for _ in range(10):
+            y = np.zeros_like(xs[i])
+            rc, _ = ops[i][0].sign_apply(xs[i], y, 1e-9, 800, 100)
+            if rc != 0 or not np.array_equal(y, want[i]):
+                bad.append((i, rc))
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for op, _ in ops:
+        op.close()
+    assert not bad
