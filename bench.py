@@ -872,13 +872,13 @@ def run_volume_sweep(args):
 
 def run_profile(args):
     """One apply of the bench workload with k fixed to args.profile_steps (small
-    enough for an ncu capture: a few GB on the device)."""
+    enough for an ncu capture: two-pass, so no basis chunks, ~2 GB on the device)."""
     import torch
 
     import paper_0910_2918_gb300 as ov
 
     U, X = make_inputs()
-    opts = ov.make_opts(k_fixed=args.profile_steps, recombination=0, block_size=256, graph_steps=0,
+    opts = ov.make_opts(k_fixed=args.profile_steps, recombination=1, block_size=256, graph_steps=0,
                         relax=args.profile_relax)
     with ov.Overlap(DIMS, U, M_W, MU, args.profile_prec, opts=opts) as op:
         xd = torch.from_numpy(X).cuda()
